@@ -20,9 +20,10 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsu2gb300.so")
 SOURCES = ["heatbath.cu", "observables.cu", "links.cu", "api.cu", "plaquette_static.cu",
            "selftest.cu", "cluster.cu"]
-# heatbath_shapes.cu once per pair of launch shapes and row of the 14-entry
-# table in csrc/su2_internal.h (FP32, FP64, FP32 site pairs): (object name,
-# defines, flags).
+# heatbath_shapes.cu once per pair of launch shapes of the FP32 rows of the
+# 14-entry table in csrc/su2_internal.h (FP32, FP32 site pairs), heatbath_fp64.cu
+# once per kernel and sampler of the FP64 row: (object name, defines, flags);
+# the source is the name's first part.
 # The FP32 phase kernels flush denormals to zero: none can occur on their
 # path (links, staple sums and uniforms are >= 2^-24 in magnitude or exactly
 # 0, the log series is evaluated in Horner form, alpha and 1/(2 alpha) stay
@@ -30,8 +31,11 @@ SOURCES = ["heatbath.cu", "observables.cu", "links.cu", "api.cu", "plaquette_sta
 # and square-root sequences are shorter (2% at 64^4).
 ROW_NAMES = ("f32", "f64", "f32pairs")
 SHAPE_UNITS = [(f"heatbath_shapes_{ROW_NAMES[row]}_{k}",
-                (f"SU2_ROW={row}", f"SU2_FIRST={k}"), ("-ftz=true",) if row != 1 else ())
-               for row in (0, 1, 2) for k in range(0, 14, 2)]
+                (f"SU2_ROW={row}", f"SU2_FIRST={k}"), ("-ftz=true",))
+               for row in (0, 2) for k in range(0, 14, 2)]
+SHAPE_UNITS += [(f"heatbath_fp64_{kind}_{hyb}",
+                 (f"SU2_KIND={kind}", f"SU2_HYB={hyb}"), ())
+                for kind in range(5) for hyb in (0, 1)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -66,7 +70,9 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,
     extra += [f"-D{d}" for d in defines]
 
     units = [(src, src.replace(".cu", ""), (), ()) for src in SOURCES]
-    units += [("heatbath_shapes.cu", name, defs, fl) for name, defs, fl in SHAPE_UNITS]
+    shape_units = [("_".join(name.split("_")[:2]) + ".cu", name, defs, fl)
+                   for name, defs, fl in SHAPE_UNITS]
+    units = shape_units + units  # the longest first
 
     def one(unit):
         src, name, defs, fl = unit

@@ -16,6 +16,7 @@
 #include "su2_testing.h"
 #include "su2_internal.h"
 #include "su2_math.cuh"
+#include "su2_fixed.cuh"
 
 using namespace su2;
 
@@ -110,7 +111,7 @@ struct su2_lattice {
     size_t link_bytes = 0, work_bytes = 0;
     size_t off_status = 0, off_desc = 0, off_sstart = 0, off_spstart = 0;
     size_t off_plaq = 0, off_obs = 0, off_field = 0, off_ring = 0, off_res = 0, off_stage = 0;
-    size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0;
+    size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0, off_fixtab = 0;
     uint32_t max_chunks = 1;
     size_t res_doubles = 0;
     // bound state
@@ -299,6 +300,7 @@ int layout(su2_lattice* L)
     L->off_res = take(8 * L->res_doubles);
     L->off_stage = take(STAGE_BYTES);
     L->off_fp64tab = take(sizeof(double2) * FP64_TABLE_ENTRIES);
+    L->off_fixtab = take(sizeof(FixTables));
     L->work_bytes = w;
     return SU2_OK;
 }
@@ -419,7 +421,7 @@ int record_sweep(su2_lattice* L, bool plaq, int rmax, cudaStream_t s)
             SU2_CUDA(launch_phase(L->cfg_ctx[L->cfg], L->row, L->cfg, mu, p, plaq, nullptr,
                                   L->hybrid, s));
     }
-    SU2_CUDA(launch_sweep_end(L->cfg_ctx[L->cfg], plaq, s));
+    SU2_CUDA(launch_sweep_end(L->cfg_ctx[L->cfg], L->row == ROW_F64, plaq, s));
     return SU2_OK;
 }
 
@@ -578,6 +580,7 @@ int heatbath_impl(su2_lattice* L, const double* betas, double beta, int nsweeps,
         const int chunk = (want && !dev_out) ? std::min(PLAQ_RING, nsweeps - done) : nsweeps;
         if (int rc = set_params(L, betas, beta, seeds, seed, dev_out ? plaq : nullptr, nsweeps))
             return rc;
+        if (L->row == ROW_F64) SU2_CUDA(launch_unit_check(L->ctx, L->stream));
         for (int s = 0; s < chunk; ++s)
             SU2_CUDA(cudaGraphLaunch(g_first && done + s == 0 ? g_first : g, L->stream));
         if (want && !dev_out) {
@@ -750,6 +753,23 @@ void su2::fill_fp64_table(double2* tab)
 // --------------------------------------------------------------------------
 namespace {
 
+// The FP64 path's tables, computed once per process (2 ms in extended
+// precision on the Arm host).
+struct HostTables {
+    double2 fp64[FP64_TABLE_ENTRIES];
+    FixTables fix;
+};
+const HostTables& host_tables()
+{
+    static const HostTables t = [] {
+        HostTables h;
+        fill_fp64_table(h.fp64);
+        fill_fix_tables(&h.fix);
+        return h;
+    }();
+    return t;
+}
+
 // Links of lattice l to / from the canonical layout with values of type C
 // (double or float): device buffers and page-locked host memory go through
 // the conversion kernel directly, pageable host memory through the staging
@@ -912,12 +932,13 @@ int su2_bind_memory(su2_lattice* lat, void* links, size_t link_bytes, void* work
         D.link_off = lat->link_off[l];
         D.field_off = lat->field_off[l];
         D.fp64_table = reinterpret_cast<const double2*>(lat->work + lat->off_fp64tab);
+        D.fix_table = reinterpret_cast<const FixTables*>(lat->work + lat->off_fixtab);
     }
     char* w = lat->work;
-    {
-        double2 tab[FP64_TABLE_ENTRIES];
-        fill_fp64_table(tab);
-        SU2_CUDA(cudaMemcpy(w + lat->off_fp64tab, tab, sizeof tab, cudaMemcpyHostToDevice));
+    if (lat->dtype == SU2_F64) {
+        const HostTables& t = host_tables();
+        SU2_CUDA(cudaMemcpy(w + lat->off_fp64tab, t.fp64, sizeof t.fp64, cudaMemcpyHostToDevice));
+        SU2_CUDA(cudaMemcpy(w + lat->off_fixtab, &t.fix, sizeof t.fix, cudaMemcpyHostToDevice));
     }
     SU2_CUDA(cudaMemset(w + lat->off_status, 0, 256));
     SU2_CUDA(cudaMemcpy(w + lat->off_desc, d.data(), sizeof(LatDesc) * lat->n,
@@ -1070,12 +1091,15 @@ int su2_heatbath_phase(su2_lattice* lat, double beta, int mu, int parity, uint64
     DeviceGuard dg(lat->device);
     // consecutive phases with the same beta and seed reuse the parameters
     // already on the device (no parameter kernel between the phases)
-    if (!(lat->phase_params_valid && lat->phase_beta == beta && lat->phase_seed == seed)) {
+    // (FP64: the parameter kernel also starts the look at the links)
+    const bool f64 = lat->row == ROW_F64;
+    if (f64 || !(lat->phase_params_valid && lat->phase_beta == beta && lat->phase_seed == seed)) {
         if (int rc = set_params(lat, nullptr, beta, nullptr, seed, nullptr, 0)) return rc;
         lat->phase_params_valid = true;
         lat->phase_beta = beta;
         lat->phase_seed = seed;
     }
+    if (f64) SU2_CUDA(launch_unit_check(lat->ctx, lat->stream));
     SU2_CUDA(launch_phase(lat->cfg_ctx[lat->cfg], lat->row, lat->cfg, mu, parity, false, trials,
                           lat->hybrid, lat->stream));
     return SU2_OK;

@@ -3,16 +3,65 @@
 // kernel and the dispatch of the phase kernels (heatbath_kernel.cuh,
 // instantiated per pair of launch shapes and precision by
 // heatbath_shapes.cu).
+#include "su2_fixed.cuh"
 #include "su2_internal.h"
 #include "su2_reduce.cuh"
 
 namespace su2 {
 
+// A link component as a float (0 below 2^-126, at least 2 for |x| >= 2, an
+// infinity or a NaN), from its words: conversion instructions run on the
+// slow FP64 unit.
+__device__ __forceinline__ float narrow(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu;
+    if (e > 1023u) return 2.0f;
+    if (e < 897u) return 0.0f;
+    return __uint_as_float((((hi & 0x7FFFFFFFu) << 3) | (lo >> 29)) - (896u << 23));
+}
+__device__ __forceinline__ bool unit_link(const double2& lo, const double2& hi)
+{
+    const float a = narrow(lo.x), b = narrow(lo.y), c = narrow(hi.x), d = narrow(hi.y);
+    return fabsf(a * a + b * b + c * c + d * d - 1.0f) <= (float)UNIT_TOLERANCE;
+}
+// whether the links eo of the eight (mu, parity) planes of an FP64 lattice
+// are unit quaternions
+__device__ __forceinline__ bool unit_links_at(const Ctx& ctx, const LatDesc& D, uint32_t eo)
+{
+    const double2* U = reinterpret_cast<const double2*>(static_cast<const char*>(ctx.links) + D.link_off);
+    bool ok = true;
+#pragma unroll
+    for (int mp = 0; mp < 8; ++mp)
+        ok = ok && unit_link(U[(size_t)(2 * mp) * D.Vh + eo], U[(size_t)(2 * mp + 1) * D.Vh + eo]);
+    return ok;
+}
+
+// One thread per two sites.  Bound by HBM: one read of the links (64^4: 2.1
+// GB) per call of any number of sweeps.
+__global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx)
+{
+    const int l = lattice_of_block(ctx.site_start, ctx.n, blockIdx.x);
+    LatDesc* D = ctx.desc + l;
+    const uint32_t eo = (blockIdx.x - first_block(ctx.site_start, l)) * TPB + threadIdx.x;
+    if (eo < D->Vh && !unit_links_at(ctx, *D, eo)) D->nonunit = 1u;
+}
+
+// the same by one block, after a sweep of a lattice that failed the check:
+// once every link has been updated the lattice takes the fixed-point path
+__device__ void unit_recheck(const Ctx& ctx, LatDesc* D)
+{
+    bool ok = true;
+    for (uint32_t eo = threadIdx.x; eo < D->Vh; eo += TPB) ok = ok && unit_links_at(ctx, *D, eo);
+    if (__syncthreads_and(ok) && threadIdx.x == 0) D->nonunit = 0u;
+}
+
 // Finishes a sweep: the fixed-order sum of the fused plaquette partials and
 // the lattice's sweep counter.  Grid (chunks, lattices); each block sums
 // SWEEP_CHUNK partials of its lattice, the last block of a lattice to finish
 // (ticket counter) adds the chunk sums in chunk order.
-template <bool PLAQ>
+// FP64 lattices with non-unit links are looked at again (F64).
+template <bool PLAQ, bool F64>
 __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
 {
     __shared__ double sred[TPB / 32];
@@ -21,6 +70,7 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
     LatDesc* D = ctx.desc + l;
     if (!PLAQ) {
         if (blockIdx.x == 0 && threadIdx.x == 0) D->sweep += 1;
+        if (F64 && D->nonunit) unit_recheck(ctx, D);
         return;
     }
     // partials are per warp: lattice l owns warps [b0, b0 + nb) of each slot
@@ -60,6 +110,7 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
         if (D->plaq_out) D->plaq_out[k] = P;
         D->sweep += 1;
     }
+    if (F64 && D->nonunit) unit_recheck(ctx, D);
 }
 
 // Per-call parameters go in by value (no host-to-device copy); the
@@ -75,38 +126,63 @@ __global__ void set_params_kernel(Ctx ctx, ParamChunk pc)
     D->half_inv_beta = 0.5 / pc.beta[j];  // inf at beta = 0, where the Haar draw applies
     D->seed = pc.seed[j];
     D->plaq_out = pc.plaq_out[j];
+    D->nonunit = 0u;
     D->sweep_base = D->sweep;
 }
 
-// one pair of launch shapes per instantiation of heatbath_shapes.cu
+// one pair of FP32 launch shapes per instantiation of heatbath_shapes.cu, one
+// FP64 kernel and sampler per instantiation of heatbath_fp64.cu
 template <int ROW, int FIRST>
 cudaError_t launch_phase_pair(const Ctx& c, int cfg, int mu, int parity, bool plaq, int32_t* dbg,
                               bool hyb, cudaStream_t s);
+template <int KIND, bool HYB>
+cudaError_t launch_fix_kind(const Ctx& c, const LaunchCfg& f, int mu, int parity, bool plaq,
+                            int32_t* dbg, cudaStream_t s);
 
 cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, bool plaq,
                          int32_t* dbg_trials, bool hybrid, cudaStream_t s)
 {
+    if (row < 0 || row >= NUM_ROWS || cfg < 0 || cfg >= NUM_LAUNCH_CFG) return cudaErrorInvalidValue;
+    if (row == ROW_F64) {
+        using Fn = cudaError_t (*)(const Ctx&, const LaunchCfg&, int, int, bool, int32_t*, cudaStream_t);
+        static_assert(NUM_FIX_KINDS == 5, "one entry per kernel below");
+        static const Fn kinds[NUM_FIX_KINDS][2] = {
+            {launch_fix_kind<0, false>, launch_fix_kind<0, true>},
+            {launch_fix_kind<1, false>, launch_fix_kind<1, true>},
+            {launch_fix_kind<2, false>, launch_fix_kind<2, true>},
+            {launch_fix_kind<3, false>, launch_fix_kind<3, true>},
+            {launch_fix_kind<4, false>, launch_fix_kind<4, true>},
+        };
+        const LaunchCfg& f = LAUNCH_CFG[ROW_F64][cfg];
+        return kinds[fix_kind(f)][hybrid](c, f, mu, parity, plaq, dbg_trials, s);
+    }
     using Fn = cudaError_t (*)(const Ctx&, int, int, int, bool, int32_t*, bool, cudaStream_t);
     static_assert(NUM_LAUNCH_CFG == 14 && NUM_ROWS == 3, "one entry per pair of shapes below");
-    static const Fn pairs[NUM_ROWS][NUM_LAUNCH_CFG / 2] = {
+    static const Fn pairs[2][NUM_LAUNCH_CFG / 2] = {
         {launch_phase_pair<0, 0>, launch_phase_pair<0, 2>, launch_phase_pair<0, 4>,
          launch_phase_pair<0, 6>, launch_phase_pair<0, 8>, launch_phase_pair<0, 10>,
          launch_phase_pair<0, 12>},
-        {launch_phase_pair<1, 0>, launch_phase_pair<1, 2>, launch_phase_pair<1, 4>,
-         launch_phase_pair<1, 6>, launch_phase_pair<1, 8>, launch_phase_pair<1, 10>,
-         launch_phase_pair<1, 12>},
         {launch_phase_pair<2, 0>, launch_phase_pair<2, 2>, launch_phase_pair<2, 4>,
          launch_phase_pair<2, 6>, launch_phase_pair<2, 8>, launch_phase_pair<2, 10>,
          launch_phase_pair<2, 12>},
     };
-    if (row < 0 || row >= NUM_ROWS || cfg < 0 || cfg >= NUM_LAUNCH_CFG) return cudaErrorInvalidValue;
-    return pairs[row][cfg >> 1](c, cfg, mu, parity, plaq, dbg_trials, hybrid, s);
+    return pairs[row == ROW_F32_PAIRS][cfg >> 1](c, cfg, mu, parity, plaq, dbg_trials, hybrid, s);
 }
 
-cudaError_t launch_sweep_end(const Ctx& c, bool plaq, cudaStream_t s)
+cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s)
 {
-    if (plaq) sweep_end_kernel<true><<<dim3(c.max_chunks, c.n), TPB, 0, s>>>(c);
-    else sweep_end_kernel<false><<<dim3(1, c.n), 32, 0, s>>>(c);
+    const dim3 grid(plaq ? c.max_chunks : 1u, c.n);
+    const unsigned nt = plaq || fp64 ? TPB : 32;
+    if (fp64 && plaq) sweep_end_kernel<true, true><<<grid, nt, 0, s>>>(c);
+    else if (fp64) sweep_end_kernel<false, true><<<grid, nt, 0, s>>>(c);
+    else if (plaq) sweep_end_kernel<true, false><<<grid, nt, 0, s>>>(c);
+    else sweep_end_kernel<false, false><<<grid, nt, 0, s>>>(c);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_unit_check(const Ctx& c, cudaStream_t s)
+{
+    unit_check_kernel<<<c.site_blocks, TPB, 0, s>>>(c);
     return cudaGetLastError();
 }
 

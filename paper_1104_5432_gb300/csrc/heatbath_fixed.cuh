@@ -1,0 +1,572 @@
+// heatbath_fixed.cuh -- the FP64 phase kernels: links stored as doubles,
+// updated in 64-bit fixed point (su2_fixed.cuh), in the three forms of the
+// launch-shape table: one link per thread, R links per thread with a
+// per-warp retry queue, eight lanes per link.
+//
+// An FP64 warp instruction holds its SM sub-partition for ~76 clocks on
+// GB300, an IMAD.WIDE or a logic operation for 2, so the FP64 sequence
+// (general_link: ~270 FP64 instructions, 20,600 clocks per warp) was
+// bound by the FP64 unit alone: 1.66 G link updates/s at 64^4, beta = 2.5,
+// whatever the shape.  The integer update issues ~4,080 instructions per
+// 32 links (2,540 on the ALU pipe, 1,330 integer multiply-adds) and runs at
+// 4.97 G/s there (R = 8) and 4.66 G/s at 32^4, beta = 6.0 (one link per
+// thread, from 1.57), bound by the half-rate integer pipes.  All forms call
+// the same functions on integers, so links and trial counts are
+// bit-identical between them.
+//
+// The fixed-point ranges hold for unit links.  unit_check_kernel looks at
+// every link before the sweeps of a call and sweep_end_kernel again after
+// each sweep of a lattice that failed; such a lattice (D.nonunit) takes the
+// FP64 sequence, one link per thread, in the same kernels.
+#pragma once
+#include "heatbath_kernel.cuh"
+#include "su2_fixed.cuh"
+
+namespace su2 {
+
+__device__ __forceinline__ FQuat fq_link(const Quat<double>& q, bool dag)
+{
+    auto f = [](double x, bool flip) {
+        return fx_link((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x), flip);
+    };
+    return {f(q.a0, false), f(q.a1, dag), f(q.a2, dag), f(q.a3, dag)};
+}
+__device__ __forceinline__ Quat<double> dq_link(const int64_t* U)
+{
+    auto f = [](int64_t v) { return __longlong_as_double((long long)double_bits(v, -60)); };
+    return {f(U[0]), f(U[1]), f(U[2]), f(U[3])};
+}
+// a stored link at 2^60
+__device__ __forceinline__ void fix_from_link(const Quat<double>& q, int64_t* U)
+{
+    const FQuat f = fq_link(q, false);
+    const Fx* c[4] = {&f.a0, &f.a1, &f.a2, &f.a3};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) U[k] = (((int64_t)c[k]->h << 32) + c[k]->l) >> 1;
+}
+
+// One staple term x y^dagger z^dagger of U_mu(x): the upper (x, y, z) =
+// (U_nu(x+mu), U_mu(x+nu), U_nu(x)), the lower (U_nu(x+mu-nu)^dagger,
+// U_mu(x-nu), U_nu(x-nu)^dagger), added to A.
+__device__ __forceinline__ void fix_term(const Links<double>& U, int mu, int nu, int p, uint32_t i,
+                                         int hpm, int hpn, int hmn, bool lower, int64_t* A)
+{
+    const int q = p ^ 1;
+    const Quat<double> x = U.load(nu, lower ? p : q, i + hpm + (lower ? hmn : 0));
+    const Quat<double> y = U.load(mu, q, i + (lower ? hmn : hpn));
+    const Quat<double> z = U.load(nu, lower ? q : p, lower ? i + hmn : i);
+    fq_mul_nd_acc(fq_mul_nd(fq_link(x, lower), fq_link(y, false)), fq_link(z, lower), A);
+}
+
+// staple_sum: A, and (PLAQ) its part P over nu < mu.  The six terms are one
+// loop body: the update's code has to fit the instruction caches (fully
+// unrolled and with the draw inlined twice, 43% of the stalls waited for
+// instructions and 64^4 ran at 3.7 G updates/s).
+template <int MU, bool PLAQ>
+__device__ __forceinline__ void fix_staple_sum(const Links<double>& U, const EoSite& s, uint32_t i,
+                                               int p, int64_t* A, int64_t* P)
+{
+    int hp[4], hm[4];
+    s.hops(hp, hm);
+    A[0] = A[1] = A[2] = A[3] = 0;
+#pragma unroll 1
+    for (int k = 0; k < 6; ++k) {
+        constexpr int n0 = nu_of<MU>(0), n1 = nu_of<MU>(1), n2 = nu_of<MU>(2);
+        const int nu = k < 2 ? n0 : (k < 4 ? n1 : n2);
+        const int hpn = k < 2 ? hp[n0] : (k < 4 ? hp[n1] : hp[n2]);
+        const int hmn = k < 2 ? hm[n0] : (k < 4 ? hm[n1] : hm[n2]);
+        fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, (k & 1) != 0, A);
+        if (PLAQ && k == 2 * MU - 1) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) P[c] = A[c];
+        }
+    }
+}
+
+// Per-lattice values of a call, in registers.
+struct FixCall {
+    HalfInvBeta hb;
+    double beta, creutz;
+    float beta_f;
+    const FixTables* tab;
+    uint32_t k0, k1, slo, shi;
+    __device__ __forceinline__ explicit FixCall(const LatDesc& D)
+    {
+        const double h = D.half_inv_beta;
+        hb = half_inv_beta_fix((uint64_t)__double_as_longlong(h));
+        beta = D.beta;
+        creutz = D.creutz_below;
+        beta_f = D.beta_f;
+        tab = D.fix_table;
+        k0 = (uint32_t)D.seed;
+        k1 = (uint32_t)(D.seed >> 32);
+        slo = (uint32_t)D.sweep;
+        shi = (uint32_t)(D.sweep >> 32);
+    }
+    __device__ __forceinline__ Stream stream(uint32_t key) const { return {k0, k1, key, slo, shi}; }
+};
+
+// alpha -> 0 limit of the conditional law (rare: kept out of the loops' code)
+static __device__ __noinline__ Quat<double> haar_link(Stream st)
+{
+    return haar_from<double>(st.draw(TAG_DIRECTION, 0));
+}
+
+// The draw's inputs from the staple sum: false for the Haar branch
+// (alpha = beta |A| below its threshold).  HYB: *qc = 1 - exp(-2 alpha) of a
+// link that takes Creutz's draw, 0 otherwise.
+template <bool HYB>
+__device__ __forceinline__ bool fix_prepare(const FixCall& C, const int64_t* A, Drawn* d, double* qc)
+{
+    uint64_t K;
+    int n;
+    *qc = 0.0;
+    if (!unit_staple(A, C.hb, d, &K, &n)) return false;
+    // |A| = sqrt(K 2^-60) 2^(7 - n); in single precision away from the threshold
+    const float kf = __fsqrt_rn((float)(uint32_t)(K >> 29)) * exp2f((float)(7 - n) - 15.5f);
+    double alpha = 0.0;
+    if (HYB || !(C.beta_f * kf > 2e-12f)) {
+        alpha = C.beta * ldexp(sqrt((double)K), 7 - n - 30);
+        if (!(alpha >= alpha_haar<double>())) return false;
+    }
+    if (HYB && alpha < C.creutz) *qc = creutz_qc(alpha);
+    return true;
+}
+
+// one trial; true when accepted
+template <bool HYB>
+__device__ __forceinline__ bool fix_try(const FixCall& C, const U4& w, int64_t inv, int ei, double qc,
+                                        Lambda* L)
+{
+    if (HYB && qc > 0.0) {
+        double delta;
+        const double inv2a = __longlong_as_double((long long)double_bits(inv, ei));
+        const bool ok = creutz_try(w, qc, inv2a, &delta);
+        *L = lambda_from_delta((uint64_t)__double_as_longlong(delta));
+        return ok;
+    }
+    *L = kp_lambda(w.x, w.y, w.z, inv, ei, C.tab);
+    return kp_accept(*L, w.w);
+}
+
+// warp sum of 64-bit integers
+__device__ __forceinline__ int64_t warp_sum64(int64_t v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v += (int64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)v, o);
+    return v;
+}
+
+// warp_totals with the plaquette already summed over the warp
+template <int MU, bool PLAQ>
+__device__ __forceinline__ void fix_totals(const Ctx& ctx, int l, uint32_t blk0, uint32_t Vh,
+                                           double wp, uint32_t ntrial, uint32_t ncap)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t wt = __reduce_add_sync(0xffffffffu, ntrial);
+    const uint32_t wc = __reduce_add_sync(0xffffffffu, ncap);
+    if (lane == 0) add_warp_totals<MU, PLAQ>(ctx, ctx.phase_wpb, l, blk0, Vh, wp, w, wt, wc);
+}
+__device__ __forceinline__ double plaq_double(int64_t v)  // v 2^-51
+{
+    return __longlong_as_double((long long)double_bits(v, -51));
+}
+
+// ---------------------------------------------------------------------------
+// lattices with non-unit links: the FP64 sequence
+// ---------------------------------------------------------------------------
+// Staple sum by the tree s_k = up_k + lo_k for the k-th nu != mu,
+// A = (s_0 + s_1) + s_2 (P = its prefix over nu < mu), FP64 draw, new link.
+// Returns what update_link returns; *un is the link's final value.
+static __device__ __noinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, uint32_t i,
+                                                    int mu, int p, bool hyb, double* plaq,
+                                                    uint32_t* lex)
+{
+    const Links<double> U(ctx.links, D, ctx.status);
+    const EoSite s(D, i, p);
+    int hp[4], hm[4];
+    s.hops(hp, hm);
+    Quat<double> A = {0, 0, 0, 0}, P = A;
+    for (int nu = 0, k = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        const Quat<double> sk = qadd(staple_term<double>(U, mu, nu, p, i, hp, hm, false),
+                                     staple_term<double>(U, mu, nu, p, i, hp, hm, true));
+        A = k++ == 0 ? sk : qadd(A, sk);
+        if (nu == mu - 1) P = A;
+    }
+    *lex = s.lex();
+    Quat<double> un;
+    const int32_t tr = draw_link<double>(D, hyb, A, s.lex() * 4u + (uint32_t)mu, D.sweep, &un);
+    if (tr >= 0) U.store(mu, p, i, un);
+    else un = U.load_rw(mu, p, i);
+    *plaq += qretr(un, P);
+    return tr;
+}
+// the links i0, i0 + step, ... below end of one thread, then the warp totals
+template <int MU, bool PLAQ>
+__device__ __noinline__ void general_links(const Ctx& ctx, int l, uint32_t blk0, uint32_t i0,
+                                           uint32_t step, uint32_t end, int p, bool hyb, int32_t* dbg)
+{
+    const LatDesc& D = ctx.desc[l];
+    double plaq = 0.0;
+    uint32_t ntrial = 0, ncap = 0, lex;
+    for (uint32_t i = i0; i < end; i += step) {
+        const int32_t tr = general_link(ctx, D, i, MU, p, hyb, &plaq, &lex);
+        ncap += tr < 0;
+        ntrial += tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
+        if (dbg) dbg[lex] = tr;
+    }
+    __syncwarp();
+    fix_totals<MU, PLAQ>(ctx, l, blk0, D.Vh, PLAQ ? warp_sum_t(plaq) : 0.0, ntrial, ncap);
+}
+
+// ---------------------------------------------------------------------------
+// one link per thread
+// ---------------------------------------------------------------------------
+// NT, MINB bound the registers (255 or 128 a thread); smaller blocks of
+// the same register count run the same kernel.
+template <int MU, bool PLAQ, bool HYB, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+fix_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
+{
+    const int l = lattice_of_block(ctx.phase_start, ctx.n, blockIdx.x);
+    const LatDesc& D = ctx.desc[l];
+    const uint32_t Vh = D.Vh;
+    const uint32_t blk0 = first_block(ctx.phase_start, l);
+    const uint32_t i = (blockIdx.x - blk0) * blockDim.x + threadIdx.x;
+    if (D.nonunit) {
+        general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, i < Vh ? i + 1 : i, p, HYB, dbg);
+        return;
+    }
+    const Links<double> U(ctx.links, D, ctx.status);
+    const FixCall C(D);
+    int64_t plaq = 0;
+    uint32_t ntrial = 0, ncap = 0;
+    if (i < Vh) {
+        const EoSite s(D, i, p);
+        int64_t A[4], P[4], un[4];
+        fix_staple_sum<MU, PLAQ>(U, s, i, p, A, P);
+        const Stream st = C.stream(s.lex() * 4u + MU);
+        Drawn d;
+        double qc;
+        int32_t tr = -1;
+        if (!fix_prepare<HYB>(C, A, &d, &qc)) {
+            const Quat<double> h = haar_link(st);
+            U.store(MU, p, i, h);
+            if (PLAQ) fix_from_link(h, un);
+            tr = 0;
+        } else {
+            // trial 0 also carries the direction in the low 9 bits of its words
+            U4 w = st.draw(TAG_TRIAL, 0u);
+            const uint32_t kd1 = spare_bits_1(w), kd2 = spare_bits_2(w);
+            Lambda L;
+            for (int t = 0;;) {
+                if (fix_try<HYB>(C, w, d.inv, d.ei, qc, &L)) {
+                    tr = t + 1;
+                    break;
+                }
+                if (++t == KP_CAP) break;
+                w = st.draw(TAG_TRIAL, (uint32_t)t);
+            }
+            if (tr > 0) {
+                new_link_fix(L, kd1, kd2, d.V, C.tab, un);
+                U.store(MU, p, i, dq_link(un));
+            } else {
+                ncap = 1;
+                if (PLAQ) fix_from_link(U.load_rw(MU, p, i), un);
+            }
+        }
+        ntrial = tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
+        if (dbg) dbg[s.lex()] = tr;
+        if (PLAQ) plaq = retr_fix(un, P);
+    }
+    fix_totals<MU, PLAQ>(ctx, l, blk0, Vh, PLAQ ? plaq_double(warp_sum64(plaq)) : 0.0, ntrial,
+                             ncap);
+}
+
+// ---------------------------------------------------------------------------
+// R links per thread with a per-warp retry queue
+// ---------------------------------------------------------------------------
+// The warp alternates between two steps.  Step 1 takes 32 links: each lane
+// forms its link's staple sum and puts the draw's inputs (unit staple,
+// 1 / (2 alpha), counter word, trial index, storage index) into a queue in
+// shared memory.  Step 2 takes the last 32 of the queue, one trial a lane:
+// an accepted link is finished, a rejected one goes back with its next
+// trial.  Step 1 runs while fewer than 32 links wait, so nearly every trial
+// runs with all lanes, each step has one copy of its code, and the registers
+// of the staple sum and of the draw are not held together.
+template <bool PLAQ, bool HYB>
+struct FixQueue {
+    static constexpr int CAP = 64;  // < 32 held before a push of at most 32
+    int64_t pl[PLAQ ? 4 : 1][PLAQ ? CAP : 1];
+    int64_t inv[CAP];
+    double qc[HYB ? CAP : 1];
+    Fx v[4][CAP];
+    int32_t ei[CAP];
+    uint32_t key[CAP];
+    uint32_t tk[CAP];    // next trial | first 18-bit direction word << 13
+    uint32_t kd2[CAP];   // second 18-bit direction word (both set by trial 0)
+    uint32_t site[CAP];  // storage index
+};
+
+// R <= FIX_MAX_ROUNDS: the warp's plaquette sum (6 * 2^51 a link, 32 R
+// links) stays below 2^63.
+constexpr int FIX_MAX_ROUNDS = 16;
+template <int MU, bool PLAQ, bool HYB, bool PERSIST>
+__global__ void __launch_bounds__(32, 16)
+fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
+{
+    static_assert(KP_CAP <= (1 << 13), "trial index must fit 13 bits");
+    constexpr uint32_t NT = 32;
+    using Queue = FixQueue<PLAQ, HYB>;
+    __shared__ Queue Q;
+
+    const int l = lattice_of_block(ctx.phase_start, ctx.n, blockIdx.x);
+    const LatDesc& D = ctx.desc[l];
+    const uint32_t Vh = D.Vh;
+    const uint32_t blk0 = first_block(ctx.phase_start, l);
+    // tiles of 32 R positions; a persistent block takes every nb-th
+    const uint32_t nb = PERSIST ? __ldg(ctx.phase_start + l + 1) - blk0 : 0u;
+    const uint32_t tile0 = blockIdx.x - blk0;
+    if (D.nonunit) {
+        if (PERSIST) {
+            general_links<MU, PLAQ>(ctx, l, blk0, tile0 * NT + threadIdx.x, nb * NT, Vh, p, HYB, dbg);
+        } else {
+            const uint32_t i0 = tile0 * (NT * R) + threadIdx.x;
+            general_links<MU, PLAQ>(ctx, l, blk0, i0, NT, min(Vh, (tile0 + 1) * (NT * R)), p, HYB, dbg);
+        }
+        return;
+    }
+    const Links<double> U(ctx.links, D, ctx.status);
+    const FixCall C(D);
+    const int lane = threadIdx.x;
+    const uint32_t below = (1u << lane) - 1u;
+
+    int64_t plaq = 0, plaq_hi = 0;  // at 2^51, and (persistent) 2^31
+    uint32_t ntrial = 0, ncap = 0;
+    int cnt = 0;                    // queued links (warp-uniform)
+    uint32_t base = tile0 * (NT * R), left = R;  // next 32 positions, rounds left in the tile
+
+    while (true) {
+        bool pend = false;
+        Drawn d;
+        int64_t P[4];
+        double qc = 0.0;
+        uint32_t key = 0, tk = 0, kd2 = 0, i;
+        if (cnt < 32 && base < Vh) {
+            // step 1
+            i = base + lane;
+            if (i < Vh) {
+                const EoSite s(D, i, p);
+                int64_t A[4];
+                fix_staple_sum<MU, PLAQ>(U, s, i, p, A, P);
+                key = s.lex() * 4u + MU;
+                pend = fix_prepare<HYB>(C, A, &d, &qc);
+                if (!pend) {
+                    const Quat<double> h = haar_link(C.stream(key));
+                    U.store(MU, p, i, h);
+                    if (PLAQ) {
+                        int64_t un[4];
+                        fix_from_link(h, un);
+                        plaq += retr_fix(un, P);
+                    }
+                    if (dbg) dbg[key >> 2] = 0;
+                }
+            }
+            base += NT;
+            if (--left == 0) {
+                left = R;
+                base = PERSIST ? base + (nb - 1) * (NT * R) : Vh;
+                if (PLAQ && PERSIST) {
+                    plaq_hi += plaq >> 20;
+                    plaq &= (int64_t(1) << 20) - 1;
+                }
+            }
+        } else if (cnt > 0) {
+            // step 2
+            const int n = cnt < 32 ? cnt : 32;
+            const bool have = lane < n;
+            const int e = have ? cnt - n + lane : 0;
+            d.V = {Q.v[0][e], Q.v[1][e], Q.v[2][e], Q.v[3][e]};
+            d.inv = Q.inv[e];
+            d.ei = Q.ei[e];
+            if (PLAQ) { P[0] = Q.pl[0][e]; P[1] = Q.pl[1][e]; P[2] = Q.pl[2][e]; P[3] = Q.pl[3][e]; }
+            if (HYB) qc = Q.qc[e];
+            key = Q.key[e];
+            tk = Q.tk[e];
+            kd2 = Q.kd2[e];
+            i = Q.site[e];
+            __syncwarp();
+            cnt -= n;
+            if (have) {
+                const uint32_t t = tk & 0x1FFFu;
+                const U4 w = C.stream(key).draw(TAG_TRIAL, t);
+                // trial 0 also carries the direction in the low 9 bits of its words
+                if (t == 0) {
+                    tk = spare_bits_1(w) << 13;
+                    kd2 = spare_bits_2(w);
+                }
+                Lambda L;
+                int64_t un[4];
+                if (fix_try<HYB>(C, w, d.inv, d.ei, qc, &L)) {
+                    new_link_fix(L, tk >> 13, kd2, d.V, C.tab, un);
+                    U.store(MU, p, i, dq_link(un));
+                    if (PLAQ) plaq += retr_fix(un, P);
+                    ntrial += t + 1;
+                    if (dbg) dbg[key >> 2] = (int32_t)t + 1;
+                } else if (t + 1 >= (uint32_t)KP_CAP) {
+                    // cap hit: the link keeps its value
+                    ncap += 1;
+                    ntrial += (uint32_t)KP_CAP;
+                    if (PLAQ) {
+                        fix_from_link(U.load_rw(MU, p, i), un);
+                        plaq += retr_fix(un, P);
+                    }
+                    if (dbg) dbg[key >> 2] = -1;
+                } else {
+                    pend = true;
+                    ++tk;
+                }
+            }
+        } else {
+            break;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, pend);
+        if (pend) {
+            const int e = cnt + __popc(m & below);
+            Q.v[0][e] = d.V.a0; Q.v[1][e] = d.V.a1; Q.v[2][e] = d.V.a2; Q.v[3][e] = d.V.a3;
+            if (PLAQ) { Q.pl[0][e] = P[0]; Q.pl[1][e] = P[1]; Q.pl[2][e] = P[2]; Q.pl[3][e] = P[3]; }
+            Q.inv[e] = d.inv;
+            Q.ei[e] = d.ei;
+            if (HYB) Q.qc[e] = qc;
+            Q.key[e] = key;
+            Q.tk[e] = tk;
+            Q.kd2[e] = kd2;
+            Q.site[e] = i;
+        }
+        cnt += __popc(m);
+        __syncwarp();
+    }
+    double wp = 0.0;
+    if (PLAQ) {
+        wp = plaq_double(warp_sum64(plaq));
+        if (PERSIST) wp += __longlong_as_double((long long)double_bits(warp_sum64(plaq_hi), -31));
+    }
+    fix_totals<MU, PLAQ>(ctx, l, blk0, Vh, wp, ntrial, ncap);
+}
+
+// ---------------------------------------------------------------------------
+// eight lanes per link: small lattices
+// ---------------------------------------------------------------------------
+// A small lattice (8^4: 2048 links per phase) has one warp of one link per
+// thread for a tenth of the SM sub-partitions, and a phase lasts as long as
+// one link's chain.  Here lanes 0..5 of a group of eight compute the six
+// staple terms at once, their integer sums meet in a butterfly (any order
+// gives the same bits), and the eight lanes try eight trials at once; the
+// link takes the first accepted one of its own sequence.
+template <int MU, bool PLAQ, bool HYB>
+__global__ void __launch_bounds__(64, 8)
+fix_coop_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
+{
+    constexpr int G = 8;
+    static_assert(KP_CAP % G == 0, "whole trial groups");
+    const int l = lattice_of_block(ctx.phase_start, ctx.n, blockIdx.x);
+    const LatDesc& D = ctx.desc[l];
+    const uint32_t Vh = D.Vh;
+    const uint32_t blk0 = first_block(ctx.phase_start, l);
+    const int lane = threadIdx.x & 31, g = lane & (G - 1), g0 = lane & ~(G - 1);
+    const uint32_t i = (blockIdx.x - blk0) * (blockDim.x / G) + threadIdx.x / G;
+    const bool act = i < Vh;  // uniform within the group
+    if (D.nonunit) {
+        general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, act && g == 0 ? i + 1 : i, p, HYB, dbg);
+        return;
+    }
+    const Links<double> U(ctx.links, D, ctx.status);
+    const FixCall C(D);
+
+    int64_t A[4] = {0, 0, 0, 0}, P[4] = {0, 0, 0, 0};
+    uint32_t key = 0;
+    if (act) {
+        const EoSite s(D, i, p);
+        int hp[4], hm[4];
+        s.hops(hp, hm);
+        key = s.lex() * 4u + MU;
+        if (g < 6) {
+            const int nu = nu_of<MU>(g >> 1);
+            const int hpn = nu == 0 ? hp[0] : (nu == 1 ? hp[1] : (nu == 2 ? hp[2] : hp[3]));
+            const int hmn = nu == 0 ? hm[0] : (nu == 1 ? hm[1] : (nu == 2 ? hm[2] : hm[3]));
+            fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, (g & 1) != 0, A);
+            if (PLAQ && nu < MU) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) P[c] = A[c];
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            A[c] += (int64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)A[c], o);
+            if (PLAQ && MU < 3)
+                P[c] += (int64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)P[c], o);
+        }
+    }
+    if (PLAQ && MU == 3) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) P[c] = A[c];
+    }
+    const Stream st = C.stream(key);
+    Drawn d;
+    double qc;
+    const bool haar = !fix_prepare<HYB>(C, A, &d, &qc);
+    bool done = !act || haar;
+    int32_t tr = -1;
+    Lambda L = {0, 0, 0};
+    uint32_t kd1 = 0, kd2 = 0;
+    for (int t0 = 0; t0 < KP_CAP; t0 += G) {
+        if (!__any_sync(0xffffffffu, !done)) break;
+        const U4 w = st.draw(TAG_TRIAL, (uint32_t)(t0 + g));
+        if (t0 == 0) {  // the direction: spare bits of trial 0 (lane g0)
+            kd1 = __shfl_sync(0xffffffffu, spare_bits_1(w), g0);
+            kd2 = __shfl_sync(0xffffffffu, spare_bits_2(w), g0);
+        }
+        Lambda M = {0, 0, 0};
+        const bool ok = !done && fix_try<HYB>(C, w, d.inv, d.ei, qc, &M);
+        const uint32_t m = (__ballot_sync(0xffffffffu, ok) >> g0) & ((1u << G) - 1u);
+        const int src = g0 + (m ? __ffs(m) - 1 : 0);
+        M.P = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)M.P, src);
+        M.lam = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)M.lam, src);
+        M.qe = __shfl_sync(0xffffffffu, M.qe, src);
+        if (!done && m) {
+            done = true;
+            tr = t0 + __ffs(m);
+            L = M;
+        }
+    }
+    int64_t plaq = 0;
+    uint32_t ntrial = 0, ncap = 0;
+    if (act && g == 0) {
+        int64_t un[4];
+        if (haar) {
+            const Quat<double> h = haar_link(st);
+            U.store(MU, p, i, h);
+            if (PLAQ) fix_from_link(h, un);
+            tr = 0;
+        } else if (tr > 0) {
+            new_link_fix(L, kd1, kd2, d.V, C.tab, un);
+            U.store(MU, p, i, dq_link(un));
+        } else {
+            ncap = 1;
+            if (PLAQ) fix_from_link(U.load_rw(MU, p, i), un);
+        }
+        ntrial = tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
+        if (dbg) dbg[key >> 2] = tr;
+        if (PLAQ) plaq = retr_fix(un, P);
+    }
+    __syncwarp();
+    fix_totals<MU, PLAQ>(ctx, l, blk0, Vh, PLAQ ? plaq_double(warp_sum64(plaq)) : 0.0, ntrial,
+                             ncap);
+}
+
+}  // namespace su2

@@ -10,7 +10,8 @@
 // A = k Vhat collects the six plaquettes through U_mu(x).  Links of one
 // phase share no staple, so all of them are updated at once.
 // (The paper's benchmark, Sec. 2.1: random SU(2) start, heat-bath
-// iterations, mean plaquette after each.)
+// iterations, mean plaquette after each.)  FP32 kernels here; the FP64 ones
+// are in heatbath_fixed.cuh.
 //
 // Per link: 18 neighbour loads (7 distinct links per update on average over
 // the phase: V/2 opposite-parity U_mu plus 3V other-direction links for V/2
@@ -78,22 +79,14 @@ __device__ __forceinline__ T warp_sum_t(T v)
 // of the planes (nu, mu).  P is A after its first mu terms, so it costs no
 // extra additions.
 //
-// The order of the additions is fixed per precision, and every kernel of a
-// precision keeps it, so all launch shapes give the same bits.  FP32 folds
-// the sums into the products' last multiply-adds (A = A + up + lo, ν by ν).
-// FP64 sums a tree: s_k = up_k + lo_k for the k-th ν != mu, then
-// A = (s_0 + s_1) + s_2 (P = the prefix over ν < mu), the order in which
-// the cooperative kernel's lanes, which compute the six terms in parallel,
-// can reproduce it.
+// The order of the additions is fixed, so all launch shapes give the same
+// bits: FP32 folds the sums into the products' last multiply-adds (A = A +
+// up + lo, nu by nu).
 template <int MU>
 __device__ __forceinline__ constexpr int nu_of(int k) { return k + (k >= MU ? 1 : 0); }
 
-// the upper (a b^dagger c^dagger) or lower ((e d)^dagger f) staple term of
-// U_mu(x) in the plane (nu, mu).  Both are formed as x y^dagger z^dagger:
-// the lower one is d^dagger e^dagger f, i.e. x = d^dagger, y = e,
-// z = f^dagger (conjugation is an exact sign flip), so that lanes computing
-// upper and lower terms side by side run one instruction stream (the
-// cooperative kernel).
+// the upper (a b^dagger c^dagger) or lower (d^dagger e^dagger f) staple term
+// of U_mu(x) in the plane (nu, mu), as the FP64 sequence forms them
 template <typename T, typename LT>
 __device__ __forceinline__ Quat<T> staple_term(const LT& U, int mu, int nu, int p, uint32_t i,
                                                const int* hp, const int* hm, bool lower)
@@ -119,38 +112,25 @@ __device__ __forceinline__ void staple_sum(const LT& U, const EoSite& s, uint32_
 {
     int hp[4], hm[4];
     s.hops(hp, hm);
-    if constexpr (std::is_same<T, double>::value) {
-        Quat<T> sk[3];
+    const int q = p ^ 1;
+    const uint32_t e_pmu = i + hp[MU];
+    A = {T(0), T(0), T(0), T(0)};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int nu = nu_of<MU>(k);
-            sk[k] = qadd(staple_term<T>(U, MU, nu, p, i, hp, hm, false),
-                         staple_term<T>(U, MU, nu, p, i, hp, hm, true));
-        }
-        const Quat<T> s01 = qadd(sk[0], sk[1]);
-        A = qadd(s01, sk[2]);
-        if (PLAQ) P = MU == 1 ? sk[0] : (MU == 2 ? s01 : A);
-    } else {
-        const int q = p ^ 1;
-        const uint32_t e_pmu = i + hp[MU];
-        A = {T(0), T(0), T(0), T(0)};
-#pragma unroll
-        for (int nu = 0; nu < 4; ++nu) {
-            if (nu == MU) continue;
-            const uint32_t e_pnu = i + hp[nu];
-            const uint32_t e_mnu = i + hm[nu];
-            const uint32_t e_pmu_mnu = i + hp[MU] + hm[nu];
-            const Quat<T> a = U.load(nu, q, e_pmu);      // U_nu(x+mu)
-            const Quat<T> b = U.load(MU, q, e_pnu);      // U_mu(x+nu)
-            const Quat<T> c = U.load(nu, p, i);          // U_nu(x)
-            const Quat<T> d = U.load(nu, p, e_pmu_mnu);  // U_nu(x+mu-nu)
-            const Quat<T> e = U.load(MU, q, e_mnu);      // U_mu(x-nu)
-            const Quat<T> f = U.load(nu, q, e_mnu);      // U_nu(x-nu)
-            // A += a b^dagger c^dagger + (e d)^dagger f, the sums fused into
-            // the products' last steps
-            A = qmul_dn_acc(qmul(e, d), f, qmul_nd_acc(qmul_nd(a, b), c, A));
-            if (PLAQ && nu == MU - 1) P = A;
-        }
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == MU) continue;
+        const uint32_t e_pnu = i + hp[nu];
+        const uint32_t e_mnu = i + hm[nu];
+        const uint32_t e_pmu_mnu = i + hp[MU] + hm[nu];
+        const Quat<T> a = U.load(nu, q, e_pmu);      // U_nu(x+mu)
+        const Quat<T> b = U.load(MU, q, e_pnu);      // U_mu(x+nu)
+        const Quat<T> c = U.load(nu, p, i);          // U_nu(x)
+        const Quat<T> d = U.load(nu, p, e_pmu_mnu);  // U_nu(x+mu-nu)
+        const Quat<T> e = U.load(MU, q, e_mnu);      // U_mu(x-nu)
+        const Quat<T> f = U.load(nu, q, e_mnu);      // U_nu(x-nu)
+        // A += a b^dagger c^dagger + (e d)^dagger f, the sums fused into
+        // the products' last steps
+        A = qmul_dn_acc(qmul(e, d), f, qmul_nd_acc(qmul_nd(a, b), c, A));
+        if (PLAQ && nu == MU - 1) P = A;
     }
 }
 
@@ -277,6 +257,25 @@ __device__ __forceinline__ uint32_t spare_bits_2(const U4& w) { return ((w.z & 5
 // block's slowest warp): trial counts go to spread per-lattice atomic slots
 // (exact integers), cap hits to an atomic only when present, the
 // plaquette to one partial per warp, summed later in a fixed order.
+// lane 0 of warp w of the block: the warp's totals wp, wt, wc
+// (wpb: warps per block)
+template <int MU, bool PLAQ>
+__device__ __forceinline__ void add_warp_totals(const Ctx& ctx, uint32_t wpb, int l, uint32_t blk0,
+                                                uint32_t Vh, double wp, int w, uint32_t wt,
+                                                uint32_t wc)
+{
+    const uint32_t gw = blockIdx.x * wpb + w;  // global warp index
+    if (PLAQ) ctx.plaq_partial[(size_t)(MU - 1) * ctx.phase_blocks * wpb + gw] = wp;
+    atomicAdd(ctx.trial_slots + (size_t)l * TRIAL_SLOTS + (gw % TRIAL_SLOTS),
+              (unsigned long long)wt);
+    LatDesc* Dw = ctx.desc + l;
+    if (w == 0 && blockIdx.x == blk0) atomicAdd(&Dw->updates, (unsigned long long)Vh);
+    if (wc) {
+        atomicAdd(&Dw->caps, (unsigned long long)wc);
+        atomicOr(ctx.status, STATUS_CAP_HIT);
+    }
+}
+
 template <typename T, int MU, bool PLAQ, int NT>
 __device__ __forceinline__ void warp_totals(const Ctx& ctx, int l, uint32_t blk0, uint32_t Vh,
                                             T plaq, uint32_t ntrial, uint32_t ncap)
@@ -286,41 +285,23 @@ __device__ __forceinline__ void warp_totals(const Ctx& ctx, int l, uint32_t blk0
     const uint32_t wc = __reduce_add_sync(0xffffffffu, ncap);
     T wp = T(0);
     if (PLAQ) wp = warp_sum_t(plaq);
-    if (lane == 0) {
-        const uint32_t gw = blockIdx.x * (NT / 32) + w;  // global warp index
-        if (PLAQ)
-            ctx.plaq_partial[(size_t)(MU - 1) * ctx.phase_blocks * (NT / 32) + gw] = (double)wp;
-        atomicAdd(ctx.trial_slots + (size_t)l * TRIAL_SLOTS + (gw % TRIAL_SLOTS),
-                  (unsigned long long)wt);
-        LatDesc* Dw = ctx.desc + l;
-        if (w == 0 && blockIdx.x == blk0) atomicAdd(&Dw->updates, (unsigned long long)Vh);
-        if (wc) {
-            atomicAdd(&Dw->caps, (unsigned long long)wc);
-            atomicOr(ctx.status, STATUS_CAP_HIT);
-        }
-    }
+    if (lane == 0) add_warp_totals<MU, PLAQ>(ctx, NT / 32, l, blk0, Vh, (double)wp, w, wt, wc);
 }
 
-// One link update, U_mu(x) at storage index i of parity p in sweep sw: the
-// staple sum, the Kennedy-Pendleton (or Creutz) draw and the new link *un.
-// Returns the trials used (> 0), 0 for the Haar branch (alpha -> 0) or -1
-// when the cap was hit (*un then undefined); *P is the staple part closing
-// the plaquettes (PLAQ).
-template <typename T, int MU, bool PLAQ, bool HYB, typename LT>
-__device__ __forceinline__ int32_t update_link(const LT& U, const LatDesc& D, const EoSite& s,
-                                               uint32_t i, int p, uint64_t sw, Quat<T>* un,
-                                               Quat<T>* P)
+// The draw of one link from its staple sum A: Kennedy-Pendleton (or, HYB,
+// Creutz) and the new link *un.  Returns the trials used (> 0), 0 for the
+// Haar branch (alpha -> 0) or -1 when the cap was hit (*un then undefined).
+template <typename T>
+__device__ __forceinline__ int32_t draw_link(const LatDesc& D, bool hyb, const Quat<T>& A,
+                                             uint32_t key, uint64_t sw, Quat<T>* un)
 {
-    Quat<T> A;
-    staple_sum<T, MU, PLAQ>(U, s, i, p, A, *P);
-
     // alpha = beta k and 1/(2 alpha) from one reciprocal square root of k^2
     const T k2 = qnorm2(A);
     const T rk = Math<T>::rsqrt(k2);
     const T beta = beta_of<T>(D);
     const T alpha = mul_(mul_(beta, k2), rk);
-    const Stream st{(uint32_t)D.seed, (uint32_t)(D.seed >> 32), s.lex() * 4u + MU,
-                    (uint32_t)sw, (uint32_t)(sw >> 32)};
+    const Stream st{(uint32_t)D.seed, (uint32_t)(D.seed >> 32), key, (uint32_t)sw,
+                    (uint32_t)(sw >> 32)};
 
     if (!(alpha >= alpha_haar<T>())) {
         // alpha -> 0 limit of the conditional law (zero staple or beta = 0)
@@ -333,7 +314,7 @@ __device__ __forceinline__ int32_t update_link(const LT& U, const LatDesc& D, co
     // trial 0 also carries the direction in the low 9 bits of its words
     const U4 w = st.draw(TAG_TRIAL, 0u);
     const uint32_t kd1 = spare_bits_1(w), kd2 = spare_bits_2(w);
-    if (HYB && alpha < creutz_of<T>(D)) {
+    if (hyb && alpha < creutz_of<T>(D)) {
         const T qc = creutz_qc(alpha);
         for (int t = 0; t < KP_CAP; ++t) {
             if (creutz_try(t == 0 ? w : st.draw(TAG_TRIAL, (uint32_t)t), qc, inv2a, &delta)) {
@@ -353,6 +334,19 @@ __device__ __forceinline__ int32_t update_link(const LT& U, const LatDesc& D, co
     }
     if (tr > 0) *un = new_link(delta, kd1, kd2, A, D.fp64_table);
     return tr;
+}
+
+// One FP32 link update, U_mu(x) at storage index i of parity p in sweep sw:
+// the staple sum and the draw (returned as draw_link returns it); *P is the
+// staple part closing the plaquettes (PLAQ).
+template <typename T, int MU, bool PLAQ, bool HYB, typename LT>
+__device__ __forceinline__ int32_t update_link(const LT& U, const LatDesc& D, const EoSite& s,
+                                               uint32_t i, int p, uint64_t sw, Quat<T>* un,
+                                               Quat<T>* P)
+{
+    Quat<T> A;
+    staple_sum<T, MU, PLAQ>(U, s, i, p, A, *P);
+    return draw_link<T>(D, HYB, A, s.lex() * 4u + MU, sw, un);
 }
 
 // ---------------------------------------------------------------------------
@@ -944,251 +938,13 @@ hb_pair_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     warp_totals<float, MU, PLAQ, NT>(ctx, l, blk0, Vh, plaq, ntrial, ncap);
 }
 
-// ---------------------------------------------------------------------------
-// FP64, G lanes per link: the cooperative kernel for small lattices
-// ---------------------------------------------------------------------------
-// On GB300 an FP64 warp instruction holds its SM sub-partition's FP64 unit
-// for ~76 cycles, with one active lane as with 32, and a dependent one
-// waits no longer than that; a small lattice (8^4: 2048 links per phase =
-// 64 warps of one link per thread) leaves most sub-partitions without
-// work.  Here G = 8 lanes share one link, and the phase takes about as long
-// as one warp's stream of FP64 instructions, so the link's work is laid
-// out for few instructions, not few lanes: lanes 0..5 compute the six
-// staple terms at once (upper and lower in one stream), the sums follow the
-// FP64 tree order above one component per lane, the lanes try
-// Kennedy-Pendleton trials t0 .. t0 + 3 at once (one logarithm per lane)
-// while two of them take the direction's cosine and sine in the trials'
-// cospi stream, the two square roots of the new link share one stream, and
-// lanes 0..3 form one component each of the final product.  The link takes the first
-// accepted trial of its own sequence, as every other kernel does, and each
-// value comes from the same operations as in the scalar kernels, so links
-// and trial counts are bit-identical to theirs.
-// x with its sign flipped where m has bit 63 set (an integer operation)
-__device__ __forceinline__ double flip_sign(double x, uint64_t m)
-{
-    return __longlong_as_double(__double_as_longlong(x) ^ (long long)m);
-}
-__device__ __forceinline__ Quat<double> qdag_if(const Quat<double>& q, uint64_t m)
-{
-    return {q.a0, flip_sign(q.a1, m), flip_sign(q.a2, m), flip_sign(q.a3, m)};
-}
-
-// the k-th of four values, by selects (no indexed local array)
-template <typename V>
-__device__ __forceinline__ V pick4(int k, V v0, V v1, V v2, V v3)
-{
-    return k == 0 ? v0 : (k == 1 ? v1 : (k == 2 ? v2 : v3));
-}
-
-// Component c of p q^dagger: qmul_nd's multiply and three fused
-// multiply-adds for that component, in its order, on operands picked per
-// lane, so four lanes form the four components in one stream with
-// qmul_nd's bits.
-__device__ __forceinline__ double qmul_nd_part(int c, const Quat<double>& p, const Quat<double>& q)
-{
-    constexpr uint64_t S = 0x8000000000000000ull;
-    const double x0 = pick4(c, p.a0, p.a1, p.a2, p.a3);
-    const double x1 = c == 0 ? p.a1 : p.a0;
-    const double x2 = (c == 1 || c == 2) ? p.a3 : p.a2;
-    const double x3 = pick4(c, p.a3, p.a2, p.a1, p.a1);
-    const double y1 = flip_sign(pick4(c, q.a1, q.a1, q.a2, q.a3), c != 0 ? S : 0ull);
-    const double y2 = flip_sign(pick4(c, q.a2, q.a2, q.a1, q.a1), (c & 1) ? S : 0ull);
-    const double y3 = flip_sign(pick4(c, q.a3, q.a3, q.a3, q.a2), c == 2 ? S : 0ull);
-    return fma_(x3, y3, fma_(x2, y2, fma_(x1, y1, mul_(x0, q.a0))));
-}
-
-template <typename T, int MU, bool PLAQ, bool DBG, int NT, int MINB, bool HYB, int G>
-__global__ void __launch_bounds__(NT, MINB)
-hb_phase_coop_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
-{
-    static_assert(G == 8 && KP_CAP % G == 0, "eight lanes per link, whole trial groups");
-    static_assert(std::is_same<T, double>::value, "the FP64 tree order of the staple");
-    constexpr uint64_t SIGN = 0x8000000000000000ull;
-    const int l = lattice_of_block(ctx.phase_start, ctx.n, blockIdx.x);
-    const LatDesc& D = ctx.desc[l];
-    const uint32_t Vh = D.Vh;
-    const uint32_t blk0 = first_block(ctx.phase_start, l);
-    const int lane = threadIdx.x & 31, g = lane & (G - 1), g0 = lane & ~(G - 1);
-    const uint32_t j = (blockIdx.x - blk0) * (NT / G) + threadIdx.x / G;  // link position
-    const bool act = j < Vh;  // uniform within the group
-    const Links<T> U(ctx.links, D, ctx.status);
-    // the per-call values, loaded up front (they are needed only after the
-    // staple, and their loads then wait on nothing)
-    const uint64_t sw = D.sweep, seed = D.seed;
-    const T beta = beta_of<T>(D), hib = D.half_inv_beta;
-    const double2* const lnt = D.fp64_table;
-
-    Quat<T> term = {T(0), T(0), T(0), T(0)};
-    uint32_t key = 0;
-    const uint32_t i = j;
-    if (act) {
-        const EoSite s(D, j, p);
-        int hp[4], hm[4];
-        s.hops(hp, hm);
-        key = s.lex() * 4u + MU;
-        if (g < 6) {
-            // lane 2k: the upper term of the k-th nu != mu, (a, b, c) =
-            // (U_nu(x+mu), U_mu(x+nu), U_nu(x)); lane 2k+1: the lower one,
-            // (d^dagger, e, f^dagger) = (U_nu(x+mu-nu)^dagger, U_mu(x-nu),
-            // U_nu(x-nu)^dagger); each lane forms x y^dagger z^dagger
-            const int nu = nu_of<MU>(g >> 1);
-            const bool lower = (g & 1) != 0;
-            const int q = p ^ 1;
-            const int hpn = pick4(nu, hp[0], hp[1], hp[2], hp[3]);
-            const int hmn = pick4(nu, hm[0], hm[1], hm[2], hm[3]);
-            const uint64_t m = lower ? SIGN : 0ull;
-            const Quat<T> x = qdag_if(U.load(nu, lower ? p : q, i + hp[MU] + (lower ? hmn : 0)), m);
-            const Quat<T> y = U.load(MU, q, i + (lower ? hmn : hpn));
-            const Quat<T> z = qdag_if(U.load(nu, lower ? q : p, lower ? i + hmn : i), m);
-            term = qmul_nd(qmul_nd(x, y), z);
-        }
-    }
-    // The tree s_k = up_k + lo_k, A = (s_0 + s_1) + s_2 one component per
-    // lane: the terms go through shared memory, lane (kk, c) = (g >> 2, g & 3)
-    // adds component c of s_kk and of s_2, lanes c and c + 4 swap theirs,
-    // and every lane then holds component c of s_0, s_1, s_01 and A (four
-    // additions in the stream instead of twelve).
-    __shared__ double terms[NT / G][6][4];
-    double* const tg6 = &terms[threadIdx.x / G][0][0];
-    if (g < 6) {
-        reinterpret_cast<double2*>(tg6 + 4 * g)[0] = make_double2(term.a0, term.a1);
-        reinterpret_cast<double2*>(tg6 + 4 * g)[1] = make_double2(term.a2, term.a3);
-    }
-    __syncwarp();
-    const int c = g & 3, kk = g >> 2;
-    const T skc = add_(tg6[4 * (2 * kk) + c], tg6[4 * (2 * kk + 1) + c]);
-    const T s2c = add_(tg6[16 + c], tg6[20 + c]);
-    const T swp = __shfl_sync(0xffffffffu, skc, lane ^ 4);
-    const T s0c = kk ? swp : skc, s1c = kk ? skc : swp;
-    const T s01c = add_(s0c, s1c);
-    const T Ac = add_(s01c, s2c);
-    auto gather = [&](T v) -> Quat<T> {
-        return {__shfl_sync(0xffffffffu, v, g0), __shfl_sync(0xffffffffu, v, g0 + 1),
-                __shfl_sync(0xffffffffu, v, g0 + 2), __shfl_sync(0xffffffffu, v, g0 + 3)};
-    };
-    const Quat<T> A = gather(Ac);
-    Quat<T> P = A;
-    if (PLAQ && MU < 3) P = gather(MU == 1 ? s0c : s01c);
-
-    const T k2 = qnorm2(A);
-    const T rk = Math<T>::rsqrt(k2);
-    const T alpha = mul_(mul_(beta, k2), rk);
-    const Stream st{(uint32_t)seed, (uint32_t)(seed >> 32), key, (uint32_t)sw,
-                    (uint32_t)(sw >> 32)};
-    const bool haar = !(alpha >= alpha_haar<T>());
-    const T inv2a = mul_(rk, hib);  // inv_two_alpha's product
-    const bool creutz = HYB && alpha < creutz_of<T>(D);
-    const T qc = creutz ? creutz_qc(alpha) : T(0);
-
-    // Kennedy-Pendleton: lanes g and g + 4 share trial t0 + (g & 3), lane g
-    // taking ln r1 and lane g + 4 ln r3, so each lane evaluates one logarithm
-    // per pass and a pass tries four trials; in the first pass lanes 4 and 5
-    // take the direction's cos(phi) and sin(phi), phi = 2 pi u2, from the
-    // table's sine/cosine stream in place of the cos(2 pi r2) that only
-    // lanes 0..3 use.
-    // Creutz's draw needs one logarithm per trial, so there each of the eight
-    // lanes tries its own (the direction still comes from lanes 4 and 5 of
-    // the first pass).  Each group advances its own t0; the warp loops while
-    // any link waits.
-    const int stride = creutz ? G : G / 2;
-    const int tg = creutz ? g : (g & 3);
-    bool done = !act || haar;
-    int32_t tr = -1;
-    T delta = T(0), cph = T(0), sph = T(0);
-    uint32_t kd1 = 0, kd2 = 0;
-    int t0 = 0;
-    for (int pass = 0;; ++pass) {
-        if (!done && t0 >= KP_CAP) done = true;  // cap hit: tr stays -1
-        if (!__any_sync(0xffffffffu, !done)) break;
-        const U4 w = st.draw(TAG_TRIAL, (uint32_t)(t0 + tg));
-        if (pass == 0) {  // the direction: spare bits of trial 0 (lane g0)
-            kd1 = __shfl_sync(0xffffffffu, spare_bits_1(w), g0);
-            kd2 = __shfl_sync(0xffffffffu, spare_bits_2(w), g0);
-        }
-        // kp_eval's pieces, with ln r3 from the partner lane (all lanes,
-        // outside the branch: the shuffles need the whole warp)
-        const T lnv = ln_u01_tab(g < 4 ? w.x : w.z, lnt);
-        const T ln3 = __shfl_sync(0xffffffffu, lnv, lane ^ 4);
-        // cos(2 pi r2) from the table; in the first pass lanes 4 and 5 take
-        // the direction's cos phi and sin phi from the same stream
-        const bool dir = pass == 0 && (g == 4 || g == 5);
-        T sv, cv;
-        sincospi_tab(dir ? 2u * kd2 + 1u : 2u * (w.y >> 9) + 1u, dir ? 18 : 23, lnt, &sv, &cv);
-        const T dv = dir && g == 5 ? sv : cv;
-        if (pass == 0) {
-            cph = __shfl_sync(0xffffffffu, dv, g0 + 4);
-            sph = __shfl_sync(0xffffffffu, dv, g0 + 5);
-        }
-        T d;
-        bool ok;
-        if (creutz) {
-            ok = creutz_try(w, qc, inv2a, &d);
-        } else {
-            const T lam2 = mul_(neg_(fma_(mul_(cv, cv), ln3, lnv)), inv2a);
-            d = add_(lam2, lam2);
-            const T r4 = u01<T>(w.w);
-            ok = g < 4 && mul_(r4, r4) <= add_(T(1), neg_(lam2));
-        }
-        ok = ok && !done;
-        const uint32_t m = (__ballot_sync(0xffffffffu, ok) >> g0) & ((1u << G) - 1u);
-        const int first = m ? __ffs(m) - 1 : 0;
-        const T dfirst = __shfl_sync(0xffffffffu, d, g0 + first);
-        if (!done && m) {
-            done = true;
-            tr = t0 + first + 1;
-            delta = dfirst;
-        }
-        t0 += stride;
-    }
-    // the new link, new_link's arithmetic: lane 4 takes sin(theta) =
-    // sqrt((1 - cth)(1 + cth)) and lane 5 |vector part| =
-    // sqrt((delta + (-0)) (2 - delta)) in one stream
-    const T one = T(1);
-    const T cth = dir_cth(kd1);
-    const bool l5 = g == 5;
-    const T root = Math<T>::sqrt_pos(
-        mul_(add_(l5 ? delta : one, l5 ? T(-0.0) : flip_sign(cth, SIGN)),
-             add_(l5 ? T(2) : one, l5 ? flip_sign(delta, SIGN) : cth)));
-    const T sth = __shfl_sync(0xffffffffu, root, g0 + 4);
-    const T vl = __shfl_sync(0xffffffffu, root, g0 + 5);
-    const T vs = mul_(vl, sth);
-    const Quat<T> X = {add_(one, neg_(delta)), mul_(vs, cph), mul_(vs, sph), mul_(vl, cth)};
-    // U = X A^dagger / |X A^dagger|: one component per lane, the norm on
-    // every lane, the scaled components gathered on lane 0
-    const T rc = qmul_nd_part(g & 3, X, A);
-    const Quat<T> r = {__shfl_sync(0xffffffffu, rc, g0), __shfl_sync(0xffffffffu, rc, g0 + 1),
-                       __shfl_sync(0xffffffffu, rc, g0 + 2), __shfl_sync(0xffffffffu, rc, g0 + 3)};
-    const T uc = mul_(rc, rsqrt_t(qnorm2(r)));
-    const Quat<T> unew = {__shfl_sync(0xffffffffu, uc, g0), __shfl_sync(0xffffffffu, uc, g0 + 1),
-                          __shfl_sync(0xffffffffu, uc, g0 + 2), __shfl_sync(0xffffffffu, uc, g0 + 3)};
-    T plaq = T(0);
-    uint32_t ntrial = 0, ncap = 0;
-    if (act && g == 0) {
-        Quat<T> un = unew;
-        if (haar) {
-            un = haar_from<T>(st.draw(TAG_DIRECTION, 0));
-            tr = 0;
-        }
-        if (tr >= 0) {
-            U.store(MU, p, i, un);
-        } else {
-            ncap = 1;
-            if (PLAQ) un = U.load_rw(MU, p, i);
-        }
-        ntrial = tr > 0 ? (uint32_t)tr : (tr < 0 ? (uint32_t)KP_CAP : 0u);
-        if (DBG) dbg[key >> 2] = tr;
-        if (PLAQ) plaq = qretr(un, P);
-    }
-    warp_totals<T, MU, PLAQ, NT>(ctx, l, blk0, Vh, plaq, ntrial, ncap);
-}
-
 // One launch shape (NT threads per block, at least MINB blocks per SM, R
 // links -- or with PAIRS, R site pairs -- per thread, persistent or not) of
 // the phase kernel; the grid covers ctx.phase_blocks blocks of NT R links
 // or pairs (fewer, each walking several tiles, for a persistent shape on a
 // single lattice).
 template <typename T, int NT, int MINB, bool SLAB, int R = 1, bool PERSIST = false,
-          bool PAIRS = false, int GROUP = 1, bool STAGE = false>
+          bool PAIRS = false, bool STAGE = false>
 cudaError_t launch_phase_shape(const Ctx& c, int mu, int parity, bool plaq, int32_t* dbg,
                                bool hyb, cudaStream_t s)
 {
@@ -1196,18 +952,14 @@ cudaError_t launch_phase_shape(const Ctx& c, int mu, int parity, bool plaq, int3
     const bool pl = plaq && parity == 1 && mu >= 1;
     const dim3 grid(c.phase_blocks), block(NT);
 #define SU2_K(MUV, PL, DB, H)                                                                   \
-    if constexpr (GROUP > 1 && std::is_same<T, double>::value)                                  \
-        hb_phase_coop_kernel<T, MUV, PL, DB, NT, MINB, H, GROUP><<<grid, block, 0, s>>>(        \
-            c, parity, dbg);                                                                    \
-    else if constexpr (PAIRS)                                                                   \
+    if constexpr (PAIRS)                                                                        \
         hb_pair_kernel<MUV, PL, DB, NT, MINB, SLAB, H, R, PERSIST><<<grid, block, 0, s>>>(      \
             c, parity, dbg);                                                                    \
     else if constexpr (R == 1 && !PERSIST && !STAGE)                                            \
         hb_phase_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H><<<grid, block, 0, s>>>(c, parity, dbg); \
     else                                                                                        \
-        hb_phase_queue_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H, R, PERSIST,                     \
-                              STAGE && std::is_same<T, float>::value><<<grid, block, 0, s>>>(     \
-            c, parity, dbg)
+        hb_phase_queue_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H, R, PERSIST, STAGE>              \
+            <<<grid, block, 0, s>>>(c, parity, dbg)
 #define SU2_LAUNCH_H(MUV, H)                                    \
     do {                                                        \
         if (dbg) { SU2_K(MUV, false, true, H); }                \

@@ -1,6 +1,6 @@
 // heatbath_shapes.cu -- phase-kernel instantiations for two launch shapes
-// of one row of the shape table.  The build compiles this file once per
-// pair, with SU2_ROW = 0 (FP32), 1 (FP64) or 2 (FP32 site pairs) and
+// of one FP32 row of the shape table.  The build compiles this file once per
+// pair, with SU2_ROW = 0 (FP32) or 2 (FP32 site pairs) and
 // SU2_FIRST the first shape index of the pair, so that the shapes compile
 // in parallel.
 #include <type_traits>
@@ -8,7 +8,7 @@
 #include "heatbath_kernel.cuh"
 
 #if !defined(SU2_ROW) || !defined(SU2_FIRST)
-#error "compile with -DSU2_ROW=<0|1|2> -DSU2_FIRST=<even shape index>"
+#error "compile with -DSU2_ROW=<0|2> -DSU2_FIRST=<even shape index>"
 #endif
 
 namespace su2 {
@@ -17,16 +17,17 @@ template <int ROW, int FIRST>
 cudaError_t launch_phase_pair(const Ctx& c, int cfg, int mu, int parity, bool plaq, int32_t* dbg,
                               bool hyb, cudaStream_t s)
 {
-    using T = typename std::conditional<ROW == ROW_F64, double, float>::type;
+    static_assert(ROW != ROW_F64, "the FP64 row is in heatbath_fp64.cu");
+    using T = float;
     constexpr bool PAIRS = ROW == ROW_F32_PAIRS;
     constexpr LaunchCfg A = LAUNCH_CFG[ROW][FIRST];
     constexpr LaunchCfg B = LAUNCH_CFG[ROW][FIRST + 1];
     if (cfg == FIRST)
         return launch_phase_shape<T, A.threads, A.min_blocks, A.slab, A.rounds, A.persistent,
-                                  PAIRS, A.group, A.stage>(c, mu, parity, plaq, dbg, hyb, s);
+                                  PAIRS, A.stage>(c, mu, parity, plaq, dbg, hyb, s);
     if (cfg == FIRST + 1)
         return launch_phase_shape<T, B.threads, B.min_blocks, B.slab, B.rounds, B.persistent,
-                                  PAIRS, B.group, B.stage>(c, mu, parity, plaq, dbg, hyb, s);
+                                  PAIRS, B.stage>(c, mu, parity, plaq, dbg, hyb, s);
     return cudaErrorInvalidValue;
 }
 

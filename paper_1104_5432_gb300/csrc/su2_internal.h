@@ -78,6 +78,19 @@ constexpr LaunchCfg LAUNCH_CFG[NUM_ROWS][NUM_LAUNCH_CFG] = {
      {32, 24, true, 4, false}, {32, 16, true, 4, false}},
 };
 static_assert(NUM_LAUNCH_CFG % 2 == 0, "shapes compile in pairs");
+// The kernels the FP64 row's shapes run: one link per thread with 255 or 128
+// registers a thread (the same kernel in blocks of 256, 64 or 32 and of 128,
+// 64 or 32 threads), eight lanes per link, R links per thread with a retry
+// queue, and the same persistent.
+enum FixKind { FIX_LINK_255, FIX_LINK_128, FIX_COOP, FIX_QUEUE, FIX_PERSIST, NUM_FIX_KINDS };
+constexpr FixKind fix_kind(const LaunchCfg& f)
+{
+    return f.group > 1 ? FIX_COOP
+           : f.persistent ? FIX_PERSIST
+           : f.rounds > 1 ? FIX_QUEUE
+           : f.threads * f.min_blocks <= 256 ? FIX_LINK_255
+                                             : FIX_LINK_128;
+}
 // largest y-slab window (sites between a site and its t neighbour, times
 // the bytes a site's update touches) kept in L2
 constexpr double SLAB_WINDOW_BYTES = 8.0 * (1 << 20);
@@ -95,6 +108,7 @@ constexpr int TRIAL_SLOTS = 64;        // per-lattice trial counters (spread ato
 // One per lattice, resident in the work buffer.  The first block is fixed
 // at bind time; the second is written by the parameter kernel at every
 // heat-bath call; the counters are advanced by the kernels.
+struct FixTables;
 struct LatDesc {
     int32_t Ns, Nt, Nh, Vs;
     uint32_t V, Vh;
@@ -107,6 +121,7 @@ struct LatDesc {
     double creutz_below;    // alpha below which Creutz's draw replaces Kennedy-Pendleton's
     float creutz_below_f;
     const double2* fp64_table;  // the FP64 path's log and sin/cos tables (work memory)
+    const FixTables* fix_table; // the fixed-point path's (work memory)
     uint64_t link_off;      // byte offset of this lattice in the link buffer
     uint64_t field_off;     // double offset of its Polyakov field
     // per call
@@ -117,6 +132,7 @@ struct LatDesc {
     uint64_t seed;
     uint64_t sweep_base;    // sweep index stored at plaq_out[0]
     double* plaq_out;       // device, nullable
+    uint32_t nonunit;       // FP64: some link is not a unit quaternion (unit_check_kernel)
     // advanced by the kernels
     uint64_t sweep;         // cumulative sweep counter
     unsigned long long trials, updates, caps;
@@ -176,7 +192,10 @@ cudaError_t launch_set_params(const Ctx& c, const ParamChunk& pc, cudaStream_t s
 // creutz_below (the plain variant never looks at it)
 cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, bool plaq,
                          int32_t* dbg_trials, bool hybrid, cudaStream_t s);
-cudaError_t launch_sweep_end(const Ctx& c, bool plaq, cudaStream_t s);
+cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s);
+// FP64 lattices, after launch_set_params: looks at every link and sets
+// nonunit where | |U|^2 - 1 | > UNIT_TOLERANCE
+cudaError_t launch_unit_check(const Ctx& c, cudaStream_t s);
 
 // the tables of the FP64 path's logarithm and sine/cosine (ln_u01_tab,
 // sincospi_tab, su2_math.cuh: layout TAB_*), filled on the host

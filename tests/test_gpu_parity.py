@@ -1115,3 +1115,36 @@ def test_staged_rows_bit_identical():
         lat.close()
     np.testing.assert_array_equal(tr[9][0], tr[0][0])
     np.testing.assert_array_equal(tr[9][1], tr[0][1])
+
+
+@pytest.mark.parametrize("cfg", [0, 4, 8, 11, 12])
+def test_fp64_lattice_with_non_unit_links(cfg):
+    """Links that are not unit quaternions (scaled by 0.5 .. 1.5, so the
+    fixed-point ranges of the FP64 kernels do not hold) take the FP64
+    sequence: single phases and sweeps against the oracle, and two calls of
+    one sweep equal one call of two, although every link is a unit
+    quaternion after the first sweep."""
+    Ns, Nt, beta, seed = 6, 4, 2.3, 17
+    V = Ns ** 3 * Nt
+    rng = np.random.default_rng(4)
+    links = inputs.random_links(Ns, Nt, 8) * rng.uniform(0.5, 1.5, size=(V, 4, 1))
+    lat = lattice(Ns, Nt, su2.F64)
+    lat.set_launch_config(cfg)
+    lat.set_links(links)
+    trials = torch.full((V,), -2, dtype=torch.int32, device="cuda")
+    lat.heatbath_phase(beta, 1, 1, seed, trials)
+    ref, rt, _ = O.heatbath_phase(Ns, Nt, links, beta, 1, 1, seed, 0)
+    assert np.max(np.abs(lat.get_links() - ref)) <= 1e-12
+    odd = parity_mask(Ns, Nt) == 1
+    np.testing.assert_array_equal(trials.cpu().numpy()[odd], rt[odd, 1])
+    out = []
+    for calls in ((2,), (1, 1)):
+        lat.set_links(links)
+        lat.set_sweep(0)
+        plaq = np.concatenate([lat.heatbath(beta, n, seed)[0] for n in calls])
+        out.append((lat.get_links(), plaq))
+    np.testing.assert_array_equal(out[1][0], out[0][0])
+    np.testing.assert_array_equal(out[1][1], out[0][1])
+    ref, rplaq, _ = O.heatbath(Ns, Nt, links, beta, 2, seed)
+    assert np.max(np.abs(out[0][0] - ref)) <= 1e-12
+    np.testing.assert_allclose(out[0][1], rplaq, rtol=1e-13, atol=0)
