@@ -131,8 +131,8 @@ def peaks():
         return 6800.0, "fallback"
 
 
-PHASE_SOURCES = ("heatbath_kernel.cuh", "heatbath_fixed.cuh", "su2_fixed.cuh", "su2_links.cuh",
-                 "su2_math.cuh", "su2_device.cuh", "su2_internal.h")
+PHASE_SOURCES = ("heatbath_kernel.cuh", "heatbath_fixed.cuh", "su2_fixed.cuh", "su2_mirror.cuh",
+                 "su2_links.cuh", "su2_math.cuh", "su2_device.cuh", "su2_internal.h")
 
 
 def phase_kernel_hash():

@@ -107,7 +107,9 @@ int su2_lattice_volume(const su2_lattice* lat, int l, uint64_t* V);
 /* Bytes of the two device buffers a handle needs.  The link buffer holds
  * 4V links per lattice (16 B each in FP32, 32 B in FP64); the work buffer
  * holds descriptors, reduction partials, the Polyakov field, the
- * plaquette ring and a 32 MiB staging area for host transfers. */
+ * plaquette ring, a 32 MiB staging area for host transfers and, for an
+ * SU2_F64 handle of at most 16 GiB of links, a fixed-point copy of the links
+ * (as large as the links). */
 int su2_memory_requirements(const su2_lattice* lat, size_t* link_bytes, size_t* work_bytes);
 
 /* Device layout of the links: SU2_LAYOUT_PLAIN by default.  An SU2_F32

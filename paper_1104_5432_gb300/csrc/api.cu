@@ -111,7 +111,8 @@ struct su2_lattice {
     size_t link_bytes = 0, work_bytes = 0;
     size_t off_status = 0, off_desc = 0, off_sstart = 0, off_spstart = 0;
     size_t off_plaq = 0, off_obs = 0, off_field = 0, off_ring = 0, off_res = 0, off_stage = 0;
-    size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0, off_fixtab = 0;
+    size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0, off_fixtab = 0, off_mirror = 0;
+    bool mirror = false;            // FP64: the work buffer holds a fixed-point copy of the links
     uint32_t max_chunks = 1;
     size_t res_doubles = 0;
     // bound state
@@ -301,6 +302,8 @@ int layout(su2_lattice* L)
     L->off_stage = take(STAGE_BYTES);
     L->off_fp64tab = take(sizeof(double2) * FP64_TABLE_ENTRIES);
     L->off_fixtab = take(sizeof(FixTables));
+    L->mirror = L->dtype == SU2_F64 && L->link_bytes <= MIRROR_MAX;
+    L->off_mirror = take(L->mirror ? L->link_bytes : 0);
     L->work_bytes = w;
     return SU2_OK;
 }
@@ -419,7 +422,7 @@ int record_sweep(su2_lattice* L, bool plaq, int rmax, cudaStream_t s)
         if (branch && mu == 3) SU2_CUDA(cudaStreamWaitEvent(s, L->join_ev, 0));
         for (int p = 0; p < 2; ++p)
             SU2_CUDA(launch_phase(L->cfg_ctx[L->cfg], L->row, L->cfg, mu, p, plaq, nullptr,
-                                  L->hybrid, s));
+                                  L->hybrid, true, s));
     }
     SU2_CUDA(launch_sweep_end(L->cfg_ctx[L->cfg], L->row == ROW_F64, plaq, s));
     return SU2_OK;
@@ -580,7 +583,7 @@ int heatbath_impl(su2_lattice* L, const double* betas, double beta, int nsweeps,
         const int chunk = (want && !dev_out) ? std::min(PLAQ_RING, nsweeps - done) : nsweeps;
         if (int rc = set_params(L, betas, beta, seeds, seed, dev_out ? plaq : nullptr, nsweeps))
             return rc;
-        if (L->row == ROW_F64) SU2_CUDA(launch_unit_check(L->ctx, L->stream));
+        if (L->row == ROW_F64) SU2_CUDA(launch_unit_check(L->ctx, true, L->stream));
         for (int s = 0; s < chunk; ++s)
             SU2_CUDA(cudaGraphLaunch(g_first && done + s == 0 ? g_first : g, L->stream));
         if (want && !dev_out) {
@@ -972,6 +975,7 @@ int su2_bind_memory(su2_lattice* lat, void* links, size_t link_bytes, void* work
 
     Ctx& c = lat->ctx;
     c.links = links;
+    c.mirror = lat->mirror ? reinterpret_cast<int4*>(w + lat->off_mirror) : nullptr;
     c.desc = reinterpret_cast<LatDesc*>(w + lat->off_desc);
     c.phase_start = reinterpret_cast<const uint32_t*>(w + lat->off_pstart_cfg[0]);
     c.site_start = reinterpret_cast<const uint32_t*>(w + lat->off_sstart);
@@ -1099,9 +1103,9 @@ int su2_heatbath_phase(su2_lattice* lat, double beta, int mu, int parity, uint64
         lat->phase_beta = beta;
         lat->phase_seed = seed;
     }
-    if (f64) SU2_CUDA(launch_unit_check(lat->ctx, lat->stream));
+    if (f64) SU2_CUDA(launch_unit_check(lat->ctx, false, lat->stream));
     SU2_CUDA(launch_phase(lat->cfg_ctx[lat->cfg], lat->row, lat->cfg, mu, parity, false, trials,
-                          lat->hybrid, lat->stream));
+                          lat->hybrid, false, lat->stream));
     return SU2_OK;
 }
 
@@ -1248,6 +1252,7 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen)
         }
     }
     if (int rc = set_params(lat, betas, TUNE_BETA, nullptr, tune_seed, nullptr, 0)) return rc;
+    if (lat->row == ROW_F64) SU2_CUDA(launch_unit_check(lat->ctx, true, s));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     SU2_CUDA(cudaEventCreate(&e0));
     SU2_CUDA(cudaEventCreate(&e1));

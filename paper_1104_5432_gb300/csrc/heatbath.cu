@@ -3,8 +3,8 @@
 // kernel and the dispatch of the phase kernels (heatbath_kernel.cuh,
 // instantiated per pair of launch shapes and precision by
 // heatbath_shapes.cu).
-#include "su2_fixed.cuh"
 #include "su2_internal.h"
+#include "su2_mirror.cuh"
 #include "su2_reduce.cuh"
 
 namespace su2 {
@@ -26,25 +26,31 @@ __device__ __forceinline__ bool unit_link(const double2& lo, const double2& hi)
     return fabsf(a * a + b * b + c * c + d * d - 1.0f) <= (float)UNIT_TOLERANCE;
 }
 // whether the links eo of the eight (mu, parity) planes of an FP64 lattice
-// are unit quaternions
-__device__ __forceinline__ bool unit_links_at(const Ctx& ctx, const LatDesc& D, uint32_t eo)
+// are unit quaternions; mirror: their fixed-point copies are written too
+__device__ __forceinline__ bool unit_links_at(const Ctx& ctx, const LatDesc& D, uint32_t eo, bool mirror)
 {
     const double2* U = reinterpret_cast<const double2*>(static_cast<const char*>(ctx.links) + D.link_off);
     bool ok = true;
 #pragma unroll
-    for (int mp = 0; mp < 8; ++mp)
-        ok = ok && unit_link(U[(size_t)(2 * mp) * D.Vh + eo], U[(size_t)(2 * mp + 1) * D.Vh + eo]);
+    for (int mp = 0; mp < 8; ++mp) {
+        const double2 lo = U[(size_t)(2 * mp) * D.Vh + eo], hi = U[(size_t)(2 * mp + 1) * D.Vh + eo];
+        ok = ok && unit_link(lo, hi);
+        if (mirror) {
+            const FixMirror M(ctx, D);
+            M.store(mp >> 1, mp & 1, eo, {lo.x, lo.y, hi.x, hi.y});
+        }
+    }
     return ok;
 }
 
 // One thread per two sites.  Bound by HBM: one read of the links (64^4: 2.1
-// GB) per call of any number of sweeps.
-__global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx)
+// GB) and one write of their copies per call of any number of sweeps.
+__global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx, bool mirror)
 {
     const int l = lattice_of_block(ctx.site_start, ctx.n, blockIdx.x);
     LatDesc* D = ctx.desc + l;
     const uint32_t eo = (blockIdx.x - first_block(ctx.site_start, l)) * TPB + threadIdx.x;
-    if (eo < D->Vh && !unit_links_at(ctx, *D, eo)) D->nonunit = 1u;
+    if (eo < D->Vh && !unit_links_at(ctx, *D, eo, mirror)) D->nonunit = 1u;
 }
 
 // the same by one block, after a sweep of a lattice that failed the check:
@@ -52,7 +58,8 @@ __global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx)
 __device__ void unit_recheck(const Ctx& ctx, LatDesc* D)
 {
     bool ok = true;
-    for (uint32_t eo = threadIdx.x; eo < D->Vh; eo += TPB) ok = ok && unit_links_at(ctx, *D, eo);
+    for (uint32_t eo = threadIdx.x; eo < D->Vh; eo += TPB)
+        if (!unit_links_at(ctx, *D, eo, ctx.mirror != nullptr)) ok = false;
     if (__syncthreads_and(ok) && threadIdx.x == 0) D->nonunit = 0u;
 }
 
@@ -137,14 +144,15 @@ cudaError_t launch_phase_pair(const Ctx& c, int cfg, int mu, int parity, bool pl
                               bool hyb, cudaStream_t s);
 template <int KIND, bool HYB>
 cudaError_t launch_fix_kind(const Ctx& c, const LaunchCfg& f, int mu, int parity, bool plaq,
-                            int32_t* dbg, cudaStream_t s);
+                            int32_t* dbg, bool mirror, cudaStream_t s);
 
 cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, bool plaq,
-                         int32_t* dbg_trials, bool hybrid, cudaStream_t s)
+                         int32_t* dbg_trials, bool hybrid, bool mirror, cudaStream_t s)
 {
     if (row < 0 || row >= NUM_ROWS || cfg < 0 || cfg >= NUM_LAUNCH_CFG) return cudaErrorInvalidValue;
     if (row == ROW_F64) {
-        using Fn = cudaError_t (*)(const Ctx&, const LaunchCfg&, int, int, bool, int32_t*, cudaStream_t);
+        using Fn = cudaError_t (*)(const Ctx&, const LaunchCfg&, int, int, bool, int32_t*, bool,
+                                   cudaStream_t);
         static_assert(NUM_FIX_KINDS == 5, "one entry per kernel below");
         static const Fn kinds[NUM_FIX_KINDS][2] = {
             {launch_fix_kind<0, false>, launch_fix_kind<0, true>},
@@ -154,7 +162,7 @@ cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, boo
             {launch_fix_kind<4, false>, launch_fix_kind<4, true>},
         };
         const LaunchCfg& f = LAUNCH_CFG[ROW_F64][cfg];
-        return kinds[fix_kind(f)][hybrid](c, f, mu, parity, plaq, dbg_trials, s);
+        return kinds[fix_kind(f)][hybrid](c, f, mu, parity, plaq, dbg_trials, mirror && c.mirror, s);
     }
     using Fn = cudaError_t (*)(const Ctx&, int, int, int, bool, int32_t*, bool, cudaStream_t);
     static_assert(NUM_LAUNCH_CFG == 14 && NUM_ROWS == 3, "one entry per pair of shapes below");
@@ -180,9 +188,9 @@ cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_unit_check(const Ctx& c, cudaStream_t s)
+cudaError_t launch_unit_check(const Ctx& c, bool mirror, cudaStream_t s)
 {
-    unit_check_kernel<<<c.site_blocks, TPB, 0, s>>>(c);
+    unit_check_kernel<<<c.site_blocks, TPB, 0, s>>>(c, mirror && c.mirror);
     return cudaGetLastError();
 }
 

@@ -7,12 +7,13 @@
 // GB300, an IMAD.WIDE or a logic operation for 2, so the FP64 sequence
 // (general_link: ~270 FP64 instructions, 20,600 clocks per warp) was
 // bound by the FP64 unit alone: 1.66 G link updates/s at 64^4, beta = 2.5,
-// whatever the shape.  The integer update issues ~4,080 instructions per
-// 32 links (2,540 on the ALU pipe, 1,330 integer multiply-adds) and runs at
-// 4.97 G/s there (R = 8) and 4.66 G/s at 32^4, beta = 6.0 (one link per
-// thread, from 1.57), bound by the half-rate integer pipes.  All forms call
-// the same functions on integers, so links and trial counts are
-// bit-identical between them.
+// whatever the shape.  The integer update issues ~2,730 instructions per
+// 32 links (1,410 on the half-rate multiply pipe, 72% busy, 1,090 on the ALU
+// pipe) and runs at 7.16 G/s there (R = 8 or 16, 24 blocks a SM; 6.76 with 16)
+// and 6.3 G/s at 32^4, beta = 6.0 (one link per thread, from 1.57); without
+// the fixed-point copy of the links 5.76 and 5.22.  All forms call the same
+// functions on integers, so links and trial counts are bit-identical between
+// them.
 //
 // The fixed-point ranges hold for unit links.  unit_check_kernel looks at
 // every link before the sweeps of a call and sweep_end_kernel again after
@@ -20,63 +21,74 @@
 // FP64 sequence, one link per thread, in the same kernels.
 #pragma once
 #include "heatbath_kernel.cuh"
-#include "su2_fixed.cuh"
+#include "su2_mirror.cuh"
 
 namespace su2 {
 
-__device__ __forceinline__ FQuat fq_link(const Quat<double>& q, bool dag)
-{
-    auto f = [](double x, bool flip) {
-        return fx_link((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x), flip);
-    };
-    return {f(q.a0, false), f(q.a1, dag), f(q.a2, dag), f(q.a3, dag)};
-}
-__device__ __forceinline__ Quat<double> dq_link(const int64_t* U)
-{
-    auto f = [](int64_t v) { return __longlong_as_double((long long)double_bits(v, -60)); };
-    return {f(U[0]), f(U[1]), f(U[2]), f(U[3])};
-}
+// An FP64 lattice's links: neighbours read as limbs, from the fixed-point copy
+// (MIR) or from the doubles; the stored values are doubles.
+template <bool MIR> struct FixLinks;
+template <> struct FixLinks<false> : Links<double> {
+    __device__ __forceinline__ FixLinks(const Ctx& c, const LatDesc& d)
+        : Links<double>(c.links, d, c.status) {}
+    __device__ __forceinline__ FQuat fix(int mu, int p, uint32_t eo) const
+    {
+        return fq_link(load(mu, p, eo));
+    }
+};
+template <> struct FixLinks<true> : Links<double> {
+    FixMirror m;
+    __device__ __forceinline__ FixLinks(const Ctx& c, const LatDesc& d)
+        : Links<double>(c.links, d, c.status), m(c, d) {}
+    __device__ __forceinline__ FQuat fix(int mu, int p, uint32_t eo) const { return m.load(mu, p, eo); }
+    __device__ __forceinline__ void store(int mu, int p, uint32_t eo, const Quat<double>& q) const
+    {
+        Links<double>::store(mu, p, eo, q);
+        m.store(mu, p, eo, q);
+    }
+};
+
 // a stored link at 2^60
 __device__ __forceinline__ void fix_from_link(const Quat<double>& q, int64_t* U)
 {
-    const FQuat f = fq_link(q, false);
+    const FQuat f = fq_link(q);
     const Fx* c[4] = {&f.a0, &f.a1, &f.a2, &f.a3};
 #pragma unroll
     for (int k = 0; k < 4; ++k) U[k] = (((int64_t)c[k]->h << 32) + c[k]->l) >> 1;
 }
 
-// One staple term x y^dagger z^dagger of U_mu(x): the upper (x, y, z) =
-// (U_nu(x+mu), U_mu(x+nu), U_nu(x)), the lower (U_nu(x+mu-nu)^dagger,
-// U_mu(x-nu), U_nu(x-nu)^dagger), added to A.
-__device__ __forceinline__ void fix_term(const Links<double>& U, int mu, int nu, int p, uint32_t i,
-                                         int hpm, int hpn, int hmn, bool lower, int64_t* A)
+// one staple term of U_mu(x) in the plane (nu, mu), added to A (fq_staple)
+template <typename LT>
+__device__ __forceinline__ void fix_term(const LT& U, int mu, int nu, int p, uint32_t i, int hpm,
+                                         int hpn, int hmn, bool lower, int64_t* A)
 {
     const int q = p ^ 1;
-    const Quat<double> x = U.load(nu, lower ? p : q, i + hpm + (lower ? hmn : 0));
-    const Quat<double> y = U.load(mu, q, i + (lower ? hmn : hpn));
-    const Quat<double> z = U.load(nu, lower ? q : p, lower ? i + hmn : i);
-    fq_mul_nd_acc(fq_mul_nd(fq_link(x, lower), fq_link(y, false)), fq_link(z, lower), A);
+    const FQuat x = U.fix(lower ? mu : nu, q, i + (lower ? hmn : hpm));
+    const FQuat y = U.fix(lower ? nu : mu, lower ? p : q, i + (lower ? hpm + hmn : hpn));
+    const FQuat z = U.fix(nu, lower ? q : p, lower ? i + hmn : i);
+    fq_staple(x, y, z, lower, A);
 }
 
-// staple_sum: A, and (PLAQ) its part P over nu < mu.  The six terms are one
+// staple_sum: A, and (PLAQ) its part P over nu < mu.  The three planes are one
 // loop body: the update's code has to fit the instruction caches (fully
 // unrolled and with the draw inlined twice, 43% of the stalls waited for
 // instructions and 64^4 ran at 3.7 G updates/s).
-template <int MU, bool PLAQ>
-__device__ __forceinline__ void fix_staple_sum(const Links<double>& U, const EoSite& s, uint32_t i,
+template <int MU, bool PLAQ, typename LT>
+__device__ __forceinline__ void fix_staple_sum(const LT& U, const EoSite& s, uint32_t i,
                                                int p, int64_t* A, int64_t* P)
 {
     int hp[4], hm[4];
     s.hops(hp, hm);
     A[0] = A[1] = A[2] = A[3] = 0;
 #pragma unroll 1
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < 3; ++k) {
         constexpr int n0 = nu_of<MU>(0), n1 = nu_of<MU>(1), n2 = nu_of<MU>(2);
-        const int nu = k < 2 ? n0 : (k < 4 ? n1 : n2);
-        const int hpn = k < 2 ? hp[n0] : (k < 4 ? hp[n1] : hp[n2]);
-        const int hmn = k < 2 ? hm[n0] : (k < 4 ? hm[n1] : hm[n2]);
-        fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, (k & 1) != 0, A);
-        if (PLAQ && k == 2 * MU - 1) {
+        const int nu = k == 0 ? n0 : (k == 1 ? n1 : n2);
+        const int hpn = k == 0 ? hp[n0] : (k == 1 ? hp[n1] : hp[n2]);
+        const int hmn = k == 0 ? hm[n0] : (k == 1 ? hm[n1] : hm[n2]);
+        fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, false, A);
+        fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, true, A);
+        if (PLAQ && k == MU - 1) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) P[c] = A[c];
         }
@@ -107,9 +119,9 @@ struct FixCall {
 };
 
 // alpha -> 0 limit of the conditional law (rare: kept out of the loops' code)
-static __device__ __noinline__ Quat<double> haar_link(Stream st)
+static __device__ __noinline__ Quat<double> haar_link(Stream st, const FixTables* tab)
 {
-    return haar_from<double>(st.draw(TAG_DIRECTION, 0));
+    return haar_double(st.draw(TAG_DIRECTION, 0), tab);
 }
 
 // The draw's inputs from the staple sum: false for the Haar branch
@@ -224,9 +236,10 @@ __device__ __noinline__ void general_links(const Ctx& ctx, int l, uint32_t blk0,
 // ---------------------------------------------------------------------------
 // one link per thread
 // ---------------------------------------------------------------------------
-// NT, MINB bound the registers (255 or 128 a thread); smaller blocks of
-// the same register count run the same kernel.
-template <int MU, bool PLAQ, bool HYB, int NT, int MINB>
+// NT, MINB bound the registers (255 or 96 a thread: 16^4 runs 95 us a sweep
+// with many registers and 98 with 96, 32^4 674 with 128 and 663 with 96);
+// smaller blocks of the same register count run the same kernel.
+template <int MU, bool PLAQ, bool HYB, bool MIR, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 fix_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
@@ -239,7 +252,7 @@ fix_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, i < Vh ? i + 1 : i, p, HYB, dbg);
         return;
     }
-    const Links<double> U(ctx.links, D, ctx.status);
+    const FixLinks<MIR> U(ctx, D);
     const FixCall C(D);
     int64_t plaq = 0;
     uint32_t ntrial = 0, ncap = 0;
@@ -252,7 +265,7 @@ fix_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         double qc;
         int32_t tr = -1;
         if (!fix_prepare<HYB>(C, A, &d, &qc)) {
-            const Quat<double> h = haar_link(st);
+            const Quat<double> h = haar_link(st, C.tab);
             U.store(MU, p, i, h);
             if (PLAQ) fix_from_link(h, un);
             tr = 0;
@@ -313,8 +326,8 @@ struct FixQueue {
 // R <= FIX_MAX_ROUNDS: the warp's plaquette sum (6 * 2^51 a link, 32 R
 // links) stays below 2^63.
 constexpr int FIX_MAX_ROUNDS = 16;
-template <int MU, bool PLAQ, bool HYB, bool PERSIST>
-__global__ void __launch_bounds__(32, 16)
+template <int MU, bool PLAQ, bool HYB, bool MIR, bool PERSIST>
+__global__ void __launch_bounds__(32, PERSIST ? 16 : 24)
 fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
 {
     static_assert(KP_CAP <= (1 << 13), "trial index must fit 13 bits");
@@ -338,7 +351,7 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
         }
         return;
     }
-    const Links<double> U(ctx.links, D, ctx.status);
+    const FixLinks<MIR> U(ctx, D);
     const FixCall C(D);
     const int lane = threadIdx.x;
     const uint32_t below = (1u << lane) - 1u;
@@ -364,7 +377,7 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
                 key = s.lex() * 4u + MU;
                 pend = fix_prepare<HYB>(C, A, &d, &qc);
                 if (!pend) {
-                    const Quat<double> h = haar_link(C.stream(key));
+                    const Quat<double> h = haar_link(C.stream(key), C.tab);
                     U.store(MU, p, i, h);
                     if (PLAQ) {
                         int64_t un[4];
@@ -465,7 +478,7 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
 // staple terms at once, their integer sums meet in a butterfly (any order
 // gives the same bits), and the eight lanes try eight trials at once; the
 // link takes the first accepted one of its own sequence.
-template <int MU, bool PLAQ, bool HYB>
+template <int MU, bool PLAQ, bool HYB, bool MIR>
 __global__ void __launch_bounds__(64, 8)
 fix_coop_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
@@ -482,7 +495,7 @@ fix_coop_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, act && g == 0 ? i + 1 : i, p, HYB, dbg);
         return;
     }
-    const Links<double> U(ctx.links, D, ctx.status);
+    const FixLinks<MIR> U(ctx, D);
     const FixCall C(D);
 
     int64_t A[4] = {0, 0, 0, 0}, P[4] = {0, 0, 0, 0};
@@ -549,7 +562,7 @@ fix_coop_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     if (act && g == 0) {
         int64_t un[4];
         if (haar) {
-            const Quat<double> h = haar_link(st);
+            const Quat<double> h = haar_link(st, C.tab);
             U.store(MU, p, i, h);
             if (PLAQ) fix_from_link(h, un);
             tr = 0;

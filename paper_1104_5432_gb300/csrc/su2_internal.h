@@ -78,18 +78,18 @@ constexpr LaunchCfg LAUNCH_CFG[NUM_ROWS][NUM_LAUNCH_CFG] = {
      {32, 24, true, 4, false}, {32, 16, true, 4, false}},
 };
 static_assert(NUM_LAUNCH_CFG % 2 == 0, "shapes compile in pairs");
-// The kernels the FP64 row's shapes run: one link per thread with 255 or 128
-// registers a thread (the same kernel in blocks of 256, 64 or 32 and of 128,
+// The kernels the FP64 row's shapes run: one link per thread with up to 255 or
+// 96 registers a thread (the same kernel in blocks of 256, 64 or 32 and of 128,
 // 64 or 32 threads), eight lanes per link, R links per thread with a retry
 // queue, and the same persistent.
-enum FixKind { FIX_LINK_255, FIX_LINK_128, FIX_COOP, FIX_QUEUE, FIX_PERSIST, NUM_FIX_KINDS };
+enum FixKind { FIX_LINK_255, FIX_LINK_96, FIX_COOP, FIX_QUEUE, FIX_PERSIST, NUM_FIX_KINDS };
 constexpr FixKind fix_kind(const LaunchCfg& f)
 {
     return f.group > 1 ? FIX_COOP
            : f.persistent ? FIX_PERSIST
            : f.rounds > 1 ? FIX_QUEUE
            : f.threads * f.min_blocks <= 256 ? FIX_LINK_255
-                                             : FIX_LINK_128;
+                                             : FIX_LINK_96;
 }
 // largest y-slab window (sites between a site and its t neighbour, times
 // the bytes a site's update touches) kept in L2
@@ -141,6 +141,7 @@ struct LatDesc {
 // Everything a kernel needs, passed by value.
 struct Ctx {
     void* links;
+    int4* mirror;                  // FP64: the links in fixed point (nullable), at link_off too
     LatDesc* desc;
     const uint32_t* phase_start;   // [n+1] first block of each lattice, V/2 links
     const uint32_t* site_start;    // [n+1] ... V sites
@@ -190,12 +191,17 @@ struct ParamChunk {
 cudaError_t launch_set_params(const Ctx& c, const ParamChunk& pc, cudaStream_t s);
 // hybrid: compile-time variant with Creutz's draw below each lattice's
 // creutz_below (the plain variant never looks at it)
+// mirror (FP64): the neighbours come from the fixed-point copy of the links
 cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, bool plaq,
-                         int32_t* dbg_trials, bool hybrid, cudaStream_t s);
+                         int32_t* dbg_trials, bool hybrid, bool mirror, cudaStream_t s);
 cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s);
 // FP64 lattices, after launch_set_params: looks at every link and sets
-// nonunit where | |U|^2 - 1 | > UNIT_TOLERANCE
-cudaError_t launch_unit_check(const Ctx& c, cudaStream_t s);
+// nonunit where | |U|^2 - 1 | > UNIT_TOLERANCE; mirror: also writes the
+// fixed-point copy
+cudaError_t launch_unit_check(const Ctx& c, bool mirror, cudaStream_t s);
+// largest link buffer (bytes) an FP64 handle keeps a fixed-point copy of, in
+// its work buffer: above it the copy's memory would matter more than its time
+constexpr size_t MIRROR_MAX = size_t(16) << 30;
 
 // the tables of the FP64 path's logarithm and sine/cosine (ln_u01_tab,
 // sincospi_tab, su2_math.cuh: layout TAB_*), filled on the host

@@ -37,11 +37,7 @@ void update(const Q<double>* L, double beta, const uint32_t* w, F* lam2, bool* o
         Q<F> x[3];
         for (int k = 0; k < 3; ++k)
             for (int c = 0; c < 4; ++c) x[k].c[c] = L[3 * i + k].c[c];
-        if (i & 1) {
-            x[0] = dag(x[0]);
-            x[2] = dag(x[2]);
-        }
-        const Q<F> t = nd(nd(x[0], x[1]), x[2]);
+        const Q<F> t = i & 1 ? nd(dag(nd(x[0], dag(x[1]))), dag(x[2])) : nd(nd(x[0], x[1]), x[2]);
         for (int c = 0; c < 4; ++c) A.c[c] += t.c[c];
     }
     F k = 0;
@@ -75,9 +71,9 @@ int main()
     }
     printf("ln %.3e %.3e\n", e0, e1);
     e0 = e1 = 0;
-    for (uint32_t k = 0; k < (1u << 23); k += 5) {
+    for (uint32_t k = 0; k < (1u << 24); k += 9) {
         const Arc a = arc_at(k, &T);
-        const LD x = 2 * std::acos(-1.0L) * (LD)k / 8388608.0L;
+        const LD x = 2 * std::acos(-1.0L) * (LD)k / 16777216.0L;
         e0 = std::max(e0, err(std::cos(x), std::ldexp((LD)arc_cos(a), -62)));
         e1 = std::max(e1, err(std::sin(x), std::ldexp((LD)arc_sin(a), -62)));
     }
@@ -99,9 +95,9 @@ int main()
         double x = (double)(int64_t)g() * 0x1p-63;
         if (i < 4) x = i == 0 ? 0.0 : (i == 1 ? 1.0 : (i == 2 ? -1.0 : -0x1p-30));
         else if (i % 3 == 0) x = std::ldexp(x, -(int)(g() % 80));
-        const Fx f = fx_link((uint32_t)(bits(x) >> 32), (uint32_t)bits(x), i & 1);
+        const Fx f = fx_link((uint32_t)(bits(x) >> 32), (uint32_t)bits(x));
         const LD v = std::ldexp((LD)f.h, -29) + std::ldexp((LD)f.l, -61);
-        e0 = std::max(e0, err(v, (i & 1) ? -x : x));
+        e0 = std::max(e0, err(v, x));
         const int64_t m = (int64_t)g() >> (3 + g() % 60);
         const LD y = std::ldexp((LD)m, -60);
         const double d = from_bits(double_bits(m, -60));
@@ -109,6 +105,41 @@ int main()
         else if (d != 0) e1 = 1;
     }
     printf("convert %.3e %.3e\n", e0, e1);
+    // Haar elements: Box-Muller and normalisation in long double and in doubles
+    double h0 = 0, h1 = 0, s0 = 0, s1 = 0;
+    for (int i = 0; i < 400000; ++i) {
+        uint32_t w[4];
+        for (uint32_t& x : w) x = (uint32_t)g();
+        if (i % 4 == 1) w[0] |= 0xFFFFFFFFu << (9 + g() % 20);  // u0 near 1
+        if (i % 4 == 2) w[0] >>= g() % 24;                      // u0 near 0
+        if (i % 8 == 3) w[0] |= 0xFFFF0000u, w[2] |= 0xFFFFF000u;
+        int64_t U[4];
+        haar_fix(w[0], w[1], w[2], w[3], &T, U);
+        auto haar = [&](auto one) {
+            using F = decltype(one);
+            Q<F> q;
+            F n = 0;
+            for (int k = 0; k < 2; ++k) {
+                const F r = std::sqrt(-2 * std::log(((F)(w[2 * k] >> 9) + (F)0.5) / 8388608));
+                const F x = 2 * std::acos((F)-1) * (((F)(w[2 * k + 1] >> 9) + (F)0.5) / 8388608);
+                q.c[2 * k] = r * std::cos(x);
+                q.c[2 * k + 1] = r * std::sin(x);
+            }
+            for (F c : q.c) n += c * c;
+            for (F& c : q.c) c /= std::sqrt(n);
+            return q;
+        };
+        const Q<LD> ref = haar((LD)1);
+        const Q<double> dbl = haar(1.0);
+        for (int c = 0; c < 4; ++c) {
+            const double f = err(from_bits(double_bits(U[c], -60)), ref.c[c]), d = err(dbl.c[c], ref.c[c]);
+            h0 = std::max(h0, f);
+            h1 = std::max(h1, d);
+            s0 += f * f;
+            s1 += d * d;
+        }
+    }
+    printf("haar %.3e %.3e %.3e %.3e\n", h0, h1, std::sqrt(s0), std::sqrt(s1));
     const double betas[] = {0.1, 0.7, 2.3, 6.0, 50.0, 1e5};
     for (double beta : betas)
         for (double spread : {0.0, 0.3, -1.0}) {  // -1: random links
@@ -140,15 +171,13 @@ int main()
                 update<double>(L, beta, w, &lamd, &okd, &Ud);
                 int64_t A[4] = {0, 0, 0, 0};
                 for (int i = 0; i < 6; ++i) {
-                    auto conv = [&](const Q<double>& q, bool d) {
+                    auto conv = [&](const Q<double>& q) {
                         auto f = [&](int c) {
-                            return fx_link((uint32_t)(bits(q.c[c]) >> 32), (uint32_t)bits(q.c[c]),
-                                           d && c > 0);
+                            return fx_link((uint32_t)(bits(q.c[c]) >> 32), (uint32_t)bits(q.c[c]));
                         };
                         return FQuat{f(0), f(1), f(2), f(3)};
                     };
-                    fq_mul_nd_acc(fq_mul_nd(conv(L[3 * i], i & 1), conv(L[3 * i + 1], false)),
-                                  conv(L[3 * i + 2], i & 1), A);
+                    fq_staple(conv(L[3 * i]), conv(L[3 * i + 1]), conv(L[3 * i + 2]), i & 1, A);
                 }
                 Drawn D;
                 uint64_t K;

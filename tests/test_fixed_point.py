@@ -35,6 +35,8 @@ def test_functions(lines):
     # a link component to one unit of 2^-61, a double to half a unit in its
     # last place (the lines carry four digits)
     assert got["convert"][0] <= 1.001 * 2.0 ** -61 and got["convert"][1] <= 1.001 * 2.0 ** -53
+    worst, worst_d, rms, rms_d = got["haar"]
+    assert worst <= worst_d and rms <= 0.5 * rms_d
 
 
 def test_new_links_are_no_further_off_than_in_doubles(lines):
