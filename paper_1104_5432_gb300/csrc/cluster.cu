@@ -47,6 +47,7 @@ struct ClusterLinks {
 // every shared-memory write before it with every read after it
 __device__ __forceinline__ void cluster_sync()
 {
+    __syncwarp();  // .aligned: the warp arrives together
     asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -183,6 +184,359 @@ hb_cluster_kernel(Ctx ctx, uint32_t C, FastDiv div_c, int pl)
         }
         Dw->sweep = sw + 1;
     }
+}
+
+// ---------------------------------------------------------------------------
+// all sweeps of a call in one launch, draws computed ahead
+// ---------------------------------------------------------------------------
+// The chain kernel runs every sweep of a call on a lattice whose share per CTA
+// is at most 512 links of each (mu, parity).  A phase of a small lattice lasts
+// as long as one link's chain of instructions, so the chain is cut:
+//   * half the threads (the updaters, one link each) form the staple, decide
+//     and store; the other half (the drawers) compute the next phase's first
+//     trials in the meantime -- Philox, both logarithms, the cosine, the
+//     direction, everything that does not depend on the links -- and leave
+//     them in shared memory;
+//   * the shared-memory addresses of a link's 20 neighbour sites of either
+//     parity are computed once per launch (a neighbour of another CTA is one
+//     mapa away) and read from a table;
+//   * the cluster barrier between the phases is the only synchronisation.
+// The FP32 operations are those of staple_sum and draw_link, in their order, so
+// the links are the other kernels' bit by bit.  C is a multiple of 32: the
+// warps hold the same 32 links as launch shape 0's, and the plaquette
+// partials are summed in that shape's order (sweep_end_kernel's), so its
+// plaquettes are reproduced bit by bit too.
+// Measured per sweep with the plaquette (beta = 2.4): 8^4 13.0 us (28.7 in
+// launch shape 0's phase launches, 22.6 in the whole-sweep kernel above),
+// 10^3 x 6 15.1 (28.7), 12^3 x 8 24.7 (28.9); 4^4 10.0, i.e. 1.2 us a phase
+// whatever the size: one update's remaining chain and the barrier.
+struct ChainShared {
+    float4* own;       // [8][C] links
+    float4* tdir;      // [2][C] (t, r4^2, cos theta, sin theta) of the coming phase
+    float2* phi;       // [2][C] (sin phi, cos phi)
+    uint32_t* addr;    // [2][20][C] site addresses: plus 0..3, minus 4..7, 8 + 3 mu + k:
+                       // x + mu - nu, nu the k-th direction other than mu
+    double* part;      // CTA 0: [2][3 npart] plaquette partials
+    __device__ __forceinline__ ChainShared(char* base, uint32_t C)
+        : own(reinterpret_cast<float4*>(base)), tdir(own + 8 * C),
+          phi(reinterpret_cast<float2*>(tdir + 2 * C)), addr(reinterpret_cast<uint32_t*>(phi + 2 * C)),
+          part(reinterpret_cast<double*>(addr + 40 * C))
+    {
+    }
+};
+constexpr size_t chain_smem(uint32_t C, uint32_t npart)
+{
+    return (size_t)C * (8 * 16 + 2 * 16 + 2 * 8 + 40 * 4) + 2 * 3 * (size_t)npart * 8;
+}
+
+__device__ __forceinline__ Quat<float> ld_cluster(uint32_t a)
+{
+    float4 v;
+    // volatile: never moved across the cluster barriers
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a));
+    return {v.x, v.y, v.z, v.w};
+}
+
+// The first trial of a link as far as it goes without the staple.
+__device__ __forceinline__ void draw_ahead(const Stream& st, float4* tdir, float2* phi)
+{
+    const U4 w = st.draw(TAG_TRIAL, 0u);
+    // kp_eval: lambda^2 = t / (2 alpha), accepted iff r4^2 <= 1 - lambda^2
+    const float t = neg_(fma_(Math<float>::cos2pi_sq(u01<float>(w.y)), Math<float>::ln_u01(u01<float>(w.z)),
+                              Math<float>::ln_u01(u01<float>(w.x))));
+    const float r4 = u01<float>(w.w);
+    // new_link_u, new_link_dir: the direction
+    const float cth = fma_(2.0f, u18<float>(spare_bits_1(w)), -1.0f);
+    const float sth = Math<float>::sqrt_pos(mul_(add_(1.0f, neg_(cth)), add_(1.0f, cth)));
+    float sph, cph;
+    Math<float>::sincos2pi(u18<float>(spare_bits_2(w)), &sph, &cph);
+    *tdir = make_float4(t, mul_(r4, r4), cth, sth);
+    *phi = make_float2(sph, cph);
+}
+
+// phase (MU, p) on this thread's link o
+template <int MU>
+__device__ __forceinline__ void chain_phase(const ChainShared& sh, const LatDesc& D, uint32_t C,
+                                            uint32_t o, int p, uint32_t key, uint64_t sw,
+                                            const float4& td, const float2& ph, Quat<float>& P,
+                                            Quat<float>& un, uint32_t& ntrial, uint32_t& ncap)
+{
+    const int q = p ^ 1;
+    const uint32_t* ad = sh.addr + (size_t)p * 20 * C + o;
+    const uint32_t plane = C * 16;  // bytes from one (mu, parity) to the next
+    const uint32_t e_pmu = ad[MU * C];
+    Quat<float> A = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int nu = nu_of<MU>(k);
+        const uint32_t e_pnu = ad[nu * C], e_mnu = ad[(4 + nu) * C];
+        const uint32_t e_pmu_mnu = ad[(8 + 3 * MU + k) * C];
+        const float4 cc = sh.own[(nu * 2 + p) * C + o];
+        const Quat<float> a = ld_cluster(e_pmu + (nu * 2 + q) * plane);      // U_nu(x+mu)
+        const Quat<float> b = ld_cluster(e_pnu + (MU * 2 + q) * plane);      // U_mu(x+nu)
+        const Quat<float> c = {cc.x, cc.y, cc.z, cc.w};                      // U_nu(x)
+        const Quat<float> d = ld_cluster(e_pmu_mnu + (nu * 2 + p) * plane);  // U_nu(x+mu-nu)
+        const Quat<float> e = ld_cluster(e_mnu + (MU * 2 + q) * plane);      // U_mu(x-nu)
+        const Quat<float> f = ld_cluster(e_mnu + (nu * 2 + q) * plane);      // U_nu(x-nu)
+        A = qmul_dn_acc(qmul(e, d), f, qmul_nd_acc(qmul_nd(a, b), c, A));
+        if (nu == MU - 1) P = A;
+    }
+    // draw_link on the values drawn ahead
+    const float k2 = qnorm2(A);
+    const float rk = Math<float>::rsqrt(k2);
+    const float alpha = mul_(mul_(D.beta_f, k2), rk);
+    const Stream st{(uint32_t)D.seed, (uint32_t)(D.seed >> 32), key, (uint32_t)sw, (uint32_t)(sw >> 32)};
+    float4& slot = sh.own[(MU * 2 + p) * C + o];
+    if (!(alpha >= alpha_haar<float>())) {
+        un = haar_from<float>(st.draw(TAG_DIRECTION, 0));
+        slot = make_float4(un.a0, un.a1, un.a2, un.a3);
+        return;
+    }
+    const float inv2a = mul_(rk, D.half_inv_beta_f);
+    const float lam2 = mul_(td.x, inv2a);
+    float delta = add_(lam2, lam2);
+    uint32_t tr = 1;
+    if (!(td.y <= add_(1.0f, neg_(lam2)))) {
+        tr = 0;
+        for (uint32_t t = 1; t < (uint32_t)KP_CAP; ++t) {
+            if (kp_try(st.draw(TAG_TRIAL, t), inv2a, &delta)) {
+                tr = t + 1;
+                break;
+            }
+        }
+    }
+    if (tr == 0) {  // cap hit: the link keeps its value
+        un = {slot.x, slot.y, slot.z, slot.w};
+        ncap += 1;
+        ntrial += (uint32_t)KP_CAP;
+        return;
+    }
+    ntrial += tr;
+    const float vl = Math<float>::sqrt_pos(mul_(delta, add_(2.0f, neg_(delta))));
+    const float vs = mul_(vl, td.w);
+    const Quat<float> X = {add_(1.0f, neg_(delta)), mul_(vs, ph.y), mul_(vs, ph.x), mul_(vl, td.z)};
+    un = qnormalise(qmul_nd(X, A));
+    slot = make_float4(un.a0, un.a1, un.a2, un.a3);
+}
+
+// nsweeps sweeps of a single-lattice handle.  Grid: one cluster of CTAs of NU
+// updaters and NU drawers (NU >= C); npart: launch shape 0's warps per phase.
+template <int NU>
+__global__ void __launch_bounds__(2 * NU, 1)
+hb_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int nsweeps)
+{
+    extern __shared__ float4 chain_mem[];
+    __shared__ double scratch[8];
+    LatDesc* const Dw = ctx.desc;
+    const LatDesc D = *Dw;  // a register copy (the barriers clobber memory)
+    const ChainShared sh(reinterpret_cast<char*>(chain_mem), C);
+    const uint32_t rank = cluster_rank(), Vh = D.Vh;
+    const bool updater = threadIdx.x < NU;
+    const uint32_t o = updater ? threadIdx.x : threadIdx.x - NU;
+    const uint32_t i = rank * C + o;
+    const bool act = o < C && i < Vh;
+    const int lane = threadIdx.x & 31, w = (int)(o >> 5);
+    const uint64_t sw0 = D.sweep;
+    float4* const glob = reinterpret_cast<float4*>(static_cast<char*>(ctx.links) + D.link_off);
+    LinkCheck chk;
+#ifdef SU2_CHECK_BOUNDS
+    chk = {ctx.status, Vh};
+#endif
+
+    // the links; each half of the threads fills one parity's address table
+    if (act && updater)
+        for (int mp = 0; mp < 8; ++mp) sh.own[mp * C + o] = glob[(size_t)mp * Vh + i];
+    uint32_t lex[2] = {0, 0};
+    if (act) {
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(sh.own);
+        lex[0] = EoSite(D, i, 0).lex();
+        lex[1] = EoSite(D, i, 1).lex();
+        const int p = updater ? 0 : 1;
+        const EoSite s(D, i, p);
+        int hp[4], hm[4];
+        s.hops(hp, hm);
+        uint32_t* ad = sh.addr + (size_t)p * 20 * C + o;
+        auto put = [&](int slot, uint32_t e) {
+            if (!chk.ok(0, 0, e)) e = 0;
+            const uint32_t r = fdiv(e, div_c);
+            uint32_t ra;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(base + ((e - r * C) << 4)), "r"(r));
+            ad[slot * C] = ra;
+        };
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            put(m, i + hp[m]);
+            put(4 + m, i + hm[m]);
+            for (int k = 0; k < 3; ++k) put(8 + 3 * m + k, i + hp[m] + hm[k + (k >= m ? 1 : 0)]);
+        }
+    }
+    if (pl && rank == 0)
+        for (uint32_t k = threadIdx.x; k < 2 * 3 * npart; k += 2 * NU) sh.part[k] = 0.0;
+    auto stream = [&](int mu, int p, uint64_t sw) {
+        return Stream{(uint32_t)D.seed, (uint32_t)(D.seed >> 32), lex[p] * 4u + (uint32_t)mu,
+                      (uint32_t)sw, (uint32_t)(sw >> 32)};
+    };
+    if (act && !updater) draw_ahead(stream(0, 0, sw0), sh.tdir + o, sh.phi + o);
+    cluster_sync();
+
+    uint32_t ntrial = 0, ncap = 0;
+    // sweep_end_kernel's sum of the partials of sweep k on CTA 0, in two steps a
+    // barrier apart (256 virtual threads, then eight warp sums in order)
+    auto sum_warps = [&](int k) {
+        const double* part = sh.part + (size_t)(k & 1) * 3 * npart;
+        for (int vw = w; vw < 8; vw += NU / 32) {
+            double acc = 0.0;
+            for (uint32_t e = vw * 32 + lane; e < 3 * npart; e += 256) acc += part[e];
+            acc = warp_sum(acc);
+            if (lane == 0) scratch[vw] = acc;
+        }
+    };
+    auto finish_sum = [&](int k) {
+        double tot = 0.0;
+        for (int vw = 0; vw < 8; ++vw) tot += scratch[vw];
+        const double P = tot / (6.0 * (double)D.V);
+        const uint64_t at = sw0 + (uint64_t)k - D.sweep_base;
+        ctx.ring[at % PLAQ_RING] = P;
+        if (D.plaq_out) D.plaq_out[at] = P;
+    };
+    for (int k = 0; k < nsweeps; ++k) {
+        const uint64_t sw = sw0 + (uint64_t)k;
+#pragma unroll 1
+        for (int ph8 = 0; ph8 < 8; ++ph8) {
+            const int mu = ph8 >> 1, p = ph8 & 1;
+            if (updater) {
+                Quat<float> P = {0.f, 0.f, 0.f, 0.f}, un = P;
+                if (act) {
+                    const float4 td = sh.tdir[p * C + o];
+                    const float2 ph = sh.phi[p * C + o];
+                    const uint32_t key = lex[p] * 4u + (uint32_t)mu;
+                    switch (mu) {
+                    case 0: chain_phase<0>(sh, D, C, o, p, key, sw, td, ph, P, un, ntrial, ncap); break;
+                    case 1: chain_phase<1>(sh, D, C, o, p, key, sw, td, ph, P, un, ntrial, ncap); break;
+                    case 2: chain_phase<2>(sh, D, C, o, p, key, sw, td, ph, P, un, ntrial, ncap); break;
+                    default: chain_phase<3>(sh, D, C, o, p, key, sw, td, ph, P, un, ntrial, ncap); break;
+                    }
+                }
+                if (pl && p == 1 && mu >= 1) {
+                    const float wp = warp_sum_t(act ? qretr(un, P) : 0.0f);
+                    const uint32_t gw = rank * (C >> 5) + (uint32_t)w;
+                    if (lane == 0 && gw < npart && o < C) {
+                        const uint32_t a = (uint32_t)__cvta_generic_to_shared(
+                            sh.part + (size_t)((k & 1) * 3 + mu - 1) * npart + gw);
+                        uint32_t ra;
+                        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(0u));
+                        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"((double)wp)
+                                     : "memory");
+                    }
+                }
+            } else {
+                if (act && !(ph8 == 7 && k + 1 == nsweeps)) {
+                    const int np = p ^ 1, nmu = (mu + p) & 3;
+                    draw_ahead(stream(nmu, np, ph8 == 7 ? sw + 1 : sw), sh.tdir + np * C + o,
+                               sh.phi + np * C + o);
+                }
+                if (pl && rank == 0 && k > 0) {
+                    if (ph8 == 0) sum_warps(k - 1);
+                    else if (ph8 == 1 && threadIdx.x == NU) finish_sum(k - 1);
+                }
+            }
+            cluster_sync();
+        }
+    }
+
+    // links back to global memory (no remote accesses after the last barrier)
+    if (act && updater)
+        for (int mp = 0; mp < 8; ++mp) glob[(size_t)mp * Vh + i] = sh.own[mp * C + o];
+    if (updater) {
+        const uint32_t wt = __reduce_add_sync(0xffffffffu, ntrial);
+        const uint32_t wc = __reduce_add_sync(0xffffffffu, ncap);
+        if (lane == 0) {
+            const uint32_t gw = rank * (NU / 32) + (uint32_t)w;
+            atomicAdd(ctx.trial_slots + (gw % TRIAL_SLOTS), (unsigned long long)wt);
+            if (wc) {
+                atomicAdd(&Dw->caps, (unsigned long long)wc);
+                atomicOr(ctx.status, STATUS_CAP_HIT);
+            }
+        }
+    }
+    if (rank == 0) {
+        if (pl) {
+            if (!updater) sum_warps(nsweeps - 1);
+            __syncthreads();
+        }
+        if (threadIdx.x == NU) {
+            if (pl) finish_sum(nsweeps - 1);
+            atomicAdd(&Dw->updates, 8ull * (unsigned long long)Vh * (unsigned long long)nsweeps);
+            Dw->sweep = sw0 + (uint64_t)nsweeps;
+        }
+    }
+}
+
+bool chain_geometry(uint32_t Vh, int S, ChainGeom* g)
+{
+    const uint32_t C = ((Vh + (uint32_t)S - 1) / (uint32_t)S + 31) & ~31u;
+    if (C > 512) return false;
+    g->S = S;
+    g->C = C;
+    g->div_c = make_fastdiv(C);
+    g->updaters = C <= 128 ? 128 : (C <= 256 ? 256 : 512);
+    g->npart = (Vh + 255) / 256 * 8;  // launch shape 0: blocks of 256 threads
+    g->smem = chain_smem(C, g->npart);
+    return 3 * g->npart <= (uint32_t)SWEEP_CHUNK;
+}
+
+static void* chain_kernel(const ChainGeom& g)
+{
+    return g.updaters == 128   ? (void*)hb_chain_kernel<128>
+           : g.updaters == 256 ? (void*)hb_chain_kernel<256>
+                               : (void*)hb_chain_kernel<512>;
+}
+static cudaError_t chain_config(const ChainGeom& g, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at)
+{
+    void* k = chain_kernel(g);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3((unsigned)g.S);
+    cfg->blockDim = dim3((unsigned)(2 * g.updaters));
+    cfg->dynamicSmemBytes = g.smem;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)g.S;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+    return e;
+}
+
+bool chain_launchable(const ChainGeom& g)
+{
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    int n = 0;
+    if (chain_config(g, &cfg, at) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, chain_kernel(g), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n >= 1;
+}
+
+cudaError_t launch_chain(const Ctx& c, const ChainGeom& g, bool plaq, int nsweeps, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    if (cudaError_t e = chain_config(g, &cfg, at)) return e;
+    cfg.stream = s;
+    const int pl = plaq ? 1 : 0;
+    if (g.updaters == 128)
+        return cudaLaunchKernelEx(&cfg, hb_chain_kernel<128>, c, g.C, g.div_c, g.npart, pl, nsweeps);
+    if (g.updaters == 256)
+        return cudaLaunchKernelEx(&cfg, hb_chain_kernel<256>, c, g.C, g.div_c, g.npart, pl, nsweeps);
+    return cudaLaunchKernelEx(&cfg, hb_chain_kernel<512>, c, g.C, g.div_c, g.npart, pl, nsweeps);
 }
 
 // cluster size and shared memory for lattice 0, or false when the lattice

@@ -222,6 +222,19 @@ bool cluster_geometry(uint32_t Vh, int dtype_f32, int n, ClusterGeom* g);
 bool cluster_launchable(const ClusterGeom& g);
 cudaError_t launch_cluster_sweep(const Ctx& c, const ClusterGeom& g, bool plaq, bool hyb,
                                  cudaStream_t s);
+// All sweeps of a call on a small single FP32 lattice in one launch of one
+// cluster (cluster.cu, hb_chain_kernel).
+struct ChainGeom {
+    int S = 0;           // CTAs in the cluster
+    uint32_t C = 0;      // links per (mu, parity) per CTA, a multiple of 32
+    FastDiv div_c{};
+    int updaters = 0;    // threads per CTA that update links (as many draw ahead)
+    uint32_t npart = 0;  // plaquette partials per odd phase (launch shape 0's warps)
+    size_t smem = 0;
+};
+bool chain_geometry(uint32_t Vh, int S, ChainGeom* g);
+bool chain_launchable(const ChainGeom& g);
+cudaError_t launch_chain(const Ctx& c, const ChainGeom& g, bool plaq, int nsweeps, cudaStream_t s);
 cudaError_t launch_init(const Ctx& c, int dtype, int l, uint32_t V, int hot, uint64_t seed,
                         cudaStream_t s);
 // canonical values in double (cdtype 1) or float (cdtype 0); pairs_whole:

@@ -1148,3 +1148,36 @@ def test_fp64_lattice_with_non_unit_links(cfg):
     ref, rplaq, _ = O.heatbath(Ns, Nt, links, beta, 2, seed)
     assert np.max(np.abs(out[0][0] - ref)) <= 1e-12
     np.testing.assert_allclose(out[0][1], rplaq, rtol=1e-13, atol=0)
+
+
+@pytest.mark.parametrize("Ns,Nt", [(2, 2), (4, 4), (10, 6), (8, 8), (6, 10), (8, 18), (16, 4),
+                                   (16, 6)])
+def test_one_launch_chain_matches_the_phase_launches(Ns, Nt):
+    """Launch shape 0 on a single small FP32 lattice runs all sweeps of a call
+    in one cluster launch (up to 16384 sites: 2^4 with one part-filled warp
+    and 15 idle CTAs, 10^3 x 6 with an uneven last CTA, 8^3 x 18 just over 256
+    links a CTA, 16^3 x 4 the largest, 16^3 x 6 beyond): links, plaquettes,
+    trial statistics and sweep counter equal, bit by bit, those of the same
+    lattice in a batch, whose sweeps are phase launches -- with host and
+    device plaquettes, without, at a coupling with many rejected trials, in
+    calls of different lengths, and across a trial-cap hit."""
+    lat = lattice(Ns, Nt, su2.F32)
+    B = su2.Lattice([Ns, 4], [Nt, 2], su2.F32)
+    lat.init(su2.HOT, 31)
+    B.batch_init(su2.HOT, [31, 32])
+    dev = torch.zeros(2, dtype=torch.float64, device="cuda")
+    for beta, n, plaq in ((2.4, 3, True), (0.7, 2, dev), (6.0, 1, None), (2.4, 4, True)):
+        p = lat.heatbath(beta, n, 41, plaq=plaq)
+        pb = B.batch_heatbath([beta, 2.0], n, [41, 42], plaq=True)
+        if plaq is dev:
+            p = dev.cpu().numpy()[None]
+        if plaq is not None:
+            np.testing.assert_array_equal(p[0], pb[0])
+        np.testing.assert_array_equal(lat.get_links(), B.get_links(0))
+        assert lat.stats() == B.stats(0) and lat.get_sweep() == B.get_sweep(0)
+    if Ns == 2:
+        before = lat.get_links()
+        with pytest.raises(su2.SU2Error) as e:
+            lat.heatbath(1e-9, 1, 3)
+        assert e.value.code == su2.SU2_E_TRIALS
+        np.testing.assert_array_equal(lat.get_links(), before)
