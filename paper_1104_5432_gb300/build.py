@@ -19,7 +19,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsu2gb300.so")
 SOURCES = ["heatbath.cu", "observables.cu", "links.cu", "api.cu", "plaquette_static.cu",
-           "selftest.cu", "cluster.cu"]
+           "selftest.cu", "cluster.cu", "cluster64.cu"]
 # heatbath_shapes.cu once per pair of launch shapes of the FP32 rows of the
 # 14-entry table in csrc/su2_internal.h (FP32, FP32 site pairs), heatbath_fp64.cu
 # once per kernel and sampler of the FP64 row: (object name, defines, flags);

@@ -543,21 +543,30 @@ bool cluster_available(su2_lattice* L)
 // The geometry of the one-launch chain when the handle's sweeps run in it
 // (without measurements, Kennedy-Pendleton only), or null.  Launch shape 0 takes
 // it on lattices of at most CHAIN0_MAX_SITES sites (the most that fit: 512
-// links of a phase on each of 16 SMs), where it is the faster (12^3 x 8: 24.7
-// us a sweep against 28.9; 8^4: 13.0 against 28.7) and gives the same links
+// links of a phase on each of 16 SMs), where it is the faster (12^3 x 8: 23.1
+// us a sweep against 28.9; 8^4: 12.2 against 28.7) and gives the same links
 // and plaquettes bit by bit.
-constexpr uint64_t CHAIN0_MAX_SITES = 16384;
+// FP64: at most 4096 sites (128 links of a phase on each SM).
+constexpr uint64_t CHAIN0_MAX_SITES = 16384, CHAIN0_MAX_SITES_F64 = 4096;
 const ChainGeom* chain_of(su2_lattice* L)
 {
-    if (L->hybrid || L->row != ROW_F32 || L->n != 1) return nullptr;
+    if (L->hybrid || L->row == ROW_F32_PAIRS || L->n != 1) return nullptr;
     if (L->cluster) return L->cluster_chain ? &L->chain_geom : nullptr;
-    if (L->cfg != 0 || L->V[0] > CHAIN0_MAX_SITES) return nullptr;
+    const bool f64 = L->row == ROW_F64;
+    if (L->cfg != 0 || L->V[0] > (f64 ? CHAIN0_MAX_SITES_F64 : CHAIN0_MAX_SITES)) return nullptr;
     if (L->chain0_ok < 0) {
         DeviceGuard dg(L->device);
-        L->chain0_ok = chain_geometry((uint32_t)(L->V[0] / 2), CLUSTER_MAX, &L->chain0_geom) &&
-                       chain_launchable(L->chain0_geom);
+        const uint32_t Vh = (uint32_t)(L->V[0] / 2);
+        ChainGeom& g = L->chain0_geom;
+        L->chain0_ok = f64 ? chain64_geometry(Vh, &g) && chain64_launchable(g)
+                           : chain_geometry(Vh, CLUSTER_MAX, &g) && chain_launchable(g);
     }
     return L->chain0_ok ? &L->chain0_geom : nullptr;
+}
+cudaError_t run_chain(su2_lattice* L, const ChainGeom& g, bool plaq, int nsweeps)
+{
+    return L->row == ROW_F64 ? launch_chain64(L->ctx, g, plaq, nsweeps, L->stream)
+                             : launch_chain(L->ctx, g, plaq, nsweeps, L->stream);
 }
 
 // select launch index cfg (0 .. NUM_LAUNCH_CFG - 1, or CFG_CLUSTER)
@@ -613,10 +622,10 @@ int heatbath_impl(su2_lattice* L, const double* betas, double beta, int nsweeps,
         const int chunk = (want && !dev_out) ? std::min(PLAQ_RING, nsweeps - done) : nsweeps;
         if (int rc = set_params(L, betas, beta, seeds, seed, dev_out ? plaq : nullptr, nsweeps))
             return rc;
-        if (L->row == ROW_F64) SU2_CUDA(launch_unit_check(L->ctx, true, L->stream));
+        if (L->row == ROW_F64) SU2_CUDA(launch_unit_check(L->ctx, !chain, L->stream));
         if (chain) {
             for (int s = 0; s < chunk; s += PLAQ_RING)
-                SU2_CUDA(launch_chain(L->ctx, *chain, want, std::min(PLAQ_RING, chunk - s), L->stream));
+                SU2_CUDA(run_chain(L, *chain, want, std::min(PLAQ_RING, chunk - s)));
         } else {
             for (int s = 0; s < chunk; ++s)
                 SU2_CUDA(cudaGraphLaunch(g_first && done + s == 0 ? g_first : g, L->stream));
@@ -1307,7 +1316,7 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen)
         if (!chain)
             if (int r = sweep_graph(lat, true, -1, &g)) return r;
         cudaError_t e = cudaEventRecord(e0, s);
-        if (chain && e == cudaSuccess) e = launch_chain(lat->ctx, *chain, true, n, s);
+        if (chain && e == cudaSuccess) e = run_chain(lat, *chain, true, n);
         for (int i = 0; i < n && !chain && e == cudaSuccess; ++i) e = cudaGraphLaunch(g, s);
         if (e == cudaSuccess) e = cudaEventRecord(e1, s);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);

@@ -17,6 +17,7 @@
 // eo in [r C, (r + 1) C), C = Vh / S, as float4s at shared-memory offset
 // (mu 2 + parity) C + (eo - r C).  A neighbour link of another CTA is read
 // with mapa + ld.shared::cluster; a CTA writes only its own links.
+#include "cluster.cuh"
 #include "heatbath_kernel.cuh"
 
 namespace su2 {
@@ -42,22 +43,6 @@ struct ClusterLinks {
         return {v.x, v.y, v.z, v.w};
     }
 };
-
-// all threads of all CTAs of the cluster; the release/acquire pair orders
-// every shared-memory write before it with every read after it
-__device__ __forceinline__ void cluster_sync()
-{
-    __syncwarp();  // .aligned: the warp arrives together
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
-                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
 
 // One phase (MU, p) on this CTA's links: thread t updates eo = r C + t,
 // r C + t + NT, ...; the plaquette part of the staple (PLAQ) goes into the
@@ -206,27 +191,31 @@ hb_cluster_kernel(Ctx ctx, uint32_t C, FastDiv div_c, int pl)
 // warps hold the same 32 links as launch shape 0's, and the plaquette
 // partials are summed in that shape's order (sweep_end_kernel's), so its
 // plaquettes are reproduced bit by bit too.
-// Measured per sweep with the plaquette (beta = 2.4): 8^4 13.0 us (28.7 in
+// Measured per sweep with the plaquette (beta = 2.4): 8^4 12.2 us (28.7 in
 // launch shape 0's phase launches, 22.6 in the whole-sweep kernel above),
-// 10^3 x 6 15.1 (28.7), 12^3 x 8 24.7 (28.9); 4^4 10.0, i.e. 1.2 us a phase
-// whatever the size: one update's remaining chain and the barrier.
+// 10^3 x 6 13.8 (28.7), 12^3 x 8 23.1 (28.8); 4^4 9.5, i.e. 1.2 us a phase
+// whatever the size: one update's remaining chain and the barrier.  (With only
+// the first trial drawn ahead 8^4 took 13.0: some link rejects it in every
+// phase, and all wait.)
 struct ChainShared {
     float4* own;       // [8][C] links
     float4* tdir;      // [2][C] (t, r4^2, cos theta, sin theta) of the coming phase
     float2* phi;       // [2][C] (sin phi, cos phi)
+    float2* second;    // [2][C] (t, r4^2) of the second trial
     uint32_t* addr;    // [2][20][C] site addresses: plus 0..3, minus 4..7, 8 + 3 mu + k:
                        // x + mu - nu, nu the k-th direction other than mu
     double* part;      // CTA 0: [2][3 npart] plaquette partials
     __device__ __forceinline__ ChainShared(char* base, uint32_t C)
         : own(reinterpret_cast<float4*>(base)), tdir(own + 8 * C),
-          phi(reinterpret_cast<float2*>(tdir + 2 * C)), addr(reinterpret_cast<uint32_t*>(phi + 2 * C)),
+          phi(reinterpret_cast<float2*>(tdir + 2 * C)), second(phi + 2 * C),
+          addr(reinterpret_cast<uint32_t*>(second + 2 * C)),
           part(reinterpret_cast<double*>(addr + 40 * C))
     {
     }
 };
 constexpr size_t chain_smem(uint32_t C, uint32_t npart)
 {
-    return (size_t)C * (8 * 16 + 2 * 16 + 2 * 8 + 40 * 4) + 2 * 3 * (size_t)npart * 8;
+    return (size_t)C * (8 * 16 + 2 * 16 + 4 * 8 + 40 * 4) + 2 * 3 * (size_t)npart * 8;
 }
 
 __device__ __forceinline__ Quat<float> ld_cluster(uint32_t a)
@@ -239,21 +228,27 @@ __device__ __forceinline__ Quat<float> ld_cluster(uint32_t a)
     return {v.x, v.y, v.z, v.w};
 }
 
-// The first trial of a link as far as it goes without the staple.
-__device__ __forceinline__ void draw_ahead(const Stream& st, float4* tdir, float2* phi)
+// The first two trials of a link as far as they go without the staple:
+// kp_eval's lambda^2 = t / (2 alpha), accepted iff r4^2 <= 1 - lambda^2
+__device__ __forceinline__ float2 trial_ahead(const U4& w)
 {
-    const U4 w = st.draw(TAG_TRIAL, 0u);
-    // kp_eval: lambda^2 = t / (2 alpha), accepted iff r4^2 <= 1 - lambda^2
     const float t = neg_(fma_(Math<float>::cos2pi_sq(u01<float>(w.y)), Math<float>::ln_u01(u01<float>(w.z)),
                               Math<float>::ln_u01(u01<float>(w.x))));
     const float r4 = u01<float>(w.w);
+    return make_float2(t, mul_(r4, r4));
+}
+__device__ __forceinline__ void draw_ahead(const Stream& st, float4* tdir, float2* phi, float2* second)
+{
+    const U4 w = st.draw(TAG_TRIAL, 0u);
+    const float2 t = trial_ahead(w);
     // new_link_u, new_link_dir: the direction
     const float cth = fma_(2.0f, u18<float>(spare_bits_1(w)), -1.0f);
     const float sth = Math<float>::sqrt_pos(mul_(add_(1.0f, neg_(cth)), add_(1.0f, cth)));
     float sph, cph;
     Math<float>::sincos2pi(u18<float>(spare_bits_2(w)), &sph, &cph);
-    *tdir = make_float4(t, mul_(r4, r4), cth, sth);
+    *tdir = make_float4(t.x, t.y, cth, sth);
     *phi = make_float2(sph, cph);
+    *second = trial_ahead(st.draw(TAG_TRIAL, 1u));
 }
 
 // phase (MU, p) on this thread's link o
@@ -299,13 +294,12 @@ __device__ __forceinline__ void chain_phase(const ChainShared& sh, const LatDesc
     float delta = add_(lam2, lam2);
     uint32_t tr = 1;
     if (!(td.y <= add_(1.0f, neg_(lam2)))) {
-        tr = 0;
-        for (uint32_t t = 1; t < (uint32_t)KP_CAP; ++t) {
-            if (kp_try(st.draw(TAG_TRIAL, t), inv2a, &delta)) {
-                tr = t + 1;
-                break;
-            }
-        }
+        const float2 t2 = sh.second[p * C + o];
+        const float l2 = mul_(t2.x, inv2a);
+        delta = add_(l2, l2);
+        tr = t2.y <= add_(1.0f, neg_(l2)) ? 2 : 0;
+        for (uint32_t t = 2; tr == 0 && t < (uint32_t)KP_CAP; ++t)
+            if (kp_try(st.draw(TAG_TRIAL, t), inv2a, &delta)) tr = t + 1;
     }
     if (tr == 0) {  // cap hit: the link keeps its value
         un = {slot.x, slot.y, slot.z, slot.w};
@@ -354,23 +348,7 @@ hb_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int 
         lex[0] = EoSite(D, i, 0).lex();
         lex[1] = EoSite(D, i, 1).lex();
         const int p = updater ? 0 : 1;
-        const EoSite s(D, i, p);
-        int hp[4], hm[4];
-        s.hops(hp, hm);
-        uint32_t* ad = sh.addr + (size_t)p * 20 * C + o;
-        auto put = [&](int slot, uint32_t e) {
-            if (!chk.ok(0, 0, e)) e = 0;
-            const uint32_t r = fdiv(e, div_c);
-            uint32_t ra;
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(base + ((e - r * C) << 4)), "r"(r));
-            ad[slot * C] = ra;
-        };
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            put(m, i + hp[m]);
-            put(4 + m, i + hm[m]);
-            for (int k = 0; k < 3; ++k) put(8 + 3 * m + k, i + hp[m] + hm[k + (k >= m ? 1 : 0)]);
-        }
+        chain_addresses(D, i, p, C, div_c, base, chk, sh.addr + (size_t)p * 20 * C + o);
     }
     if (pl && rank == 0)
         for (uint32_t k = threadIdx.x; k < 2 * 3 * npart; k += 2 * NU) sh.part[k] = 0.0;
@@ -378,29 +356,14 @@ hb_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int 
         return Stream{(uint32_t)D.seed, (uint32_t)(D.seed >> 32), lex[p] * 4u + (uint32_t)mu,
                       (uint32_t)sw, (uint32_t)(sw >> 32)};
     };
-    if (act && !updater) draw_ahead(stream(0, 0, sw0), sh.tdir + o, sh.phi + o);
+    if (act && !updater) draw_ahead(stream(0, 0, sw0), sh.tdir + o, sh.phi + o, sh.second + o);
     cluster_sync();
 
     uint32_t ntrial = 0, ncap = 0;
-    // sweep_end_kernel's sum of the partials of sweep k on CTA 0, in two steps a
-    // barrier apart (256 virtual threads, then eight warp sums in order)
     auto sum_warps = [&](int k) {
-        const double* part = sh.part + (size_t)(k & 1) * 3 * npart;
-        for (int vw = w; vw < 8; vw += NU / 32) {
-            double acc = 0.0;
-            for (uint32_t e = vw * 32 + lane; e < 3 * npart; e += 256) acc += part[e];
-            acc = warp_sum(acc);
-            if (lane == 0) scratch[vw] = acc;
-        }
+        chain_sum_warps(sh.part + (size_t)(k & 1) * 3 * npart, npart, w, NU / 32, scratch);
     };
-    auto finish_sum = [&](int k) {
-        double tot = 0.0;
-        for (int vw = 0; vw < 8; ++vw) tot += scratch[vw];
-        const double P = tot / (6.0 * (double)D.V);
-        const uint64_t at = sw0 + (uint64_t)k - D.sweep_base;
-        ctx.ring[at % PLAQ_RING] = P;
-        if (D.plaq_out) D.plaq_out[at] = P;
-    };
+    auto finish_sum = [&](int k) { chain_finish_sum(ctx, D, scratch, sw0 + (uint64_t)k); };
     for (int k = 0; k < nsweeps; ++k) {
         const uint64_t sw = sw0 + (uint64_t)k;
 #pragma unroll 1
@@ -422,20 +385,15 @@ hb_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int 
                 if (pl && p == 1 && mu >= 1) {
                     const float wp = warp_sum_t(act ? qretr(un, P) : 0.0f);
                     const uint32_t gw = rank * (C >> 5) + (uint32_t)w;
-                    if (lane == 0 && gw < npart && o < C) {
-                        const uint32_t a = (uint32_t)__cvta_generic_to_shared(
-                            sh.part + (size_t)((k & 1) * 3 + mu - 1) * npart + gw);
-                        uint32_t ra;
-                        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(0u));
-                        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"((double)wp)
-                                     : "memory");
-                    }
+                    if (lane == 0 && gw < npart && o < C)
+                        chain_put_partial(sh.part + (size_t)((k & 1) * 3 + mu - 1) * npart + gw,
+                                          (double)wp);
                 }
             } else {
                 if (act && !(ph8 == 7 && k + 1 == nsweeps)) {
                     const int np = p ^ 1, nmu = (mu + p) & 3;
                     draw_ahead(stream(nmu, np, ph8 == 7 ? sw + 1 : sw), sh.tdir + np * C + o,
-                               sh.phi + np * C + o);
+                               sh.phi + np * C + o, sh.second + np * C + o);
                 }
                 if (pl && rank == 0 && k > 0) {
                     if (ph8 == 0) sum_warps(k - 1);

@@ -157,7 +157,7 @@ __device__ __forceinline__ bool fix_try(const FixCall& C, const U4& w, int64_t i
         *L = lambda_from_delta((uint64_t)__double_as_longlong(delta));
         return ok;
     }
-    *L = kp_lambda(w.x, w.y, w.z, inv, ei, C.tab);
+    *L = kp_lambda(kp_sum(w.x, w.y, w.z, C.tab), inv, ei);
     return kp_accept(*L, w.w);
 }
 
@@ -191,11 +191,11 @@ __device__ __forceinline__ double plaq_double(int64_t v)  // v 2^-51
 // Staple sum by the tree s_k = up_k + lo_k for the k-th nu != mu,
 // A = (s_0 + s_1) + s_2 (P = its prefix over nu < mu), FP64 draw, new link.
 // Returns what update_link returns; *un is the link's final value.
-static __device__ __noinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, uint32_t i,
-                                                    int mu, int p, bool hyb, double* plaq,
-                                                    uint32_t* lex)
+template <typename LT>
+__device__ __noinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, uint32_t i, int mu,
+                                             int p, bool hyb, double* plaq, uint32_t* lex)
 {
-    const Links<double> U(ctx.links, D, ctx.status);
+    const LT U(ctx.links, D, ctx.status);
     const EoSite s(D, i, p);
     int hp[4], hm[4];
     s.hops(hp, hm);
@@ -224,7 +224,7 @@ __device__ __noinline__ void general_links(const Ctx& ctx, int l, uint32_t blk0,
     double plaq = 0.0;
     uint32_t ntrial = 0, ncap = 0, lex;
     for (uint32_t i = i0; i < end; i += step) {
-        const int32_t tr = general_link(ctx, D, i, MU, p, hyb, &plaq, &lex);
+        const int32_t tr = general_link<Links<double>>(ctx, D, i, MU, p, hyb, &plaq, &lex);
         ncap += tr < 0;
         ntrial += tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
         if (dbg) dbg[lex] = tr;

@@ -448,8 +448,13 @@ SU2_HD Lambda lambda_of(int64_t P, int qe)
     const int s = -(qe + 61);
     return {P, s < 0 ? int64_t(-1) : (int64_t)shr64((uint64_t)P, (uint32_t)s), qe};
 }
-SU2_HD Lambda kp_lambda(uint32_t w0, uint32_t w1, uint32_t w2, int64_t inv, int ei,
-                        const FixTables* __restrict__ tab)
+// -(ln r1 + cos^2(2 pi r2) ln r3) = t 2^e, t in [2^61, 2^62): lambda^2 times
+// 2 alpha, which needs no staple
+struct KpSum {
+    int64_t t;
+    int e;
+};
+SU2_HD KpSum kp_sum(uint32_t w0, uint32_t w1, uint32_t w2, const FixTables* __restrict__ tab)
 {
     const NegLn l1 = neg_ln(2u * (w0 >> 9) + 1u, tab), l3 = neg_ln(2u * (w2 >> 9) + 1u, tab);
     // the logarithms at 2^57 (up to 16.64), or at 2^61 where both uniforms
@@ -461,8 +466,11 @@ SU2_HD Lambda kp_lambda(uint32_t w0, uint32_t w1, uint32_t w2, int64_t inv, int 
     const int64_t c2 = ((int64_t(1) << 62) + arc_cos(a)) >> 1;
     const uint64_t T = (uint64_t)(L1 + mulk<2>(limbs(c2), limbs(L3)));  // below 2^62.1
     const int z = clz64(T);
-    const int64_t t = (int64_t)((T << z) >> 2);  // in [2^61, 2^62)
-    return lambda_of(mulk<2>(limbs(t), limbs(inv)), 3 + s - z + ei);
+    return {(int64_t)((T << z) >> 2), s - z - 59};
+}
+SU2_HD Lambda kp_lambda(const KpSum& k, int64_t inv, int ei)
+{
+    return lambda_of(mulk<2>(limbs(k.t), limbs(inv)), 62 + k.e + ei);
 }
 // accepted iff r4^2 <= 1 - lambda^2
 SU2_HD bool kp_accept(const Lambda& L, uint32_t w3)
@@ -497,32 +505,48 @@ SU2_HD int64_t sqrt_fix(uint64_t v, int e)
 // delta (2 - delta) = 4 lambda^2 (1 - lambda^2), the direction n from the two
 // 18-bit integers of the first trial.  X and V are unit to 2^-57, so the
 // product needs no normalisation.
-SU2_HD void new_link_fix(const Lambda& L, uint32_t kd1, uint32_t kd2, const FQuat& V,
-                         const FixTables* __restrict__ tab, int64_t* U)
+// the direction: cos theta at 2^18, the rest at 2^62
+struct FixDir {
+    int32_t cth;
+    int64_t sth, cph, sph;
+};
+SU2_HD FixDir direction_fix(uint32_t kd1, uint32_t kd2, const FixTables* __restrict__ tab)
+{
+    FixDir d;
+    d.cth = (int32_t)(2u * kd1 + 1u) - (1 << 18);
+    const uint64_t N = (uint64_t(1) << 36) - (uint64_t)((int64_t)d.cth * d.cth);
+    const int zn = (clz64(N) - 4) & ~1;
+    d.sth = sqrt_fix(N << zn, -36 - zn);
+    const Arc a = arc_at((2u * kd2 + 1u) << 5, tab);
+    d.cph = arc_cos(a);
+    d.sph = arc_sin(a);
+    return d;
+}
+SU2_HD void new_link_dir_fix(const Lambda& L, const FixDir& d, const FQuat& V, int64_t* U)
 {
     const int64_t W = (int64_t(1) << 61) - L.lam;  // 1 - lambda^2 >= 0
     const int nw = clz64((uint64_t)W | 1u) - 2;
     const int64_t Q = mulk<2>(limbs(L.P), limbs(shl64(W, nw)));  // in [2^59, 2^62)
     // |x|^2 / 4 = Q 2^(qe - nw + 1): |x| = sqrt(Q 2^(qe - nw + 3))
     const int64_t vl = W == 0 ? 0 : sqrt_fix((uint64_t)Q, L.qe - nw + 3);
-    const int32_t cth = (int32_t)(2u * kd1 + 1u) - (1 << 18);  // at 2^18
-    const uint64_t N = (uint64_t(1) << 36) - (uint64_t)((int64_t)cth * cth);
-    const int zn = (clz64(N) - 4) & ~1;
-    const int64_t sth = sqrt_fix(N << zn, -36 - zn);
     const Fx v = limbs(vl);
-    const Fx vs = limbs(mulk<2>(v, limbs(sth)));
-    const Arc a = arc_at((2u * kd2 + 1u) << 5, tab);
+    const Fx vs = limbs(mulk<2>(v, limbs(d.sth)));
     FQuat X;
     X.a0 = limbs((int64_t(1) << 62) - shl64(L.lam, 2));
-    X.a1 = limbs(mulk<2>(vs, limbs(arc_cos(a))));
-    X.a2 = limbs(mulk<2>(vs, limbs(arc_sin(a))));
-    X.a3 = limbs(shl64((int64_t)v.h * cth, 14) + (((int64_t)v.l * cth) >> 18));
+    X.a1 = limbs(mulk<2>(vs, limbs(d.cph)));
+    X.a2 = limbs(mulk<2>(vs, limbs(d.sph)));
+    X.a3 = limbs(shl64((int64_t)v.h * d.cth, 14) + (((int64_t)v.l * d.cth) >> 18));
     // |sum of the cross terms| <= 2 * 2^30 * 2^31 + 2 * 2^26 * 2^31
     const Fx n1 = neg(V.a1), n2 = neg(V.a2), n3 = neg(V.a3);
     U[0] = dot4_k<4>(X.a0, V.a0, X.a1, V.a1, X.a2, V.a2, X.a3, V.a3);
     U[1] = dot4_k<4>(X.a1, V.a0, X.a0, n1, X.a3, n2, X.a2, V.a3);
     U[2] = dot4_k<4>(X.a2, V.a0, X.a0, n2, X.a3, V.a1, X.a1, n3);
     U[3] = dot4_k<4>(X.a3, V.a0, X.a0, n3, X.a2, n1, X.a1, V.a2);
+}
+SU2_HD void new_link_fix(const Lambda& L, uint32_t kd1, uint32_t kd2, const FQuat& V,
+                         const FixTables* __restrict__ tab, int64_t* U)
+{
+    new_link_dir_fix(L, direction_fix(kd1, kd2, tab), V, U);
 }
 
 // Haar element of SU(2) at 2^60 from one Philox block: Box-Muller on (w0, w1)

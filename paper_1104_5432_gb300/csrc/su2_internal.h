@@ -234,6 +234,11 @@ struct ChainGeom {
 };
 bool chain_geometry(uint32_t Vh, int S, ChainGeom* g);
 bool chain_launchable(const ChainGeom& g);
+// ... and on a small single FP64 lattice (cluster64.cu, fix_chain_kernel), after
+// launch_unit_check
+bool chain64_geometry(uint32_t Vh, ChainGeom* g);
+bool chain64_launchable(const ChainGeom& g);
+cudaError_t launch_chain64(const Ctx& c, const ChainGeom& g, bool plaq, int nsweeps, cudaStream_t s);
 cudaError_t launch_chain(const Ctx& c, const ChainGeom& g, bool plaq, int nsweeps, cudaStream_t s);
 cudaError_t launch_init(const Ctx& c, int dtype, int l, uint32_t V, int hot, uint64_t seed,
                         cudaStream_t s);

@@ -23,6 +23,22 @@ __device__ __forceinline__ FQuat fq_link(const Quat<double>& q)
     return {f(q.a0), f(q.a1), f(q.a2), f(q.a3)};
 }
 
+// A link component as a float (0 below 2^-126, at least 2 for |x| >= 2, an
+// infinity or a NaN), from its words: conversion instructions run on the
+// slow FP64 unit.
+__device__ __forceinline__ float narrow(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu;
+    if (e > 1023u) return 2.0f;
+    if (e < 897u) return 0.0f;
+    return __uint_as_float((((hi & 0x7FFFFFFFu) << 3) | (lo >> 29)) - (896u << 23));
+}
+__device__ __forceinline__ bool unit_link(const double2& lo, const double2& hi)
+{
+    const float a = narrow(lo.x), b = narrow(lo.y), c = narrow(hi.x), d = narrow(hi.y);
+    return fabsf(a * a + b * b + c * c + d * d - 1.0f) <= (float)UNIT_TOLERANCE;
+}
 // a quaternion at 2^60 as doubles
 __device__ __forceinline__ Quat<double> dq_link(const int64_t* U)
 {

@@ -183,7 +183,7 @@ int main()
                 uint64_t K;
                 int sc;
                 if (!unit_staple(A, half_inv_beta_fix(bits(0.5 / beta)), &D, &K, &sc)) return 1;
-                const Lambda l = kp_lambda(w[0], w[1], w[2], D.inv, D.ei, &T);
+                const Lambda l = kp_lambda(kp_sum(w[0], w[1], w[2], &T), D.inv, D.ei);
                 const bool okf = kp_accept(l, w[3]);
                 flips += okf != ok;
                 if (!ok || !okf) continue;

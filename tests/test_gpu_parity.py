@@ -1150,19 +1150,21 @@ def test_fp64_lattice_with_non_unit_links(cfg):
     np.testing.assert_allclose(out[0][1], rplaq, rtol=1e-13, atol=0)
 
 
-@pytest.mark.parametrize("Ns,Nt", [(2, 2), (4, 4), (10, 6), (8, 8), (6, 10), (8, 18), (16, 4),
-                                   (16, 6)])
-def test_one_launch_chain_matches_the_phase_launches(Ns, Nt):
-    """Launch shape 0 on a single small FP32 lattice runs all sweeps of a call
-    in one cluster launch (up to 16384 sites: 2^4 with one part-filled warp
-    and 15 idle CTAs, 10^3 x 6 with an uneven last CTA, 8^3 x 18 just over 256
-    links a CTA, 16^3 x 4 the largest, 16^3 x 6 beyond): links, plaquettes,
-    trial statistics and sweep counter equal, bit by bit, those of the same
+@pytest.mark.parametrize("dtype,Ns,Nt", [
+    (su2.F32, 2, 2), (su2.F32, 4, 4), (su2.F32, 10, 6), (su2.F32, 8, 8), (su2.F32, 6, 10),
+    (su2.F32, 8, 18), (su2.F32, 16, 4), (su2.F32, 16, 6),
+    (su2.F64, 2, 2), (su2.F64, 6, 4), (su2.F64, 6, 10), (su2.F64, 8, 8), (su2.F64, 10, 6)])
+def test_one_launch_chain_matches_the_phase_launches(dtype, Ns, Nt):
+    """Launch shape 0 on a single small lattice runs all sweeps of a call in one
+    cluster launch (FP32 up to 16384 sites: 2^4 with one part-filled warp and
+    15 idle CTAs, 10^3 x 6 with an uneven last CTA, 8^3 x 18 just over 256
+    links a CTA, 16^3 x 4 the largest, 16^3 x 6 beyond; FP64 up to 4096 sites:
+    8^4 the largest, 10^3 x 6 beyond): links, plaquettes, trial statistics and sweep counter equal, bit by bit, those of the same
     lattice in a batch, whose sweeps are phase launches -- with host and
     device plaquettes, without, at a coupling with many rejected trials, in
     calls of different lengths, and across a trial-cap hit."""
-    lat = lattice(Ns, Nt, su2.F32)
-    B = su2.Lattice([Ns, 4], [Nt, 2], su2.F32)
+    lat = lattice(Ns, Nt, dtype)
+    B = su2.Lattice([Ns, 4], [Nt, 2], dtype)
     lat.init(su2.HOT, 31)
     B.batch_init(su2.HOT, [31, 32])
     dev = torch.zeros(2, dtype=torch.float64, device="cuda")
