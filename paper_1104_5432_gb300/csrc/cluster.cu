@@ -28,7 +28,8 @@ struct ClusterLinks {
     uint32_t C;     // links per (mu, parity) per CTA
     FastDiv div_c;
     LinkCheck chk;  // bounds-checked builds: a bad index is recorded, link 0 read
-    __device__ __forceinline__ Quat<float> load(int mu, int p, uint32_t eo) const
+    static constexpr int UNIT = 1;
+    __device__ __forceinline__ Quat<float> load_at(int mu, int p, uint32_t eo) const
     {
         if (!chk.ok(mu, p, eo)) eo = 0;
         const uint32_t r = fdiv(eo, div_c);

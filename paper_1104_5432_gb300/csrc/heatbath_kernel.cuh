@@ -104,29 +104,30 @@ __device__ __forceinline__ Quat<T> staple_term(const LT& U, int mu, int nu, int 
     return qmul_nd(qmul_nd(qdag(d), e), qdag(f));
 }
 
-// (U: any link source with load(mu, parity, eo) -- global memory, or the
-// distributed shared memory of a cluster)
+// (U: any link source with load_at(mu, parity, UNIT eo) -- global memory, or
+// the distributed shared memory of a cluster)
 template <typename T, int MU, bool PLAQ, typename LT>
 __device__ __forceinline__ void staple_sum(const LT& U, const EoSite& s, uint32_t i, int p,
                                            Quat<T>& A, Quat<T>& P)
 {
     int hp[4], hm[4];
-    s.hops(hp, hm);
+    s.hops(hp, hm, LT::UNIT);
     const int q = p ^ 1;
-    const uint32_t e_pmu = i + hp[MU];
+    const uint32_t o = i * (uint32_t)LT::UNIT;
+    const uint32_t e_pmu = o + hp[MU];
     A = {T(0), T(0), T(0), T(0)};
 #pragma unroll
     for (int nu = 0; nu < 4; ++nu) {
         if (nu == MU) continue;
-        const uint32_t e_pnu = i + hp[nu];
-        const uint32_t e_mnu = i + hm[nu];
-        const uint32_t e_pmu_mnu = i + hp[MU] + hm[nu];
-        const Quat<T> a = U.load(nu, q, e_pmu);      // U_nu(x+mu)
-        const Quat<T> b = U.load(MU, q, e_pnu);      // U_mu(x+nu)
-        const Quat<T> c = U.load(nu, p, i);          // U_nu(x)
-        const Quat<T> d = U.load(nu, p, e_pmu_mnu);  // U_nu(x+mu-nu)
-        const Quat<T> e = U.load(MU, q, e_mnu);      // U_mu(x-nu)
-        const Quat<T> f = U.load(nu, q, e_mnu);      // U_nu(x-nu)
+        const uint32_t e_pnu = o + hp[nu];
+        const uint32_t e_mnu = o + hm[nu];
+        const uint32_t e_pmu_mnu = e_pmu + hm[nu];
+        const Quat<T> a = U.load_at(nu, q, e_pmu);      // U_nu(x+mu)
+        const Quat<T> b = U.load_at(MU, q, e_pnu);      // U_mu(x+nu)
+        const Quat<T> c = U.load_at(nu, p, o);          // U_nu(x)
+        const Quat<T> d = U.load_at(nu, p, e_pmu_mnu);  // U_nu(x+mu-nu)
+        const Quat<T> e = U.load_at(MU, q, e_mnu);      // U_mu(x-nu)
+        const Quat<T> f = U.load_at(nu, q, e_mnu);      // U_nu(x-nu)
         // A += a b^dagger c^dagger + (e d)^dagger f, the sums fused into
         // the products' last steps
         A = qmul_dn_acc(qmul(e, d), f, qmul_nd_acc(qmul_nd(a, b), c, A));
@@ -350,6 +351,54 @@ __device__ __forceinline__ int32_t update_link(const LT& U, const LatDesc& D, co
 }
 
 // ---------------------------------------------------------------------------
+// lattices of more than 2^29 sites: 64-bit link indices, one link at a time
+// ---------------------------------------------------------------------------
+template <bool HYB>
+__device__ __noinline__ int32_t wide_link(const Ctx& ctx, const LatDesc& D, uint32_t j, bool slab, int mu,
+                                          int p, float* plaq, uint32_t* lex)
+{
+    const WideLinks U(ctx.links, D, ctx.status);
+    uint32_t i = j;
+    const EoSite s = slab ? EoSite::from_slab(D, j, p, &i) : EoSite(D, j, p);
+    Quat<float> un, P = {0.f, 0.f, 0.f, 0.f};
+    int32_t tr;
+    switch (mu) {
+    case 0: tr = update_link<float, 0, false, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
+    case 1: tr = update_link<float, 1, true, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
+    case 2: tr = update_link<float, 2, true, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
+    default: tr = update_link<float, 3, true, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
+    }
+    if (tr >= 0) U.store(mu, p, i, un);
+    else un = U.load_rw(mu, p, i);
+    *plaq = add_(*plaq, qretr(un, P));
+    *lex = s.lex();
+    return tr;
+}
+// a block's tiles of NT R positions, as the kernels below take them
+template <int MU, bool PLAQ, int NT, bool HYB>
+__device__ __noinline__ void wide_links(const Ctx& ctx, int l, uint32_t blk0, uint32_t tile, uint32_t nb,
+                                        int R, bool slab, int p, int32_t* dbg)
+{
+    const LatDesc& D = ctx.desc[l];
+    float plaq = 0.0f;
+    uint32_t ntrial = 0, ncap = 0, lex;
+    const uint32_t ntiles = (D.Vh + NT * (uint32_t)R - 1) / (NT * (uint32_t)R);
+    do {
+        for (int r = 0; r < R; ++r) {
+            const uint32_t j = tile * (NT * (uint32_t)R) + (uint32_t)r * NT + threadIdx.x;
+            if (j >= D.Vh) break;
+            const int32_t tr = wide_link<HYB>(ctx, D, j, slab, MU, p, &plaq, &lex);
+            ncap += tr < 0;
+            ntrial += tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
+            if (dbg) dbg[lex] = tr;
+        }
+        tile += nb;
+    } while (nb && tile < ntiles);
+    __syncwarp();
+    warp_totals<float, MU, PLAQ, NT>(ctx, l, blk0, D.Vh, plaq, ntrial, ncap);
+}
+
+// ---------------------------------------------------------------------------
 // one link per thread
 // ---------------------------------------------------------------------------
 template <typename T, int MU, bool PLAQ, bool DBG, int NT, int MINB, bool SLAB, bool HYB>
@@ -361,6 +410,10 @@ hb_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const uint32_t Vh = D.Vh;
     const uint32_t blk0 = first_block(ctx.phase_start, l);
     const uint32_t j = (blockIdx.x - blk0) * NT + threadIdx.x;  // traversal position
+    if (Vh > OFF32_MAX_VH) {
+        wide_links<MU, PLAQ, NT, HYB>(ctx, l, blk0, blockIdx.x - blk0, 0u, 1, SLAB, p, dbg);
+        return;
+    }
     const Links<T> U(ctx.links, D, ctx.status);
 
     T plaq = T(0);
@@ -540,6 +593,10 @@ hb_phase_queue_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const uint32_t nb = PERSIST ? __ldg(ctx.phase_start + l + 1) - blk0 : 0u;
     const uint32_t ntiles = PERSIST ? (Vh + NT * R - 1) / (NT * R) : 0u;
     uint32_t tile = blockIdx.x - blk0;
+    if (Vh > OFF32_MAX_VH) {
+        wide_links<MU, PLAQ, NT, HYB>(ctx, l, blk0, tile, nb, R, SLAB, p, dbg);
+        return;
+    }
     const Links<T> U(ctx.links, D, ctx.status);
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;

@@ -1183,3 +1183,33 @@ def test_one_launch_chain_matches_the_phase_launches(dtype, Ns, Nt):
             lat.heatbath(1e-9, 1, 3)
         assert e.value.code == su2.SU2_E_TRIALS
         np.testing.assert_array_equal(lat.get_links(), before)
+
+
+@pytest.mark.parametrize("shape", [0, 7])
+def test_lattice_beyond_32_bit_link_offsets(shape):
+    """128^3 x 258 FP32 (2^29 + 2^22 sites, 35 GB of links): a (mu, parity)
+    plane is longer than a 32-bit byte offset reaches, so the phase kernels
+    index links in 64 bits.  The first phase from the hot start, links sampled
+    over the whole lattice and in its last time slices, against the oracle's
+    draws from its own hot start."""
+    Ns, Nt, seed = 128, 258, 3
+    V = Ns ** 3 * Nt
+    lat = lattice(Ns, Nt, su2.F32)
+    lat.set_launch_config(shape)
+    lat.init(su2.HOT, seed)
+    lat.heatbath_phase(2.5, 0, 0, seed)
+    lat.sync()
+    st = lat.stats()
+    assert st["updates"] == V // 2 and st["cap_hits"] == 0
+    rng = np.random.default_rng(2)
+    lex = np.concatenate([rng.integers(0, V, 400), V - 1 - rng.integers(0, 2 * Ns ** 3, 400)])
+    x, y, z, t = lex % Ns, (lex // Ns) % Ns, (lex // Ns ** 2) % Ns, lex // Ns ** 3
+    lex = lex[(x + y + z + t) % 2 == 0]
+    got = sampled_links(lat, V, lex, su2.F32)
+    lat.close()
+    torch.cuda.empty_cache()
+    flips = 0
+    for k, i in enumerate(lex):
+        u, tr = O.heatbath_link_hot(Ns, Nt, seed, 2.5, 0, int(i), seed, 0)
+        flips += float(np.max(np.abs(got[k, 0] - u))) > 2e-5
+    assert len(lex) > 300 and flips <= 1
