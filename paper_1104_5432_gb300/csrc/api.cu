@@ -117,7 +117,8 @@ struct su2_lattice {
     size_t link_bytes = 0, work_bytes = 0;
     size_t off_status = 0, off_desc = 0, off_sstart = 0, off_spstart = 0;
     size_t off_plaq = 0, off_obs = 0, off_field = 0, off_ring = 0, off_res = 0, off_stage = 0;
-    size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0, off_fixtab = 0, off_mirror = 0;
+    size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0, off_fixtab = 0, off_mirror = 0, off_oflag = 0;
+    bool wide = false;              // some lattice of more than 2^29 sites
     bool mirror = false;            // FP64: the work buffer holds a fixed-point copy of the links
     uint32_t max_chunks = 1;
     size_t res_doubles = 0;
@@ -251,6 +252,7 @@ int layout(su2_lattice* L)
         const uint64_t Ns = (uint64_t)L->Ns[l], Nt = (uint64_t)L->Nt[l];
         L->Vs[l] = Ns * Ns * Ns;
         L->V[l] = L->Vs[l] * Nt;
+        L->wide = L->wide || L->V[l] > (uint64_t(1) << 29);
         L->link_off[l] = lb;
         lb += align256(4 * L->V[l] * link_size);
         L->field_off[l] = fo;
@@ -288,7 +290,12 @@ int layout(su2_lattice* L)
         w += align256(bytes);
         return o;
     };
+    // the status word, the results and the plaquette ring lie together: one
+    // copy brings a call's results and its status to the host
+    L->res_doubles = (size_t)n * (L->rmax_limit + 1) + 2 * (size_t)n;
     L->off_status = take(256);
+    L->off_res = take(8 * L->res_doubles);
+    L->off_ring = take(8 * (size_t)PLAQ_RING * n);
     L->off_desc = take(sizeof(LatDesc) * n);
     for (int k = 0; k < NUM_LAUNCH_CFG; ++k) L->off_pstart_cfg[k] = take(4 * (n + 1));
     L->off_sstart = take(4 * (n + 1));
@@ -298,13 +305,11 @@ int layout(su2_lattice* L)
                                              (size_t)L->spat_blocks * (size_t)(L->rmax_limit + 1));
     L->off_obs = take(8 * obs_rows);
     L->off_field = take(8 * fo);
-    L->off_ring = take(8 * (size_t)PLAQ_RING * n);
     L->off_chunks = take(8 * (size_t)L->max_chunks * n);
     L->off_tickets = take(4 * (size_t)n);
     L->off_tslots = take(8 * (size_t)TRIAL_SLOTS * n);
-    L->res_doubles = (size_t)n * (L->rmax_limit + 1) + 2 * (size_t)n;
+    L->off_oflag = take(4 * (size_t)n);
     L->off_acc = take(8 * L->res_doubles);
-    L->off_res = take(8 * L->res_doubles);
     L->off_stage = take(STAGE_BYTES);
     L->off_fp64tab = take(sizeof(double2) * FP64_TABLE_ENTRIES);
     L->off_fixtab = take(sizeof(FixTables));
@@ -398,7 +403,7 @@ int set_params(su2_lattice* L, const double* betas, double beta, const uint64_t*
 int record_measure(su2_lattice* L, int rmax, cudaStream_t s)
 {
     double* acc = L->acc_dev();
-    SU2_CUDA(launch_polyakov(L->ctx, L->dtype, acc, acc + L->n, 1, s));
+    SU2_CUDA(launch_polyakov(L->ctx, L->row, L->wide, acc, acc + L->n, 1, s));
     SU2_CUDA(launch_correlator(L->ctx, L->dtype, rmax, acc + 2 * L->n, 1, s));
     return SU2_OK;
 }
@@ -500,12 +505,9 @@ int measure_tail_graph(su2_lattice* L, int rmax, cudaGraphExec_t* exec)
     return SU2_OK;
 }
 
-// synchronise and turn a latched cap hit into SU2_E_TRIALS
-int sync_status(su2_lattice* L)
+// turn a latched status word (fetched to the host) into its error, once
+int report_status(su2_lattice* L, uint32_t st)
 {
-    SU2_CUDA(cudaStreamSynchronize(L->stream));
-    uint32_t st = 0;
-    SU2_CUDA(cudaMemcpy(&st, L->status_dev(), sizeof st, cudaMemcpyDeviceToHost));
     if (st) {
         SU2_CUDA(cudaMemset(L->status_dev(), 0, sizeof st));
         if (st & STATUS_BOUNDS)
@@ -516,6 +518,32 @@ int sync_status(su2_lattice* L)
             return fail(SU2_E_TRIALS, "Kennedy-Pendleton trial cap (%d) hit; links kept", KP_CAP);
     }
     return SU2_OK;
+}
+
+// synchronise and turn a latched cap hit into SU2_E_TRIALS
+int sync_status(su2_lattice* L)
+{
+    uint32_t st = 0;
+    SU2_CUDA(cudaMemcpyAsync(&st, L->status_dev(), sizeof st, cudaMemcpyDeviceToHost, L->stream));
+    SU2_CUDA(cudaStreamSynchronize(L->stream));
+    return report_status(L, st);
+}
+
+// As sync_status, and the work buffer's bytes between the status word and
+// `bytes` past src come with it in the same copy (each copy to pageable memory
+// and its wait take ~10 us): *host points at src's values.
+int fetch_status(su2_lattice* L, const double* src, size_t bytes, const double** host)
+{
+    static thread_local std::vector<char> buf;
+    const size_t at = (size_t)(reinterpret_cast<const char*>(src) - (L->work + L->off_status));
+    buf.resize(at + bytes);
+    SU2_CUDA(cudaMemcpyAsync(buf.data(), L->work + L->off_status, at + bytes, cudaMemcpyDeviceToHost,
+                             L->stream));
+    SU2_CUDA(cudaStreamSynchronize(L->stream));
+    uint32_t st = 0;
+    memcpy(&st, buf.data(), sizeof st);
+    *host = reinterpret_cast<const double*>(buf.data() + at);
+    return report_status(L, st);
 }
 
 // Whether the whole-sweep cluster kernel applies to this handle: one FP32
@@ -631,10 +659,15 @@ int heatbath_impl(su2_lattice* L, const double* betas, double beta, int nsweeps,
                 SU2_CUDA(cudaGraphLaunch(g_first && done + s == 0 ? g_first : g, L->stream));
         }
         if (want && !dev_out) {
-            for (int l = 0; l < L->n; ++l)
-                SU2_CUDA(cudaMemcpyAsync(plaq + (size_t)l * nsweeps + done,
-                                         L->ring_dev() + (size_t)l * PLAQ_RING,
-                                         sizeof(double) * chunk, cudaMemcpyDeviceToHost, L->stream));
+            if (L->n == 1 && rmax < 0 && done + chunk == nsweeps) {
+                const double* host = nullptr;
+                const int rc = fetch_status(L, L->ring_dev(), sizeof(double) * chunk, &host);
+                if (host) memcpy(plaq + done, host, sizeof(double) * chunk);
+                return rc;
+            }
+            SU2_CUDA(cudaMemcpy2DAsync(plaq + done, sizeof(double) * nsweeps, L->ring_dev(),
+                                       sizeof(double) * PLAQ_RING, sizeof(double) * chunk, L->n,
+                                       cudaMemcpyDeviceToHost, L->stream));
         }
         done += chunk;
     }
@@ -671,9 +704,10 @@ int init_impl(su2_lattice* L, int start, const uint64_t* seeds, uint64_t seed)
 // out: host or device; produce n*rows doubles through the result area
 int finish_output(su2_lattice* L, double* out, const double* dev_src, size_t count)
 {
-    SU2_CUDA(cudaMemcpyAsync(out, dev_src, sizeof(double) * count, cudaMemcpyDeviceToHost,
-                             L->stream));
-    return sync_status(L);
+    const double* host = nullptr;
+    const int rc = fetch_status(L, dev_src, sizeof(double) * count, &host);
+    if (host) memcpy(out, host, sizeof(double) * count);
+    return rc;
 }
 
 }  // namespace
@@ -1015,6 +1049,7 @@ int su2_bind_memory(su2_lattice* lat, void* links, size_t link_bytes, void* work
                         cudaMemcpyHostToDevice));
     SU2_CUDA(cudaMemset(w + lat->off_ring, 0, 8 * (size_t)PLAQ_RING * lat->n));
     SU2_CUDA(cudaMemset(w + lat->off_tickets, 0, 4 * (size_t)lat->n));
+    SU2_CUDA(cudaMemset(w + lat->off_oflag, 0, 4 * (size_t)lat->n));
     SU2_CUDA(cudaMemset(w + lat->off_tslots, 0, 8 * (size_t)TRIAL_SLOTS * lat->n));
 
     Ctx& c = lat->ctx;
@@ -1034,6 +1069,7 @@ int su2_bind_memory(su2_lattice* lat, void* links, size_t link_bytes, void* work
     c.max_chunks = lat->cfg_chunks[0];
     c.phase_wpb = (uint32_t)LAUNCH_CFG[lat->row][0].threads / 32;
     c.status = reinterpret_cast<uint32_t*>(w + lat->off_status);
+    c.obs_flag = reinterpret_cast<uint32_t*>(w + lat->off_oflag);
     c.n = lat->n;
     c.phase_blocks = lat->phase_blocks[0];
     c.site_blocks = lat->site_blocks;
@@ -1160,7 +1196,7 @@ int su2_plaquette(su2_lattice* lat, double* out)
     DeviceGuard dg(lat->device);
     const bool dev = is_device_ptr(out);
     double* tgt = dev ? out : lat->res_dev();
-    SU2_CUDA(launch_plaquette(lat->ctx, lat->dtype, tgt, lat->stream));
+    SU2_CUDA(launch_plaquette(lat->ctx, lat->row, lat->wide, tgt, lat->stream));
     if (!dev) return finish_output(lat, out, tgt, lat->n);
     return SU2_OK;
 }
@@ -1175,14 +1211,15 @@ int su2_polyakov_loop(su2_lattice* lat, double* out_signed, double* out_abs)
         return fail(SU2_E_INVAL, "out_signed and out_abs must both be host or both device");
     double* ts = dev ? out_signed : lat->res_dev();
     double* ta = out_abs ? (dev ? out_abs : lat->res_dev() + lat->n) : nullptr;
-    SU2_CUDA(launch_polyakov(lat->ctx, lat->dtype, ts, ta, 0, lat->stream));
+    SU2_CUDA(launch_polyakov(lat->ctx, lat->row, lat->wide, ts, ta, 0, lat->stream));
     if (!dev) {
-        SU2_CUDA(cudaMemcpyAsync(out_signed, ts, sizeof(double) * lat->n, cudaMemcpyDeviceToHost,
-                                 lat->stream));
-        if (out_abs)
-            SU2_CUDA(cudaMemcpyAsync(out_abs, ta, sizeof(double) * lat->n,
-                                     cudaMemcpyDeviceToHost, lat->stream));
-        return sync_status(lat);
+        const double* host = nullptr;
+        const int rc = fetch_status(lat, ts, sizeof(double) * 2 * lat->n, &host);
+        if (host) {
+            memcpy(out_signed, host, sizeof(double) * lat->n);
+            if (out_abs) memcpy(out_abs, host + lat->n, sizeof(double) * lat->n);
+        }
+        return rc;
     }
     return SU2_OK;
 }
@@ -1198,7 +1235,7 @@ int su2_polyakov_correlator(su2_lattice* lat, int rmax, double* out, int accumul
     const size_t cnt = (size_t)lat->n * (rmax + 1);
     double* scratch = lat->res_dev();  // [2n] Polyakov means, then correlator rows
     double* tgt = dev ? out : scratch + 2 * lat->n;
-    SU2_CUDA(launch_polyakov(lat->ctx, lat->dtype, scratch, scratch + lat->n, 0, lat->stream));
+    SU2_CUDA(launch_polyakov(lat->ctx, lat->row, lat->wide, nullptr, nullptr, 0, lat->stream));
     if (!dev && accumulate)
         SU2_CUDA(cudaMemcpyAsync(tgt, out, sizeof(double) * cnt, cudaMemcpyHostToDevice,
                                  lat->stream));

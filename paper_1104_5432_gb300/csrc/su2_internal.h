@@ -153,6 +153,7 @@ struct Ctx {
     double* chunk_partial;         // [n][max_chunks] sweep_end chunk sums
     uint32_t* chunk_count;         // [n] sweep_end tickets (zero between sweeps)
     unsigned long long* trial_slots;  // [n][TRIAL_SLOTS] Kennedy-Pendleton trial counts
+    uint32_t* obs_flag;            // [n] FP64 plaquette: a non-unit link was seen (zero between)
     uint32_t* status;
     int n;
     uint32_t phase_blocks, site_blocks, spat_blocks;
@@ -252,8 +253,10 @@ cudaError_t launch_links_from_canonical(const Ctx& c, int dtype, int l, uint32_t
                                         uint32_t nsite, const void* src, int cdtype,
                                         cudaStream_t s, bool pairs_whole = false);
 cudaError_t launch_gauge(const Ctx& c, int dtype, int l, uint32_t V, uint64_t seed, cudaStream_t s);
-cudaError_t launch_plaquette(const Ctx& c, int dtype, double* out_dev, cudaStream_t s);
-cudaError_t launch_polyakov(const Ctx& c, int dtype, double* out_signed_dev,
+// row: the links' layout; wide: some lattice of more than 2^29 sites.
+// launch_polyakov with a null out_signed_dev fills the field only.
+cudaError_t launch_plaquette(const Ctx& c, int row, bool wide, double* out_dev, cudaStream_t s);
+cudaError_t launch_polyakov(const Ctx& c, int row, bool wide, double* out_signed_dev,
                             double* out_abs_dev, int accumulate, cudaStream_t s);
 cudaError_t launch_correlator(const Ctx& c, int dtype, int rmax, double* out_dev, int accumulate,
                               cudaStream_t s);

@@ -110,6 +110,11 @@ template <> struct Links<double> {
         const double2 hi = __ldg(base + idx(mu, p, 1, eo));
         return {lo.x, lo.y, hi.x, hi.y};
     }
+    static constexpr int UNIT = 1;
+    __device__ __forceinline__ Quat<double> load_at(int mu, int p, uint32_t off) const
+    {
+        return load(mu, p, off);
+    }
     __device__ __forceinline__ Quat<double> load_rw(int mu, int p, uint32_t eo) const
     {
         const double2 lo = base[idx(mu, p, 0, eo)];
@@ -160,6 +165,11 @@ struct PairLinks {
         const size_t i = size_t(mu * 2 + p) * Vh + 2 * (size_t)q;
         base[i] = make_float4(u.a0.x, u.a0.y, u.a1.x, u.a1.y);
         base[i + 1] = make_float4(u.a2.x, u.a2.y, u.a3.x, u.a3.y);
+    }
+    static constexpr int UNIT = 1;
+    __device__ __forceinline__ Quat<float> load_at(int mu, int p, uint32_t off) const
+    {
+        return load(mu, p, off);
     }
     // one site eo (either lane): the floats at lane, 2 + lane, 4 + lane, 6 + lane
     __device__ __forceinline__ const float* site(int mu, int p, uint32_t eo) const
@@ -289,7 +299,9 @@ struct EoSite {
         const uint32_t z = q - t * (uint32_t)d.Ns;
         const int p = (int)((x + y + z + t) & 1u);
         *parity = p;
-        return EoSite(d, lex >> 1, p);
+        EoSite s;
+        s.set(d, x >> 1, y, z, t, r, p);
+        return s;
     }
 
     // eo offsets of x + e_d (plus) and x - e_d (minus), wrap included, in units

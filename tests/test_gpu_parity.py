@@ -1213,3 +1213,26 @@ def test_lattice_beyond_32_bit_link_offsets(shape):
         u, tr = O.heatbath_link_hot(Ns, Nt, seed, 2.5, 0, int(i), seed, 0)
         flips += float(np.max(np.abs(got[k, 0] - u))) > 2e-5
     assert len(lex) > 300 and flips <= 1
+
+
+def test_fp64_plaquette_fixed_point_and_non_unit_links():
+    """The FP64 plaquette in fixed point on unit links (identity, random, one
+    sweep on), and the FP64 kernel's on a lattice of a batch whose links are
+    not unit quaternions (one component of one link off by 1%, and all links
+    scaled), each to 1e-13 of the oracle; the look at the norms does not
+    stick to the next call."""
+    shapes = [(6, 4), (4, 6), (2, 2)]
+    B = su2.Lattice([s[0] for s in shapes], [s[1] for s in shapes], su2.F64)
+    B.batch_init(su2.COLD, [1, 2, 3])
+    np.testing.assert_array_equal(B.plaquette(), np.ones(3))
+    clean = [inputs.random_links(*s, 5 + l) for l, s in enumerate(shapes)]
+    bent = [c.copy() for c in clean]
+    bent[0][17, 2, 1] *= 1.01
+    bent[1] *= 1.7
+    for links in (clean, bent, clean):
+        for l in range(3):
+            B.set_links(links[l], l)
+        P = B.plaquette()
+        for l, (Ns, Nt) in enumerate(shapes):
+            ref = O.plaquette(Ns, Nt, links[l])
+            assert abs(P[l] - ref) <= 1e-13 * max(1.0, abs(ref)), (l, P[l], ref)
