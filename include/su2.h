@@ -262,8 +262,8 @@ int su2_set_sweep(su2_lattice* lat, int l, uint64_t sweep);
  *          6 32x32 /2  7 32x32 /4  8 32x32 /8  9 32x16 /4 staged
  *          10 32x32 /2 P  11 32x32 /1 P  12 32x32 slab /8  13 32x32 slab /16
  *   FP64:  0 256x1   1 128x4   2 64x8   3 64x4   4 32x16   5 32x8
- *          6 32x16 /2  7 32x16 /4  8 32x16 /8  9 32x16 /16  10 64x8 G8
- *          11 32x16 G8  12 32x16 /2 P  13 32x16 /8 P
+ *          6 32x16 /2  7 32x16 /4  8 32x16 /8  9 32x16 /16  10 128x4 G4
+ *          11 128x7 G4  12 32x16 /2 P  13 32x16 /8 P
  *   FP32 site pairs (SU2_LAYOUT_PAIRS; R counts pairs): 0 256x2  1 32x16
  *          2 32x20  3 32x24  4 32x28  5 32x16 /2  6 32x20 /2  7 32x24 /2
  *          8 32x24 /4  9 32x20 /4  10 32x24 /1 P  11 32x16 /1 P
@@ -274,8 +274,8 @@ int su2_set_sweep(su2_lattice* lat, int l, uint64_t sweep);
  * lattice only the blocks that fit on the GPU at once are launched, each
  * walking tiles of R rounds in grid-stride order with one queue drain at
  * the end; on a batch one block per tile, as the other shapes; staged: the
- * neighbour rows of a warp copied into shared memory by bulk copies; G8:
- * eight lanes per link, the staple terms and trials in parallel, for small
+ * neighbour rows of a warp copied into shared memory by bulk copies; G4:
+ * four threads per link, the staple terms and trials in parallel, for small
  * FP64 lattices.)  Small blocks spread tiny lattices over more SMs; several
  * links per thread pay off on large ones.  Results never depend on the
  * shape (the random streams are keyed by link and sweep). */

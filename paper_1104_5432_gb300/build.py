@@ -35,7 +35,7 @@ SHAPE_UNITS = [(f"heatbath_shapes_{ROW_NAMES[row]}_{k}",
                for row in (0, 2) for k in range(0, 14, 2)]
 SHAPE_UNITS += [(f"heatbath_fp64_{kind}_{hyb}",
                  (f"SU2_KIND={kind}", f"SU2_HYB={hyb}"), ())
-                for kind in range(5) for hyb in (0, 1)]
+                for kind in range(6) for hyb in (0, 1)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

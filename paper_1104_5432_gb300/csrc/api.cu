@@ -226,7 +226,7 @@ bool is_device_ptr(const void* p)
 }
 
 // links one block of launch shape k updates per phase (a site-pair shape's
-// rounds count pairs; a cooperative shape gives each link `group` lanes)
+// rounds count pairs; FP64 shapes 10 and 11 give each link `group` threads)
 uint64_t links_per_block(const su2_lattice* L, int k)
 {
     const LaunchCfg& c = LAUNCH_CFG[L->row][k];

@@ -11,8 +11,8 @@
 // cosines, the direction -- in the meantime.  Some of 2048 links reject a
 // trial or two in every phase and all wait for them, so two more trials per
 // link are drawn ahead, by the two idle plane threads (8^4, beta = 2.3, us a
-// sweep with 1, 2, 3, 4 trials ahead: 39.4, 37.4, 36.0, 37.2; eight lanes per
-// link in phase launches: 47.2).  Bound by the integer pipes of 16 SMs:
+// sweep with 1, 2, 3, 4 trials ahead: 39.4, 37.4, 36.0, 37.2; phase
+// launches of four threads per link: 44.0).  Bound by the integer pipes of 16 SMs:
 // ~2,900 instructions per 32 links on 64 sub-partitions.  The stored doubles go straight
 // to global memory.  Every value comes from the functions of su2_fixed.cuh,
 // and the plaquette partials are summed in launch shape 0's order: links and
@@ -30,17 +30,6 @@ constexpr int C64_LINKS = 128;  // threads per quarter: links of a phase per CTA
 // drawn ahead for one link: its direction (trial 0's spare bits) and trials
 // 0 .. AHEAD - 1 (KpSum, and the word the accept test takes)
 constexpr int AHEAD = 3;
-struct Trial64 {
-    int64_t t;
-    int32_t e;
-    uint32_t w3;
-};
-struct Dir64 {
-    int64_t sth, cph, sph;
-    int32_t cth, pad;
-};
-static_assert(sizeof(Trial64) == 16 && sizeof(Dir64) == 32, "16-byte accesses");
-
 struct Chain64Shared {
     int4* own;        // [8][2][C] limbs of the links
     longlong2* sums;  // [3][2][C] staple sums of the three planes

@@ -137,13 +137,14 @@ cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, boo
     if (row == ROW_F64) {
         using Fn = cudaError_t (*)(const Ctx&, const LaunchCfg&, int, int, bool, int32_t*, bool,
                                    cudaStream_t);
-        static_assert(NUM_FIX_KINDS == 5, "one entry per kernel below");
+        static_assert(NUM_FIX_KINDS == 6, "one entry per kernel below");
         static const Fn kinds[NUM_FIX_KINDS][2] = {
             {launch_fix_kind<0, false>, launch_fix_kind<0, true>},
             {launch_fix_kind<1, false>, launch_fix_kind<1, true>},
             {launch_fix_kind<2, false>, launch_fix_kind<2, true>},
             {launch_fix_kind<3, false>, launch_fix_kind<3, true>},
             {launch_fix_kind<4, false>, launch_fix_kind<4, true>},
+            {launch_fix_kind<5, false>, launch_fix_kind<5, true>},
         };
         const LaunchCfg& f = LAUNCH_CFG[ROW_F64][cfg];
         return kinds[fix_kind(f)][hybrid](c, f, mu, parity, plaq, dbg_trials, mirror && c.mirror, s);

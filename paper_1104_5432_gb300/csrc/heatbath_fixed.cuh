@@ -1,7 +1,7 @@
 // heatbath_fixed.cuh -- the FP64 phase kernels: links stored as doubles,
 // updated in 64-bit fixed point (su2_fixed.cuh), in the three forms of the
 // launch-shape table: one link per thread, R links per thread with a
-// per-warp retry queue, eight lanes per link.
+// per-warp retry queue, four threads per link.
 //
 // An FP64 warp instruction holds its SM sub-partition for ~76 clocks on
 // GB300, an IMAD.WIDE or a logic operation for 2, so the FP64 sequence
@@ -470,116 +470,194 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
 }
 
 // ---------------------------------------------------------------------------
-// eight lanes per link: small lattices
+// four threads per link: small lattices
 // ---------------------------------------------------------------------------
-// A small lattice (8^4: 2048 links per phase) has one warp of one link per
-// thread for a tenth of the SM sub-partitions, and a phase lasts as long as
-// one link's chain.  Here lanes 0..5 of a group of eight compute the six
-// staple terms at once, their integer sums meet in a butterfly (any order
-// gives the same bits), and the eight lanes try eight trials at once; the
-// link takes the first accepted one of its own sequence.
-template <int MU, bool PLAQ, bool HYB, bool MIR>
-__global__ void __launch_bounds__(64, 8)
-fix_coop_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
+// A lattice that gives each SM sub-partition a warp or two of one link per
+// thread (16^4: 1024 warps per phase) spends a phase in one link's chain of
+// ~2,700 instructions.  Here four warps share 32 links: three form the staple
+// terms of one plane each (exact integer sums: any order gives the same bits),
+// the fourth draws the first trial and the direction meanwhile.  The first
+// warp then adds the sums, decides and stores; among 32 links some nearly
+// always reject, so the others draw the next trials while it does.  Links
+// still waiting get four trials at a time, one from each warp, and take the
+// first accepted one of their own sequence.  us a sweep at beta = 2.3, the
+// best one link per thread / eight lanes per link (which this replaced) /
+// here with 128 registers / with 72, which hold 7 blocks an SM instead of 4:
+//   8^4  74.5 / 47.2 / 44.0 / 47.7    12^4  78.3 / 87.9 / 53.3 / 56.4
+//   16^4 95.1 / 184.5 / 88.3 / 79.1   20^4 164 / 391 / 178 / 148
+//   24^4 266 against 349 in an earlier form: one link per thread takes over.
+// Trials drawn ahead: with 128 registers 2 or 3 give 53.7, 53.3 at 12^4; with
+// 72, where the SM is full, 79.1, 80.0 at 16^4 and 148, 152 at 20^4.
+struct Trial64 {
+    int64_t t;
+    int32_t e;
+    uint32_t w3;
+};
+struct Dir64 {
+    int64_t sth, cph, sph;
+    int32_t cth, pad;
+};
+static_assert(sizeof(Trial64) == 16 && sizeof(Dir64) == 32, "16-byte accesses");
+
+template <int MU, bool PLAQ, bool HYB, bool MIR, int MINB>
+__global__ void __launch_bounds__(128, MINB)
+fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
-    constexpr int G = 8;
-    static_assert(KP_CAP % G == 0, "whole trial groups");
+    struct Group {
+        longlong2 sums[2][2][32];  // planes 1 and 2
+        Trial64 trial[4][32];
+        Dir64 dir[32];
+        uint32_t pend;
+    };
+    constexpr int SPEC = MINB > 4 ? 2 : 3;  // trials drawn ahead besides the first
+    __shared__ Group G;
     const int l = lattice_of_block(ctx.phase_start, ctx.n, blockIdx.x);
     const LatDesc& D = ctx.desc[l];
     const uint32_t Vh = D.Vh;
     const uint32_t blk0 = first_block(ctx.phase_start, l);
-    const int lane = threadIdx.x & 31, g = lane & (G - 1), g0 = lane & ~(G - 1);
-    const uint32_t i = (blockIdx.x - blk0) * (blockDim.x / G) + threadIdx.x / G;
-    const bool act = i < Vh;  // uniform within the group
+    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+    const uint32_t i = (blockIdx.x - blk0) * 32u + (uint32_t)lane;
+    const bool act = i < Vh;
     if (D.nonunit) {
-        general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, act && g == 0 ? i + 1 : i, p, HYB, dbg);
+        general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, act && role == 0 ? i + 1 : i, p, HYB, dbg);
         return;
     }
     const FixLinks<MIR> U(ctx, D);
     const FixCall C(D);
+    auto draw = [&](const Stream& st, int t, int slot) {
+        const U4 w = st.draw(TAG_TRIAL, (uint32_t)t);
+        const KpSum k = kp_sum(w.x, w.y, w.z, C.tab);
+        G.trial[slot][lane] = {k.t, k.e, w.w};
+        if (t == 0) {
+            const FixDir f = direction_fix(spare_bits_1(w), spare_bits_2(w), C.tab);
+            G.dir[lane] = {f.sth, f.cph, f.sph, f.cth, 0};
+        }
+    };
 
-    int64_t A[4] = {0, 0, 0, 0}, P[4] = {0, 0, 0, 0};
-    uint32_t key = 0;
+    int64_t A[4] = {0, 0, 0, 0}, P[4];
+    uint32_t lex = 0;
     if (act) {
         const EoSite s(D, i, p);
-        int hp[4], hm[4];
-        s.hops(hp, hm);
-        key = s.lex() * 4u + MU;
-        if (g < 6) {
-            const int nu = nu_of<MU>(g >> 1);
+        lex = s.lex();
+        if (role < 3) {
+            int hp[4], hm[4];
+            s.hops(hp, hm);
+            const int nu = nu_of<MU>(role);
             const int hpn = nu == 0 ? hp[0] : (nu == 1 ? hp[1] : (nu == 2 ? hp[2] : hp[3]));
             const int hmn = nu == 0 ? hm[0] : (nu == 1 ? hm[1] : (nu == 2 ? hm[2] : hm[3]));
-            fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, (g & 1) != 0, A);
-            if (PLAQ && nu < MU) {
+            fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, false, A);
+            fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, true, A);
+            if (role > 0) {
+                G.sums[role - 1][0][lane] = make_longlong2(A[0], A[1]);
+                G.sums[role - 1][1][lane] = make_longlong2(A[2], A[3]);
+            }
+        } else if (!HYB) {
+            draw(C.stream(lex * 4u + MU), 0, 0);
+        }
+    }
+    __syncthreads();
+    const Stream st = C.stream(lex * 4u + MU);
+    Drawn d;
+    double qc = 0.0;
+    Lambda L = {0, 0, 0};
+    int32_t tr = -1;
+    uint32_t kd1 = 0, kd2 = 0;
+    bool haar = false, wait = false;
+    if (role == 0 && act) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) P[c] = A[c];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const longlong2 lo = G.sums[r][0][lane], hi = G.sums[r][1][lane];
+            A[0] += lo.x;
+            A[1] += lo.y;
+            A[2] += hi.x;
+            A[3] += hi.y;
+            if (PLAQ && r + 1 < MU) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) P[c] = A[c];
             }
         }
-    }
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            A[c] += (int64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)A[c], o);
-            if (PLAQ && MU < 3)
-                P[c] += (int64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)P[c], o);
+        haar = !fix_prepare<HYB>(C, A, &d, &qc);
+        if (haar) {
+            tr = 0;
+        } else if (HYB) {
+            U4 w = st.draw(TAG_TRIAL, 0u);
+            kd1 = spare_bits_1(w);
+            kd2 = spare_bits_2(w);
+            for (int t = 0; t < KP_CAP; w = st.draw(TAG_TRIAL, (uint32_t)++t))
+                if (fix_try<true>(C, w, d.inv, d.ei, qc, &L)) {
+                    tr = t + 1;
+                    break;
+                }
+        } else {
+            const Trial64 a = G.trial[0][lane];
+            L = kp_lambda(KpSum{a.t, a.e}, d.inv, d.ei);
+            if (kp_accept(L, a.w3)) tr = 1;
+            else wait = true;
         }
     }
-    if (PLAQ && MU == 3) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) P[c] = A[c];
+    if (!HYB) {
+        // tests trials t0 .. t0 + n - 1 (slots t & 3) of the waiting links
+        auto pick = [&](int t0, int n) {
+            for (int k = 0; k < n && wait; ++k) {
+                const Trial64 a = G.trial[(t0 + k) & 3][lane];
+                L = kp_lambda(KpSum{a.t, a.e}, d.inv, d.ei);
+                if (kp_accept(L, a.w3)) {
+                    tr = t0 + k + 1;
+                    wait = false;
+                }
+            }
+        };
+        if (act && role > 0 && role <= SPEC) draw(st, role, role);
+        __syncthreads();
+        pick(1, SPEC);
+        for (int t0 = 1 + SPEC; t0 < KP_CAP; t0 += 4) {
+            if (role == 0) {
+                const uint32_t m = __ballot_sync(0xffffffffu, wait);
+                if (lane == 0) G.pend = m;
+            }
+            __syncthreads();
+            const uint32_t m = G.pend;
+            if (m == 0) break;
+            if (((m >> lane) & 1u) && t0 + role < KP_CAP) draw(st, t0 + role, (t0 + role) & 3);
+            __syncthreads();
+            pick(t0, KP_CAP - t0 < 4 ? KP_CAP - t0 : 4);
+        }
     }
-    const Stream st = C.stream(key);
-    Drawn d;
-    double qc;
-    const bool haar = !fix_prepare<HYB>(C, A, &d, &qc);
-    bool done = !act || haar;
-    int32_t tr = -1;
-    Lambda L = {0, 0, 0};
-    uint32_t kd1 = 0, kd2 = 0;
-    for (int t0 = 0; t0 < KP_CAP; t0 += G) {
-        if (!__any_sync(0xffffffffu, !done)) break;
-        const U4 w = st.draw(TAG_TRIAL, (uint32_t)(t0 + g));
-        if (t0 == 0) {  // the direction: spare bits of trial 0 (lane g0)
-            kd1 = __shfl_sync(0xffffffffu, spare_bits_1(w), g0);
-            kd2 = __shfl_sync(0xffffffffu, spare_bits_2(w), g0);
-        }
-        Lambda M = {0, 0, 0};
-        const bool ok = !done && fix_try<HYB>(C, w, d.inv, d.ei, qc, &M);
-        const uint32_t m = (__ballot_sync(0xffffffffu, ok) >> g0) & ((1u << G) - 1u);
-        const int src = g0 + (m ? __ffs(m) - 1 : 0);
-        M.P = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)M.P, src);
-        M.lam = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)M.lam, src);
-        M.qe = __shfl_sync(0xffffffffu, M.qe, src);
-        if (!done && m) {
-            done = true;
-            tr = t0 + __ffs(m);
-            L = M;
-        }
+    if (role != 0) {
+        // one partial per warp: only the first of a group has plaquettes
+        if (PLAQ && lane == 0)
+            ctx.plaq_partial[((size_t)(MU - 1) * ctx.phase_blocks + blockIdx.x) * ctx.phase_wpb +
+                             (threadIdx.x >> 5)] = 0.0;
+        return;
     }
     int64_t plaq = 0;
     uint32_t ntrial = 0, ncap = 0;
-    if (act && g == 0) {
+    if (act) {
         int64_t un[4];
         if (haar) {
             const Quat<double> h = haar_link(st, C.tab);
             U.store(MU, p, i, h);
             if (PLAQ) fix_from_link(h, un);
-            tr = 0;
         } else if (tr > 0) {
-            new_link_fix(L, kd1, kd2, d.V, C.tab, un);
+            if (HYB) {
+                new_link_fix(L, kd1, kd2, d.V, C.tab, un);
+            } else {
+                const Dir64 f = G.dir[lane];
+                new_link_dir_fix(L, {f.cth, f.sth, f.cph, f.sph}, d.V, un);
+            }
             U.store(MU, p, i, dq_link(un));
         } else {
             ncap = 1;
             if (PLAQ) fix_from_link(U.load_rw(MU, p, i), un);
         }
         ntrial = tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
-        if (dbg) dbg[key >> 2] = tr;
+        if (dbg) dbg[lex] = tr;
         if (PLAQ) plaq = retr_fix(un, P);
     }
     __syncwarp();
-    fix_totals<MU, PLAQ>(ctx, l, blk0, Vh, PLAQ ? plaq_double(warp_sum64(plaq)) : 0.0, ntrial,
-                             ncap);
+    fix_totals<MU, PLAQ>(ctx, l, blk0, Vh, PLAQ ? plaq_double(warp_sum64(plaq)) : 0.0, ntrial, ncap);
 }
 
 }  // namespace su2

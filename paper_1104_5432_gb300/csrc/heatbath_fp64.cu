@@ -1,11 +1,11 @@
 // heatbath_fp64.cu -- the FP64 row of the launch-shape table: its 14 shapes run
-// five kernels (heatbath_fixed.cuh).  The build compiles this file once per
-// kernel and sampler, with SU2_KIND = 0 .. 4 and SU2_HYB = 0 or 1, so that
+// six kernels (heatbath_fixed.cuh).  The build compiles this file once per
+// kernel and sampler, with SU2_KIND = 0 .. 5 and SU2_HYB = 0 or 1, so that
 // they compile in parallel.
 #include "heatbath_fixed.cuh"
 
 #if !defined(SU2_KIND) || !defined(SU2_HYB)
-#error "compile with -DSU2_KIND=<0..4> -DSU2_HYB=<0|1>"
+#error "compile with -DSU2_KIND=<0..5> -DSU2_HYB=<0|1>"
 #endif
 
 namespace su2 {
@@ -18,8 +18,10 @@ static void launch_fix_k(const Ctx& c, const LaunchCfg& f, int parity, int32_t* 
         fix_phase_kernel<MU, PLAQ, HYB, MIR, 256, 1><<<grid, block, 0, s>>>(c, parity, dbg);
     else if constexpr (KIND == FIX_LINK_96)
         fix_phase_kernel<MU, PLAQ, HYB, MIR, 128, 5><<<grid, block, 0, s>>>(c, parity, dbg);
-    else if constexpr (KIND == FIX_COOP)
-        fix_coop_kernel<MU, PLAQ, HYB, MIR><<<grid, block, 0, s>>>(c, parity, dbg);
+    else if constexpr (KIND == FIX_QUAD_128)
+        fix_quad_kernel<MU, PLAQ, HYB, MIR, 4><<<grid, block, 0, s>>>(c, parity, dbg);
+    else if constexpr (KIND == FIX_QUAD_72)
+        fix_quad_kernel<MU, PLAQ, HYB, MIR, 7><<<grid, block, 0, s>>>(c, parity, dbg);
     else
         fix_queue_kernel<MU, PLAQ, HYB, MIR, KIND == FIX_PERSIST>
             <<<grid, block, 0, s>>>(c, parity, f.rounds, dbg);

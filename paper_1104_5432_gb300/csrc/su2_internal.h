@@ -36,10 +36,9 @@ constexpr int TPB = 256;            // threads per block of the non-phase kernel
 // persistent (single-lattice handles): only the blocks that fit on the GPU
 // at once are launched, and each walks tiles of R rounds in grid-stride
 // order, so its retry queue carries over from tile to tile and drains once.
-// group (FP64): lanes per link; above 1 the cooperative kernel runs, whose
-// G lanes share one link's staple terms and try several Kennedy-Pendleton
-// trials at once (small lattices, where the FP64 work of few links per warp
-// sets the time).
+// group (FP64): threads per link; above 1 fix_quad_kernel runs, four warps of
+// a block sharing 32 links' staple terms and trials (small lattices, where one
+// link's chain of instructions sets the time).
 // stage (FP32 queued kernel, lattices with Nh = 32): each round one lane
 // brings the 18 neighbour rows of the warp's 32 sites into shared memory
 // with bulk copies (cp.async.bulk behind an mbarrier), and the lanes read
@@ -67,7 +66,7 @@ constexpr LaunchCfg LAUNCH_CFG[NUM_ROWS][NUM_LAUNCH_CFG] = {
     {{256, 1, false, 1, false}, {128, 4, false, 1, false}, {64, 8, false, 1, false},
      {64, 4, false, 1, false}, {32, 16, false, 1, false}, {32, 8, false, 1, false},
      {32, 16, false, 2, false}, {32, 16, false, 4, false}, {32, 16, false, 8, false},
-     {32, 16, false, 16, false}, {64, 8, false, 1, false, 8}, {32, 16, false, 1, false, 8},
+     {32, 16, false, 16, false}, {128, 4, false, 1, false, 4}, {128, 7, false, 1, false, 4},
      {32, 16, false, 2, true}, {32, 16, false, 8, true}},
     // FP32 site pairs: one thread updates two links (t and t + Nt/2) per
     // round with packed two-lane arithmetic; `rounds` counts pairs
@@ -80,12 +79,20 @@ constexpr LaunchCfg LAUNCH_CFG[NUM_ROWS][NUM_LAUNCH_CFG] = {
 static_assert(NUM_LAUNCH_CFG % 2 == 0, "shapes compile in pairs");
 // The kernels the FP64 row's shapes run: one link per thread with up to 255 or
 // 96 registers a thread (the same kernel in blocks of 256, 64 or 32 and of 128,
-// 64 or 32 threads), eight lanes per link, R links per thread with a retry
-// queue, and the same persistent.
-enum FixKind { FIX_LINK_255, FIX_LINK_96, FIX_COOP, FIX_QUEUE, FIX_PERSIST, NUM_FIX_KINDS };
+// 64 or 32 threads), four threads per link with up to 128 or 72 registers, R
+// links per thread with a retry queue, and the same persistent.
+enum FixKind {
+    FIX_LINK_255,
+    FIX_LINK_96,
+    FIX_QUAD_128,
+    FIX_QUAD_72,
+    FIX_QUEUE,
+    FIX_PERSIST,
+    NUM_FIX_KINDS
+};
 constexpr FixKind fix_kind(const LaunchCfg& f)
 {
-    return f.group > 1 ? FIX_COOP
+    return f.group > 1 ? (f.min_blocks > 4 ? FIX_QUAD_72 : FIX_QUAD_128)
            : f.persistent ? FIX_PERSIST
            : f.rounds > 1 ? FIX_QUEUE
            : f.threads * f.min_blocks <= 256 ? FIX_LINK_255

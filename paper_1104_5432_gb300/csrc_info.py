@@ -2,8 +2,8 @@
 csrc/su2_internal.h), for reporting which one the autotuner chose.
 Entries: (threads per block, minimum blocks per SM, y-slab walk, links per
 thread, persistent: on a single lattice only the blocks that fit on the GPU
-at once are launched and each walks several tiles[, lanes per link of the
-cooperative FP64 kernel[, neighbour rows staged in shared memory by bulk
+at once are launched and each walks several tiles[, threads per link of the
+FP64 kernel for small lattices[, neighbour rows staged in shared memory by bulk
 copies]])."""
 
 _F32 = [(256, 4, False, 1, False), (128, 8, False, 1, False), (64, 16, False, 1, False),
@@ -14,7 +14,7 @@ _F32 = [(256, 4, False, 1, False), (128, 8, False, 1, False), (64, 16, False, 1,
 _F64 = [(256, 1, False, 1, False), (128, 4, False, 1, False), (64, 8, False, 1, False),
         (64, 4, False, 1, False), (32, 16, False, 1, False), (32, 8, False, 1, False),
         (32, 16, False, 2, False), (32, 16, False, 4, False), (32, 16, False, 8, False),
-        (32, 16, False, 16, False), (64, 8, False, 1, False, 8), (32, 16, False, 1, False, 8),
+        (32, 16, False, 16, False), (128, 4, False, 1, False, 4), (128, 7, False, 1, False, 4),
         (32, 16, False, 2, True), (32, 16, False, 8, True)]
 
 
@@ -58,7 +58,7 @@ def launch_shapes(row):
                    + (", packed FP32x2" if pairs else "")
                    + (", retry queue" if r > 1 or ps or pairs else "")
                    + (", persistent" if ps else "")
-                   + (f", {g} lanes per link (staple terms and trials in parallel)" if g > 1
+                   + (f", {g} threads per link (staple terms and trials in parallel)" if g > 1
                       else "")
                    + (", neighbour rows staged by bulk copies" if stage else ""))
     return out

@@ -908,6 +908,39 @@ def test_persistent_shapes_walk_several_tiles(dtype, layout, persistent, plain):
     np.testing.assert_allclose(pb, pa, rtol=0, atol=1e-13 if dtype == su2.F64 else 1e-7)
 
 
+@pytest.mark.parametrize("cfg", [10, 11])
+@pytest.mark.parametrize("shapes,beta", [
+    (((2, 2), (6, 2), (10, 4), (4, 6)), 2.4),  # tiles of 8, 8, 32 and 0 links at the end
+    # several rounds of four; acceptance ~ alpha^(3/2), so a link of |A| = 0.1 still accepts
+    # one trial in 200 and the cap of 4096 is out of reach
+    (((8, 8), (2, 4)), 0.3),
+    (((4, 4),), 0.0),                          # every link takes the Haar branch
+    (((4, 2),), 1e-9)])                        # every link runs to the trial cap
+def test_four_threads_per_link_match_one_thread(cfg, shapes, beta):
+    """The staple sum is a sum of integers and a link's trials keep their
+    order, so both kernels give the same bits, trial counts and caps."""
+    out = []
+    for c in (0, cfg):
+        B = su2.Lattice([s[0] for s in shapes], [s[1] for s in shapes], su2.F64)
+        B.set_launch_config(c)
+        n = range(len(shapes))
+        B.batch_init(su2.HOT, [5 + k for k in n])
+        if len(shapes) == 1 and shapes[0] == (4, 2):
+            B.batch_heatbath([beta], 1, [3], plaq=None)
+            with pytest.raises(su2.SU2Error):
+                B.sync()
+            plaq = np.zeros(1)
+        else:
+            plaq = B.batch_heatbath([beta] * len(shapes), 2, [3 + k for k in n])
+        out.append(([B.get_links(l) for l in n], [B.stats(l) for l in n], plaq))
+        B.close()
+    for k in range(len(shapes)):
+        np.testing.assert_array_equal(out[1][0][k], out[0][0][k])
+    assert out[1][1] == out[0][1]
+    # the same integers summed in groups of 32 links
+    np.testing.assert_allclose(out[1][2], out[0][2], rtol=0, atol=1e-14)
+
+
 @pytest.mark.parametrize("dtype,layout,cfg", [(su2.F32, su2.LAYOUT_PLAIN, 8),
                                               (su2.F32, su2.LAYOUT_PAIRS, 8),
                                               (su2.F32, su2.LAYOUT_PAIRS, 0), (su2.F64, None, 9)])
