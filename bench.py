@@ -165,15 +165,18 @@ def recorded_traffic(kernel_key, field="dram_bytes_per_launch_full_size"):
     return ent.get(field)
 
 
-# FP64 arithmetic of one link update (the FP64 arm is bound by GB300's FP64
-# units, not by memory): algorithmic flops outside the math functions --
+# FP64 arithmetic of one link update, if it ran on GB300's FP64 units: the
+# kernels do it in 64-bit fixed point on the integer pipes, so `frac` says
+# how many times faster than that bound they are.  Algorithmic flops outside
+# the math functions --
 # 12 quaternion products (336), staple additions (20), k (8), alpha and
 # 1/(2 alpha) (5), per Kennedy-Pendleton trial 10, the direction, X Vhat^+
 # and the renormalisation (~40) -- and the math-function calls the update
 # makes: per trial 2 log + 1 cospi (lambda^2), and once 2 rsqrt (1/k, the
 # renormalisation), 2 sqrt (sin theta, |vector part|), 1 sincospi (phi).
-# Each at the measured rate of the routine the kernels call (the logarithm,
-# the cosine and the sine + cosine are their own table-driven ones).
+# Each at the measured rate of the routine the FP64 sequence calls (the
+# logarithm, the cosine and the sine + cosine are its own table-driven ones;
+# lattices with non-unit links run it).
 FP64_FLOPS_FIXED, FP64_FLOPS_PER_TRIAL = 420.0, 10.0
 FP64_CALLS = {"log": (0, 2), "cospi": (0, 1), "sincospi": (1, 0), "sqrt": (2, 0),
               "rsqrt": (2, 0)}  # (per update, per trial)
@@ -185,7 +188,7 @@ def fp64_roofline(su2, ups, trials_per_update):
     function, calls / its measured call rate.  peak = 1 / that time."""
     t = trials_per_update
     fma = su2.probe_fma_rate(su2.F64)
-    # the routines the FP64 kernels call: their table-driven logarithm,
+    # the routines the FP64 sequence calls: its table-driven logarithm,
     # cosine and sine + cosine, CUDA's sqrt and rsqrt
     ids = {"log": su2.PROBE_LN_TABLE, "cospi": su2.PROBE_COS_TABLE,
            "sincospi": su2.PROBE_SINCOS_TABLE, "sqrt": su2.PROBE_SQRT, "rsqrt": su2.PROBE_RSQRT}
@@ -201,7 +204,8 @@ def fp64_roofline(su2, ups, trials_per_update):
             "frac": round(ups * T, 4), "traffic": None,
             "peak_kind": "measured here: algorithmic FP64 work per update over the DFMA-chain "
                          "rate (su2_probe_fma_rate) and each math function's call rate "
-                         "(su2_probe_special_rate)",
+                         "(su2_probe_special_rate); the kernels compute in 64-bit fixed point "
+                         "on the integer pipes, so frac exceeds 1",
             "trials_per_update": round(t, 5),
             "algorithmic_flops_per_update": round(flops, 2),
             "fma_per_s": fma, "calls_per_s": {k: round(v, 0) for k, v in rates.items()},
@@ -411,6 +415,10 @@ def gpu_arm(args, rank, world, local):
         arms["fp64_plain"] = {"value": v64, "unit": UNIT,
                               "roofline": fp64_roofline(su2, v64 / world,
                                                         st64["trials"] / st64["updates"]),
+                              "roofline_hbm": {
+                                  "bound": "hbm", "unit": "GB/s", "peak": hbm,
+                                  "achieved": round(v64 / world * BYTES_PER_UPDATE["f64"] / 1e9, 1),
+                                  "frac": round(v64 / world * BYTES_PER_UPDATE["f64"] / 1e9 / hbm, 4)},
                               "workload": workload_name("FP64 throughout").replace(
                                   f"{sweeps} checkerboard", f"{sw64} checkerboard"),
                               "ms_per_sweep": t64 / sw64 * 1e3}
