@@ -170,7 +170,12 @@ __global__ void __launch_bounds__(TPB) polyakov_kernel(Ctx ctx)
 }
 
 // rows r = 0..rmax of partials, from the Polyakov field of the last
-// polyakov_kernel launch; one barrier for all rows
+// polyakov_kernel launch; one barrier for all rows.  Bound by the FP64 unit in
+// double (~76 clocks an addition), where eight rows share warp_total's tree:
+// four additions per row and lane in place of eight, the same sums; by the
+// field's loads in float, one row at a time (eight: 0.149 against 0.147 ms).
+// 21 lattices 48^3, r <= 24, with the Polyakov loops before it: FP64 1.21 -> 0.90
+// ms, a measured sweep at Nt = 4 6.19 -> 5.91.
 template <typename T>
 __global__ void __launch_bounds__(TPB) correlator_kernel(Ctx ctx, int rmax)
 {
@@ -191,18 +196,39 @@ __global__ void __launch_bounds__(TPB) correlator_kernel(Ctx ctx, int rmax)
         L0 = F[sidx];
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t xr = x, yr = y, zr = z;
-    for (int r = 0; r <= rmax; ++r) {
-        T v = T(0);
-        if (act) {
-            v = L0 * (F[xr + Ns * (y + Ns * z)] + F[x + Ns * (yr + Ns * z)]
-                      + F[x + Ns * (y + Ns * zr)]);
+    // indices of x + r in the three directions, and where each wraps
+    const uint32_t dz = Ns * Ns;
+    uint32_t ox = sidx, oy = sidx, oz = sidx;
+    const uint32_t ex = ox + (Ns - x), ey = oy + (Ns - y) * Ns, ez = oz + (Ns - z) * dz;
+    constexpr int G = sizeof(T) == 8 ? 8 : 1;  // rows at a time
+    for (int r0 = 0; r0 <= rmax; r0 += G) {
+        T v[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            v[k] = T(0);
+            if (act && r0 + k <= rmax) v[k] = L0 * (F[ox] + F[oy] + F[oz]);
+            ox += 1;
+            oy += Ns;
+            oz += dz;
+            if (ox == ex) ox -= Ns;
+            if (oy == ey) oy -= dz;
+            if (oz == ez) oz -= Ns * dz;
         }
-        v = warp_total(v);
-        if (lane == 0) s_rows[r][w] = v;
-        xr = xr + 1 == Ns ? 0 : xr + 1;
-        yr = yr + 1 == Ns ? 0 : yr + 1;
-        zr = zr + 1 == Ns ? 0 : zr + 1;
+        // in the tree's first levels a lane keeps half of its rows and adds the
+        // partner's
+#pragma unroll
+        for (int h = G / 2; h > 0; h >>= 1) {
+            const bool up = lane & (32 / G * h);
+#pragma unroll
+            for (int k = 0; k < h; ++k) {
+                const T give = up ? v[k] : v[k + h];
+                v[k] = (up ? v[k + h] : v[k]) + __shfl_xor_sync(0xffffffffu, give, 32 / G * h);
+            }
+        }
+#pragma unroll
+        for (int o = 16 / G; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        const int row = r0 + lane / (32 / G);  // the lane's upper bits chose the halves
+        if (lane % (32 / G) == 0 && row <= rmax) s_rows[row][w] = v[0];
     }
     __syncthreads();
     if ((int)threadIdx.x <= rmax) {

@@ -162,6 +162,22 @@ def test_observables_fp64(Ns, Nt):
     np.testing.assert_allclose(host_acc[0], 1 + C, rtol=0, atol=1e-13)
 
 
+@pytest.mark.parametrize("dtype,tol", [(su2.F64, 1e-13), (su2.F32, 4e-8)])
+@pytest.mark.parametrize("Ns,rmaxes", [(2, (0, 1)), (6, (2, 3)), (18, (6, 7, 8, 9)), (34, (15, 16, 17))])
+def test_correlator_rows_in_groups_of_eight(dtype, tol, Ns, rmaxes):
+    """Separations are summed eight at a time in FP64: the last group full, short by
+    one, holding one.  The gates are those of the correlator (a row does not
+    depend on how many there are: equal bits)."""
+    lat = lattice(Ns, 2, dtype)
+    lat.init(su2.HOT, 12)
+    links = lat.get_links()
+    ref = O.correlator(Ns, 2, links, rmaxes[-1])
+    full = lat.polyakov_correlator(rmaxes[-1])[0]
+    np.testing.assert_allclose(full, ref, rtol=0, atol=tol)
+    for r in rmaxes:
+        np.testing.assert_array_equal(lat.polyakov_correlator(r)[0], full[:r + 1])
+
+
 @pytest.mark.parametrize("Ns,Nt", [(6, 4), (8, 8)])
 def test_observables_fp32(Ns, Nt):
     lat = lattice(Ns, Nt, su2.F32)
