@@ -665,9 +665,20 @@ int heatbath_impl(su2_lattice* L, const double* betas, double beta, int nsweeps,
                 if (host) memcpy(plaq + done, host, sizeof(double) * chunk);
                 return rc;
             }
-            SU2_CUDA(cudaMemcpy2DAsync(plaq + done, sizeof(double) * nsweeps, L->ring_dev(),
-                                       sizeof(double) * PLAQ_RING, sizeof(double) * chunk, L->n,
-                                       cudaMemcpyDeviceToHost, L->stream));
+            // one pitched copy when its rows fill the caller's buffer; a pitched
+            // copy of part of the sweeps would span a whole pitch past its last
+            // row, beyond the buffer's end
+            if (chunk == nsweeps) {
+                SU2_CUDA(cudaMemcpy2DAsync(plaq, sizeof(double) * nsweeps, L->ring_dev(),
+                                           sizeof(double) * PLAQ_RING, sizeof(double) * chunk, L->n,
+                                           cudaMemcpyDeviceToHost, L->stream));
+            } else {
+                for (int l = 0; l < L->n; ++l)
+                    SU2_CUDA(cudaMemcpyAsync(plaq + (size_t)l * nsweeps + done,
+                                             L->ring_dev() + (size_t)l * PLAQ_RING,
+                                             sizeof(double) * chunk, cudaMemcpyDeviceToHost,
+                                             L->stream));
+            }
         }
         done += chunk;
     }

@@ -162,6 +162,25 @@ def test_observables_fp64(Ns, Nt):
     np.testing.assert_allclose(host_acc[0], 1 + C, rtol=0, atol=1e-13)
 
 
+@pytest.mark.parametrize("n,nsweeps", [(1, 4096), (1, 9000), (3, 4096), (3, 4097), (3, 40)])
+def test_host_plaquettes_stay_inside_the_buffer(n, nsweeps):
+    """Plaquettes reach the host in chunks of 4096 sweeps: every chunk lands
+    in its place, nothing is written past the last value, and the values are
+    those of a device buffer."""
+    out = []
+    for dev in (True, False):
+        B = su2.Lattice([2] * n, [2] * n, su2.F32)
+        B.batch_init(su2.HOT, list(range(1, n + 1)))
+        buf = np.full(n * nsweeps + 20000, -7.0)
+        dst = torch.zeros(n * nsweeps, dtype=torch.float64, device="cuda") if dev else buf[:n * nsweeps]
+        B.batch_heatbath([2.3] * n, nsweeps, list(range(5, 5 + n)), plaq=dst)
+        torch.cuda.synchronize()
+        out.append(dst.cpu().numpy() if dev else dst.copy())
+        assert np.all(buf[0 if dev else n * nsweeps:] == -7.0)
+        B.close()
+    np.testing.assert_array_equal(out[1], out[0])
+
+
 @pytest.mark.parametrize("dtype,tol", [(su2.F64, 1e-13), (su2.F32, 4e-8)])
 @pytest.mark.parametrize("Ns,rmaxes", [(2, (0, 1)), (6, (2, 3)), (18, (6, 7, 8, 9)), (34, (15, 16, 17))])
 def test_correlator_rows_in_groups_of_eight(dtype, tol, Ns, rmaxes):
