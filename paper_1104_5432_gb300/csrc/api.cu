@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -536,7 +537,11 @@ int fetch_status(su2_lattice* L, const double* src, size_t bytes, const double**
 {
     static thread_local std::vector<char> buf;
     const size_t at = (size_t)(reinterpret_cast<const char*>(src) - (L->work + L->off_status));
-    buf.resize(at + bytes);
+    try {
+        buf.resize(at + bytes);
+    } catch (const std::bad_alloc&) {
+        return fail(SU2_E_NOMEM, "no host memory for the results");
+    }
     SU2_CUDA(cudaMemcpyAsync(buf.data(), L->work + L->off_status, at + bytes, cudaMemcpyDeviceToHost,
                              L->stream));
     SU2_CUDA(cudaStreamSynchronize(L->stream));
