@@ -446,18 +446,18 @@ bool chain_geometry(uint32_t Vh, int S, ChainGeom* g)
     return 3 * g->npart <= (uint32_t)SWEEP_CHUNK;
 }
 
-static void* chain_kernel(const ChainGeom& g)
+static_assert(chain_smem(512, SWEEP_CHUNK / 3) + 64 <= 227 * 1024, "the largest geometry fits an SM");
+
+static const void* chain_kernel(const ChainGeom& g)
 {
-    return g.updaters == 128   ? (void*)hb_chain_kernel<128>
-           : g.updaters == 256 ? (void*)hb_chain_kernel<256>
-                               : (void*)hb_chain_kernel<512>;
+    return g.updaters == 128   ? (const void*)hb_chain_kernel<128>
+           : g.updaters == 256 ? (const void*)hb_chain_kernel<256>
+                               : (const void*)hb_chain_kernel<512>;
 }
 static cudaError_t chain_config(const ChainGeom& g, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at)
 {
-    void* k = chain_kernel(g);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    const cudaError_t e = allow_cluster(
+        chain_kernel(g), chain_smem((uint32_t)g.updaters, (uint32_t)SWEEP_CHUNK / 3));
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3((unsigned)g.S);
     cfg->blockDim = dim3((unsigned)(2 * g.updaters));
@@ -498,19 +498,27 @@ cudaError_t launch_chain(const Ctx& c, const ChainGeom& g, bool plaq, int nsweep
     return cudaLaunchKernelEx(&cfg, hb_chain_kernel<512>, c, g.C, g.div_c, g.npart, pl, nsweeps);
 }
 
+// dynamic shared memory of a CTA of the current device beside the whole-sweep
+// kernel's static part (warp and CTA partials); 0 if unknown
+static size_t cluster_room()
+{
+    int max_smem = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return (size_t)max_smem - 8 * (1024 / 32) - 8 * CLUSTER_MAX;
+}
+
 // cluster size and shared memory for lattice 0, or false when the lattice
 // does not fit: the largest S in {16, 8, 4, 2} dividing Vh whose share of
 // the links fits a CTA
 bool cluster_geometry(uint32_t Vh, int dtype_f32, int n, ClusterGeom* g)
 {
     if (!dtype_f32 || n != 1) return false;
-    int max_smem = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-            cudaSuccess)
-        return false;
-    // static shared memory of the kernel: warp and CTA partials
-    const size_t room = (size_t)max_smem - 8 * (1024 / 32) - 8 * CLUSTER_MAX;
+    const size_t room = cluster_room();
     for (int S = CLUSTER_MAX; S >= 2; S /= 2) {
         if (Vh % (uint32_t)S) continue;
         const uint32_t C = Vh / (uint32_t)S;
@@ -529,10 +537,7 @@ template <bool HYB, int NT>
 static cudaError_t launch_cluster_nt(const Ctx& c, const ClusterGeom& g, bool plaq, cudaStream_t s)
 {
     auto k = hb_cluster_kernel<HYB, NT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
-    if (e != cudaSuccess) return e;
+    if (cudaError_t e = allow_cluster((const void*)k, cluster_room())) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g.S);
     cfg.blockDim = dim3(NT);
@@ -562,9 +567,7 @@ cudaError_t launch_cluster_sweep(const Ctx& c, const ClusterGeom& g, bool plaq, 
 bool cluster_launchable(const ClusterGeom& g)
 {
     auto k = g.threads == 128 ? hb_cluster_kernel<false, 128> : hb_cluster_kernel<false, 1024>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) !=
-            cudaSuccess) {
+    if (allow_cluster((const void*)k, cluster_room()) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }

@@ -16,6 +16,18 @@ __device__ __forceinline__ void cluster_sync()
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Lets kernel k run in clusters of 16 CTAs of up to max_smem bytes of dynamic
+// shared memory.  The limits belong to the kernel, not to a launch: max_smem
+// is the most any lattice asks of k, one value for all of them, so that a
+// host thread of another lattice never lowers the limit under a launch.
+inline cudaError_t allow_cluster(const void* k, size_t max_smem)
+{
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e != cudaSuccess
+               ? e
+               : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
+}
+
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;

@@ -347,13 +347,13 @@ bool chain64_geometry(uint32_t Vh, ChainGeom* g)
     return 3 * g->npart <= (uint32_t)SWEEP_CHUNK;
 }
 
+static_assert(chain64_smem(C64_LINKS, SWEEP_CHUNK / 3) + 128 <= 227 * 1024, "the largest geometry fits an SM");
+
 static cudaError_t chain64_config(const ChainGeom& g, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(fix_chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fix_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)g.smem);
+    const cudaError_t e =
+        allow_cluster((const void*)fix_chain_kernel,
+                      chain64_smem((uint32_t)C64_LINKS, (uint32_t)SWEEP_CHUNK / 3));
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3((unsigned)g.S);
     cfg->blockDim = dim3((unsigned)(4 * C64_LINKS));

@@ -1253,6 +1253,47 @@ def test_one_launch_chain_matches_the_phase_launches(dtype, Ns, Nt):
         np.testing.assert_array_equal(lat.get_links(), before)
 
 
+@pytest.mark.parametrize("dtype,big", [(su2.F32, (16, 4)), (su2.F64, (8, 8))])
+def test_small_lattices_from_two_host_threads(dtype, big):
+    """Two host threads sweep lattices of different size through the same
+    one-launch kernel (FP32 16^3 x 4 and 12^3 x 8, 512 links a CTA and 432; FP64
+    8^4 and 4^4), each on its own stream: neither thread's launch changes what
+    the other's may ask of the kernel, so every call succeeds, and both chains
+    end where they end alone."""
+    import threading
+    small = (4, 4) if dtype == su2.F64 else (12, 8)
+    ncall = 3000
+    runs = [(big, 1), (small, 2)]
+
+    def run(shape, seed, stream, errors):
+        try:
+            lat = su2.Lattice(shape[0], shape[1], dtype, stream=stream)
+            lat.init(su2.HOT, seed)
+            for _ in range(ncall):
+                lat.heatbath(2.3, 1, seed, plaq=None)
+            lat.sync()
+            return lat.get_links(), lat.stats()
+        except su2.SU2Error as e:
+            errors.append(str(e))
+
+    errors, got = [], [None, None]
+    streams = [torch.cuda.Stream() for _ in runs]
+
+    def worker(k):
+        got[k] = run(*runs[k], streams[k], errors)
+
+    ts = [threading.Thread(target=worker, args=(k,)) for k in range(2)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not errors, errors
+    for k in range(2):
+        links, stats = run(*runs[k], streams[k], errors)
+        np.testing.assert_array_equal(got[k][0], links)
+        assert got[k][1] == stats
+
+
 @pytest.mark.parametrize("shape", [0, 7])
 def test_lattice_beyond_32_bit_link_offsets(shape):
     """128^3 x 258 FP32 (2^29 + 2^22 sites, 35 GB of links): a (mu, parity)
