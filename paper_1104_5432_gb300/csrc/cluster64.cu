@@ -18,8 +18,9 @@
 // and the plaquette partials are summed in launch shape 0's order: links and
 // plaquettes are those of the phase launches bit by bit.
 //
-// A lattice with non-unit links (D.nonunit) runs its sweeps in the FP64
-// sequence here, through L2, until all links are unit quaternions.
+// A lattice with non-unit links (D.general) runs its sweeps in the FP64
+// sequence here, through L2, until all links are unit quaternions; one at a
+// coupling above FIX_BETA_MAX runs all of them so.
 #include "cluster.cuh"
 #include "heatbath_fixed.cuh"
 
@@ -146,7 +147,7 @@ fix_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int
 
     // sweeps in the FP64 sequence while some link is not a unit quaternion
     int k = 0;
-    for (bool nonunit = D.nonunit != 0; nonunit && k < nsweeps; ++k) {
+    for (bool general = D.general != 0; general && k < nsweeps; ++k) {
         LatDesc Dk = D;
         Dk.sweep = sw0 + (uint64_t)k;
         for (int ph = 0; ph < 8; ++ph) {
@@ -165,8 +166,8 @@ fix_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int
             __threadfence();
             cluster_sync();
         }
-        bool ok = true;
-        if (role == 0 && act)
+        bool ok = (D.general & GENERAL_BETA) == 0;
+        if (ok && role == 0 && act)
             for (int mp = 0; mp < 8; ++mp) {
                 const Quat<double> q = G.load_rw(mp >> 1, mp & 1, i);  // this thread's own stores
                 if (!unit_link(make_double2(q.a0, q.a1), make_double2(q.a2, q.a3))) ok = false;
@@ -182,10 +183,10 @@ fix_chain_kernel(Ctx ctx, uint32_t C, FastDiv div_c, uint32_t npart, int pl, int
         }
         cluster_sync();
         if (pl && rank == 0 && threadIdx.x == 0) finish_sum(k);
-        nonunit = false;
-        for (uint32_t r = 0; r < S; ++r) nonunit = nonunit || bad[r] != 0;
+        general = false;
+        for (uint32_t r = 0; r < S; ++r) general = general || bad[r] != 0;
         cluster_sync();  // bad[] and scratch may be written again
-        if (!nonunit && rank == 0 && threadIdx.x == 0) Dw->nonunit = 0u;
+        if (!general && rank == 0 && threadIdx.x == 0) Dw->general = 0u;
     }
 
     const int k0 = k;  // sweeps k0 .. nsweeps - 1 in fixed point

@@ -34,7 +34,8 @@ __global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx, bool mirror)
     const int l = lattice_of_block(ctx.site_start, ctx.n, blockIdx.x);
     LatDesc* D = ctx.desc + l;
     const uint32_t eo = (blockIdx.x - first_block(ctx.site_start, l)) * TPB + threadIdx.x;
-    if (eo < D->Vh && !unit_links_at(ctx, *D, eo, mirror)) D->nonunit = 1u;
+    if (D->general & GENERAL_BETA) return;
+    if (eo < D->Vh && !unit_links_at(ctx, *D, eo, mirror)) D->general = GENERAL_LINKS;
 }
 
 // the same by one block, after a sweep of a lattice that failed the check:
@@ -44,7 +45,7 @@ __device__ void unit_recheck(const Ctx& ctx, LatDesc* D)
     bool ok = true;
     for (uint32_t eo = threadIdx.x; eo < D->Vh; eo += TPB)
         if (!unit_links_at(ctx, *D, eo, ctx.mirror != nullptr)) ok = false;
-    if (__syncthreads_and(ok) && threadIdx.x == 0) D->nonunit = 0u;
+    if (__syncthreads_and(ok) && threadIdx.x == 0) D->general = 0u;
 }
 
 // Finishes a sweep: the fixed-order sum of the fused plaquette partials and
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
     LatDesc* D = ctx.desc + l;
     if (!PLAQ) {
         if (blockIdx.x == 0 && threadIdx.x == 0) D->sweep += 1;
-        if (F64 && D->nonunit) unit_recheck(ctx, D);
+        if (F64 && D->general == GENERAL_LINKS) unit_recheck(ctx, D);
         return;
     }
     // partials are per warp: lattice l owns warps [b0, b0 + nb) of each slot
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
         if (D->plaq_out) D->plaq_out[k] = P;
         D->sweep += 1;
     }
-    if (F64 && D->nonunit) unit_recheck(ctx, D);
+    if (F64 && D->general == GENERAL_LINKS) unit_recheck(ctx, D);
 }
 
 // Per-call parameters go in by value (no host-to-device copy); the
@@ -117,7 +118,7 @@ __global__ void set_params_kernel(Ctx ctx, ParamChunk pc)
     D->half_inv_beta = 0.5 / pc.beta[j];  // inf at beta = 0, where the Haar draw applies
     D->seed = pc.seed[j];
     D->plaq_out = pc.plaq_out[j];
-    D->nonunit = 0u;
+    D->general = pc.beta[j] > FIX_BETA_MAX ? GENERAL_BETA : 0u;
     D->sweep_base = D->sweep;
 }
 

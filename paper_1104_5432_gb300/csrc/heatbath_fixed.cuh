@@ -17,8 +17,9 @@
 //
 // The fixed-point ranges hold for unit links.  unit_check_kernel looks at
 // every link before the sweeps of a call and sweep_end_kernel again after
-// each sweep of a lattice that failed; such a lattice (D.nonunit) takes the
-// FP64 sequence, one link per thread, in the same kernels.
+// each sweep of a lattice that failed; such a lattice, and one at a coupling
+// above FIX_BETA_MAX (D.general), takes the FP64 sequence, one link per
+// thread, in the same kernels.
 #pragma once
 #include "heatbath_kernel.cuh"
 #include "su2_mirror.cuh"
@@ -186,7 +187,7 @@ __device__ __forceinline__ double plaq_double(int64_t v)  // v 2^-51
 }
 
 // ---------------------------------------------------------------------------
-// lattices with non-unit links: the FP64 sequence
+// lattices with non-unit links or a large coupling: the FP64 sequence
 // ---------------------------------------------------------------------------
 // Staple sum by the tree s_k = up_k + lo_k for the k-th nu != mu,
 // A = (s_0 + s_1) + s_2 (P = its prefix over nu < mu), FP64 draw, new link.
@@ -248,7 +249,7 @@ fix_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const uint32_t Vh = D.Vh;
     const uint32_t blk0 = first_block(ctx.phase_start, l);
     const uint32_t i = (blockIdx.x - blk0) * blockDim.x + threadIdx.x;
-    if (D.nonunit) {
+    if (D.general) {
         general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, i < Vh ? i + 1 : i, p, HYB, dbg);
         return;
     }
@@ -342,7 +343,7 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
     // tiles of 32 R positions; a persistent block takes every nb-th
     const uint32_t nb = PERSIST ? __ldg(ctx.phase_start + l + 1) - blk0 : 0u;
     const uint32_t tile0 = blockIdx.x - blk0;
-    if (D.nonunit) {
+    if (D.general) {
         if (PERSIST) {
             general_links<MU, PLAQ>(ctx, l, blk0, tile0 * NT + threadIdx.x, nb * NT, Vh, p, HYB, dbg);
         } else {
@@ -518,7 +519,7 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
     const uint32_t i = (blockIdx.x - blk0) * 32u + (uint32_t)lane;
     const bool act = i < Vh;
-    if (D.nonunit) {
+    if (D.general) {
         general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, act && role == 0 ? i + 1 : i, p, HYB, dbg);
         return;
     }

@@ -16,9 +16,14 @@
 // Precision: the links enter at 2^-61, the staple sum is kept at 2^-55 (an
 // FP64 sum of the same size rounds to 2^-51) with one rounding per staple,
 // the unit staple and the draw at 2^-57 .. 2^-62, the new link at 2^-60, and
-// it is rounded once, to nearest, to the double that is stored.  The errors
-// against 128-bit arithmetic are below those of the FP64 sequence
-// (tests/test_fixed_point.py).
+// it is rounded once, to nearest, to the double that is stored.  These are
+// absolute errors, where a double's shrink with its value, and the vector part
+// of a link at coupling beta is of the size of beta^-1/2: its rms error
+// against extended precision is 0.2 of the FP64 sequence's at beta = 2.3, 0.36
+// to 0.49 at 64, the same from about 300 on and 12 to 15 times larger at 10^5
+// (tests/test_fixed_point.py).  So lattices at couplings above FIX_BETA_MAX
+// take the FP64 sequence (general_link), at its speed: beta = 1000, us a
+// sweep, 16^4 216, 32^4 2558, 64^4 39800 (fixed point 80, 596, 8650).
 //
 // Range: |sum of four h l'| <= |h|_1 2^31, and |h|_1 <= 2 |h|_2 for four
 // components, so with unit quaternions at 2^61 (h <= 2^29) the two cross
@@ -43,6 +48,7 @@
 namespace su2 {
 
 constexpr double UNIT_TOLERANCE = 1.0 / 1024.0;
+constexpr double FIX_BETA_MAX = 64.0;
 
 // the tables (filled on the host): 512 intervals of the logarithm's argument
 // and 1024 points of the circle, 16 bytes each

@@ -111,6 +111,10 @@ constexpr uint32_t STATUS_STAGE = 4u;   // a bulk copy of neighbour rows did not
 constexpr int SWEEP_CHUNK = TPB * 8;   // plaquette partials summed per sweep_end block
 constexpr int MAX_RMAX = 128;          // largest correlator separation
 constexpr int TRIAL_SLOTS = 64;        // per-lattice trial counters (spread atomics)
+// reasons for an FP64 lattice to take the FP64 sequence: some link is not a
+// unit quaternion (unit_check_kernel, looked at again after each sweep), the
+// coupling is above FIX_BETA_MAX (set_params_kernel, for the whole call)
+constexpr uint32_t GENERAL_LINKS = 1u, GENERAL_BETA = 2u;
 
 // One per lattice, resident in the work buffer.  The first block is fixed
 // at bind time; the second is written by the parameter kernel at every
@@ -139,7 +143,7 @@ struct LatDesc {
     uint64_t seed;
     uint64_t sweep_base;    // sweep index stored at plaq_out[0]
     double* plaq_out;       // device, nullable
-    uint32_t nonunit;       // FP64: some link is not a unit quaternion (unit_check_kernel)
+    uint32_t general;       // FP64: why the sweeps take the FP64 sequence (GENERAL_*), or 0
     // advanced by the kernels
     uint64_t sweep;         // cumulative sweep counter
     unsigned long long trials, updates, caps;
@@ -204,7 +208,7 @@ cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, boo
                          int32_t* dbg_trials, bool hybrid, bool mirror, cudaStream_t s);
 cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s);
 // FP64 lattices, after launch_set_params: looks at every link and sets
-// nonunit where | |U|^2 - 1 | > UNIT_TOLERANCE; mirror: also writes the
+// GENERAL_LINKS where | |U|^2 - 1 | > UNIT_TOLERANCE; mirror: also writes the
 // fixed-point copy
 cudaError_t launch_unit_check(const Ctx& c, bool mirror, cudaStream_t s);
 // largest link buffer (bytes) an FP64 handle keeps a fixed-point copy of, in

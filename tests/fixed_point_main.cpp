@@ -57,6 +57,80 @@ void update(const Q<double>* L, double beta, const uint32_t* w, F* lam2, bool* o
     for (F& c : U->c) c /= std::sqrt(n);
 }
 
+// errors of accepted new links in fixed point (f) and in doubles (d)
+struct Errors {
+    double mf = 0, md = 0, sf = 0, sd = 0;
+    long n = 0, flips = 0, values = 0;
+    void print(const char* name, double beta, double spread) const
+    {
+        printf("%s %g %g %ld %ld %.3e %.3e %.3e %.3e\n", name, beta, spread, n, flips, mf, md,
+               std::sqrt(sf / values), std::sqrt(sd / values));
+    }
+};
+// components c0 .. 3 of new links among random neighbours of spread `spread`
+// around the identity (negative: any); in every near1-th draw (0: none) both
+// logarithms are near zero
+bool new_links(double beta, double spread, int iters, int near1, int c0, std::mt19937_64& g,
+               std::normal_distribution<double>& N, Errors* e)
+{
+    for (int it = 0; it < iters; ++it) {
+        Q<double> L[18];
+        for (auto& q : L) {
+            double s = 0;
+            for (int c = 0; c < 4; ++c) {
+                q.c[c] = N(g);
+                if (spread >= 0) q.c[c] = c == 0 ? 1 : spread * q.c[c];
+                s += q.c[c] * q.c[c];
+            }
+            for (double& c : q.c) c /= std::sqrt(s);
+        }
+        uint32_t w[4];
+        for (uint32_t& x : w) x = (uint32_t)g();
+        if (near1 && it % near1 == 0) {
+            w[0] |= 0xFFFF0000u;
+            w[2] |= 0xFFF00000u;
+        }
+        LD lam;
+        double lamd;
+        bool ok, okd;
+        Q<LD> U;
+        Q<double> Ud;
+        update<LD>(L, beta, w, &lam, &ok, &U);
+        update<double>(L, beta, w, &lamd, &okd, &Ud);
+        int64_t A[4] = {0, 0, 0, 0};
+        for (int i = 0; i < 6; ++i) {
+            auto conv = [&](const Q<double>& q) {
+                auto f = [&](int c) {
+                    return fx_link((uint32_t)(bits(q.c[c]) >> 32), (uint32_t)bits(q.c[c]));
+                };
+                return FQuat{f(0), f(1), f(2), f(3)};
+            };
+            fq_staple(conv(L[3 * i]), conv(L[3 * i + 1]), conv(L[3 * i + 2]), i & 1, A);
+        }
+        Drawn D;
+        uint64_t K;
+        int sc;
+        if (!unit_staple(A, half_inv_beta_fix(bits(0.5 / beta)), &D, &K, &sc)) return false;
+        const Lambda l = kp_lambda(kp_sum(w[0], w[1], w[2], &T), D.inv, D.ei);
+        const bool okf = kp_accept(l, w[3]);
+        e->flips += okf != ok;
+        if (!ok || !okf) continue;
+        int64_t u[4];
+        new_link_fix(l, ((w[0] & 511) << 9) | (w[1] & 511), ((w[2] & 511) << 9) | (w[3] & 511), D.V, &T, u);
+        for (int c = c0; c < 4; ++c) {
+            const double ef = err(from_bits(double_bits(u[c], -60)), U.c[c]);
+            const double ed = err(Ud.c[c], U.c[c]);
+            e->mf = std::max(e->mf, ef);
+            e->md = std::max(e->md, ed);
+            e->sf += ef * ef;
+            e->sd += ed * ed;
+            ++e->values;
+        }
+        ++e->n;
+    }
+    return true;
+}
+
 int main()
 {
     fill_fix_tables(&T);
@@ -143,65 +217,18 @@ int main()
     const double betas[] = {0.1, 0.7, 2.3, 6.0, 50.0, 1e5};
     for (double beta : betas)
         for (double spread : {0.0, 0.3, -1.0}) {  // -1: random links
-            double mf = 0, md = 0, sf = 0, sd = 0;
-            long n = 0, flips = 0;
-            for (int it = 0; it < 60000; ++it) {
-                Q<double> L[18];
-                for (auto& q : L) {
-                    double s = 0;
-                    for (int c = 0; c < 4; ++c) {
-                        q.c[c] = N(g);
-                        if (spread >= 0) q.c[c] = c == 0 ? 1 : spread * q.c[c];
-                        s += q.c[c] * q.c[c];
-                    }
-                    for (double& c : q.c) c /= std::sqrt(s);
-                }
-                uint32_t w[4];
-                for (uint32_t& x : w) x = (uint32_t)g();
-                if (it % 4 == 0) {  // both logarithms near zero
-                    w[0] |= 0xFFFF0000u;
-                    w[2] |= 0xFFF00000u;
-                }
-                LD lam;
-                double lamd;
-                bool ok, okd;
-                Q<LD> U;
-                Q<double> Ud;
-                update<LD>(L, beta, w, &lam, &ok, &U);
-                update<double>(L, beta, w, &lamd, &okd, &Ud);
-                int64_t A[4] = {0, 0, 0, 0};
-                for (int i = 0; i < 6; ++i) {
-                    auto conv = [&](const Q<double>& q) {
-                        auto f = [&](int c) {
-                            return fx_link((uint32_t)(bits(q.c[c]) >> 32), (uint32_t)bits(q.c[c]));
-                        };
-                        return FQuat{f(0), f(1), f(2), f(3)};
-                    };
-                    fq_staple(conv(L[3 * i]), conv(L[3 * i + 1]), conv(L[3 * i + 2]), i & 1, A);
-                }
-                Drawn D;
-                uint64_t K;
-                int sc;
-                if (!unit_staple(A, half_inv_beta_fix(bits(0.5 / beta)), &D, &K, &sc)) return 1;
-                const Lambda l = kp_lambda(kp_sum(w[0], w[1], w[2], &T), D.inv, D.ei);
-                const bool okf = kp_accept(l, w[3]);
-                flips += okf != ok;
-                if (!ok || !okf) continue;
-                int64_t u[4];
-                new_link_fix(l, ((w[0] & 511) << 9) | (w[1] & 511), ((w[2] & 511) << 9) | (w[3] & 511),
-                             D.V, &T, u);
-                for (int c = 0; c < 4; ++c) {
-                    const double ef = err(from_bits(double_bits(u[c], -60)), U.c[c]);
-                    const double ed = err(Ud.c[c], U.c[c]);
-                    mf = std::max(mf, ef);
-                    md = std::max(md, ed);
-                    sf += ef * ef;
-                    sd += ed * ed;
-                }
-                ++n;
-            }
-            printf("link %g %g %ld %ld %.3e %.3e %.3e %.3e\n", beta, spread, n, flips, mf, md,
-                   std::sqrt(sf / (4 * n)), std::sqrt(sd / (4 * n)));
+            Errors e;
+            if (!new_links(beta, spread, 60000, 4, 0, g, N, &e)) return 1;
+            e.print("link", beta, spread);
+        }
+    // the vector parts apart: their size, and with it a double's error, shrinks
+    // as beta^-1/2, the fixed point's does not
+    printf("limit %g\n", FIX_BETA_MAX);
+    for (double beta : {2.3, FIX_BETA_MAX, 1e5})
+        for (double spread : {1e-4, 0.5 / std::sqrt(beta)}) {
+            Errors e;
+            if (!new_links(beta, spread, 60000, 0, 1, g, N, &e)) return 1;
+            e.print("vector", beta, spread);
         }
     return 0;
 }

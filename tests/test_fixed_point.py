@@ -2,7 +2,8 @@
 compiled for the host, against long double: each function within the error
 its place in the update allows, and the new link closer to the exact one than
 the same update in doubles, over couplings from 0.1 to 1e5 and links from
-ordered to random."""
+ordered to random (all components together; the vector part alone up to the
+coupling FIX_BETA_MAX, above which the kernels take the FP64 sequence)."""
 import os
 import shutil
 import subprocess
@@ -26,7 +27,7 @@ def lines(tmp_path_factory):
 
 
 def test_functions(lines):
-    got = {ln[0]: [float(x) for x in ln[1:]] for ln in lines if ln[0] != "link"}
+    got = {ln[0]: [float(x) for x in ln[1:]] for ln in lines if ln[0] not in ("link", "vector")}
     u = 2.0 ** -57
     # -ln u at 2^-61 (u > 1/2) and 2^-57, a truncation or two each
     assert got["ln"][0] <= 2.0 ** -59 and got["ln"][1] <= 2 * u
@@ -46,3 +47,19 @@ def test_new_links_are_no_further_off_than_in_doubles(lines):
         assert n > 10000 and flips == 0, (beta, spread)
         assert rms <= 0.5 * rms_d, (beta, spread, rms, rms_d)
         assert worst <= worst_d, (beta, spread, worst, worst_d)
+
+
+def test_vector_parts_up_to_the_largest_coupling(lines):
+    """At coupling beta the vector part of a link is of the size of beta^-1/2 and
+    a double's error shrinks with it, an absolute error at 2^-61 .. 2^-57 does
+    not: up to FIX_BETA_MAX the fixed point is still the closer, and at 1e5,
+    where the kernels do not use it, it is not (so the limit is needed)."""
+    limit = [float(ln[1]) for ln in lines if ln[0] == "limit"][0]
+    rows = [[float(x) for x in ln[1:]] for ln in lines if ln[0] == "vector"]
+    assert [r[0] for r in rows] == [2.3, 2.3, limit, limit, 1e5, 1e5]
+    for beta, spread, n, flips, worst, worst_d, rms, rms_d in rows:
+        assert n > 50000 and flips == 0, (beta, spread)
+        if beta <= limit:
+            assert rms <= 0.6 * rms_d and worst <= worst_d, (beta, spread, rms, rms_d, worst, worst_d)
+        else:
+            assert rms > rms_d, (beta, spread, rms, rms_d)

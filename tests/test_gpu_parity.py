@@ -1218,6 +1218,51 @@ def test_fp64_lattice_with_non_unit_links(cfg):
     np.testing.assert_allclose(out[0][1], rplaq, rtol=1e-13, atol=0)
 
 
+@pytest.mark.parametrize("cfg", [0, 4, 8, 11, 12])
+def test_fp64_vector_parts_at_large_couplings(cfg):
+    """At beta = 1e8 the vector part of a link is of the size of 1e-4 and its
+    FP64 errors of 1e-4 2^-53: an update at an absolute 2^-57 (5e-18 rms) would
+    lose two digits of it, so couplings above 64 take the FP64 sequence.  The
+    eight phases of a sweep from the identity, each against the oracle on the
+    GPU's own links, to 8 units of 2^-53 of the largest vector component (the
+    staple's six products, their sum, the draw and the new link each round at
+    about one such unit); the same lattice in a batch beside one at beta = 2.3,
+    and in one call of two sweeps, ends with the same links bit by bit."""
+    Ns, Nt, beta, seed = 6, 4, 1e8, 23
+    lat = lattice(Ns, Nt, su2.F64)
+    lat.set_launch_config(cfg)
+    lat.init(su2.COLD, 1)
+    before = lat.get_links()
+    for mu, p in PHASES:
+        lat.heatbath_phase(beta, mu, p, seed)
+        got = lat.get_links()
+        ref, _, _ = O.heatbath_phase(Ns, Nt, before, beta, mu, p, seed, 0)
+        vec = np.abs(ref[:, mu, 1:]).max()
+        assert 1e-5 < vec < 1e-2
+        assert np.abs(got[:, :, 1:] - ref[:, :, 1:]).max() <= 8 * 2.0 ** -53 * vec
+        assert np.abs(got - ref).max() <= 4 * 2.0 ** -53
+        before = got
+    B = su2.Lattice([Ns, 4], [Nt, 4], su2.F64)
+    B.set_launch_config(cfg)
+    B.batch_init(su2.COLD, [1, 2])
+    pb = B.batch_heatbath([beta, 2.3], 2, [seed, seed + 1])
+    lat.init(su2.COLD, 1)
+    p1 = lat.heatbath(beta, 1, seed)
+    np.testing.assert_array_equal(lat.get_links(), before)
+    p2 = lat.heatbath(beta, 1, seed)
+    np.testing.assert_array_equal(lat.get_links(), B.get_links(0))
+    np.testing.assert_allclose(np.concatenate([p1[0], p2[0]]), pb[0], rtol=1e-13, atol=0)
+    lat.init(su2.COLD, 1)
+    lat.heatbath(beta, 2, seed, plaq=None)
+    np.testing.assert_array_equal(lat.get_links(), B.get_links(0))
+    assert lat.stats()["cap_hits"] == 0
+    # the batch's other lattice keeps the fixed point's bits
+    one = lattice(4, 4, su2.F64)
+    one.init(su2.COLD, 2)
+    one.heatbath(2.3, 2, seed + 1, plaq=None)
+    np.testing.assert_array_equal(one.get_links(), B.get_links(1))
+
+
 @pytest.mark.parametrize("dtype,Ns,Nt", [
     (su2.F32, 2, 2), (su2.F32, 4, 4), (su2.F32, 10, 6), (su2.F32, 8, 8), (su2.F32, 6, 10),
     (su2.F32, 8, 18), (su2.F32, 16, 4), (su2.F32, 16, 6),
