@@ -306,7 +306,10 @@ int su2_set_sweep(su2_lattice* lat, int l, uint64_t sweep);
  * a file, the choice is appended there under a key made of the GPU name,
  * the precision and link layout, the lattice shapes, the shape table and
  * the coupling band, and su2_bind_memory of any later handle with the same
- * key (at beta = 2.4) starts with the cached shape.
+ * key (at beta = 2.4) starts with the cached shape.  Where the fastest index
+ * is one whose sweeps without measurements run in one launch, the fastest
+ * index of sweeps replayed from a graph is kept beside it, for runs under the
+ * Creutz sampler, with measurements and for single phases.
  * chosen (nullable): the index picked.  Synchronous. */
 int su2_autotune(su2_lattice* lat, int* chosen);
 

@@ -28,11 +28,18 @@ extern "C" {
  * (SU2_E_INVAL if it does not fit). */
 int su2_tune_key(const su2_lattice* lat, char* buf, size_t len);
 
-/* Lookup in / append to a tuning-cache file ("key cfg ms" per line, later
- * lines win).  Lookup returns 1 if the key is found (*cfg set), 0 if not;
+/* Lookup in / append to a tuning-cache file ("key cfg ms replay measured" per
+ * line, the last two as in su2_replay_config and cfg where absent; later lines
+ * win).  Lookup returns 1 if the key is found (*cfg set), 0 if not;
  * store returns SU2_OK or SU2_E_INVAL (bad shape index, unwritable file). */
 int su2_tune_cache_lookup(const char* path, const char* key, int* cfg);
 int su2_tune_cache_store(const char* path, const char* key, int cfg, double ms);
+
+/* The launch indices of sweeps replayed from a graph: *plain without
+ * measurements (under the Creutz sampler, and wherever the selected index has
+ * no one-launch form), *measured with.  Tuning chooses them apart from the
+ * index that su2_get_launch_config reports; su2_set_launch_config sets all. */
+int su2_replay_config(const su2_lattice* lat, int* plain, int* measured);
 
 /* Walk every lattice in S y-slabs under the slab launch shapes (S must
  * divide every Ns; by default S is chosen from the lattice size so that

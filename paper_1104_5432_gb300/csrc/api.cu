@@ -95,10 +95,19 @@ struct su2_lattice {
     uint32_t cfg_chunks[NUM_LAUNCH_CFG] = {};
     size_t off_pstart_cfg[NUM_LAUNCH_CFG] = {};
     uint32_t max_phase_blocks = 0;
-    int cfg = 0;                    // active launch shape
-    // whole sweeps in one thread-block cluster (launch index CFG_CLUSTER):
-    // on, and the cluster geometry (cluster_ok: -1 not yet known, 0 / 1)
-    bool cluster = false;
+    // the launch index selected or tuned: sweeps without measurements
+    int chosen = 0;
+    // sweeps replayed from a graph (with measurements, under the Creutz
+    // sampler, and wherever the chosen index has no one-launch chain): the
+    // cluster sweep (index CFG_CLUSTER) or the shape cfg, which single phases
+    // take too.  Tuning sets them apart from `chosen`, since the chain is the
+    // fastest on lattices whose phase launches in the same shape are not; and
+    // the measured sweeps apart from the others, since their measurements run
+    // beside phase launches and before a cluster sweep (8^4 FP32: 31 us a
+    // measured sweep against 37, 29 and 23 without).
+    int cfg = 0;
+    bool cluster = false, cluster_measured = false;
+    // cluster geometry (cluster_ok: -1 not yet known, 0 / 1)
     int cluster_ok = -1;
     ClusterGeom cgeom{};
     // all sweeps of a call in one cluster launch: index CFG_CLUSTER where a
@@ -415,7 +424,7 @@ int record_measure(su2_lattice* L, int rmax, cudaStream_t s)
 // leave alone, so it overlaps them and joins before phase (3, 0).
 int record_sweep(su2_lattice* L, bool plaq, int rmax, cudaStream_t s)
 {
-    if (L->cluster) {
+    if (rmax >= 0 ? L->cluster_measured : L->cluster) {
         // the cluster kernel holds all links for the whole sweep: the
         // previous sweep's result is measured before it, not beside it
         if (rmax >= 0)
@@ -480,10 +489,10 @@ void set_measure_rmax(su2_lattice* L, int rmax)
 int sweep_graph(su2_lattice* L, bool plaq, int rmax, cudaGraphExec_t* exec)
 {
     if (rmax >= 0) set_measure_rmax(L, rmax);
-    cudaGraphExec_t& g = L->cluster ? (rmax >= 0 ? L->cluster_measure_graph[plaq ? 1 : 0]
-                                                 : L->cluster_graph[plaq ? 1 : 0])
-                         : rmax >= 0 ? L->measure_graph[L->cfg][plaq ? 1 : 0]
-                                     : L->sweep_graph[L->cfg][plaq ? 1 : 0];
+    const int pl = plaq ? 1 : 0;
+    cudaGraphExec_t& g =
+        rmax >= 0 ? (L->cluster_measured ? L->cluster_measure_graph[pl] : L->measure_graph[L->cfg][pl])
+                  : (L->cluster ? L->cluster_graph[pl] : L->sweep_graph[L->cfg][pl]);
     if (!g) {
         if (int rc = capture_graph(
                 L, [&](cudaStream_t s) { return record_sweep(L, plaq, rmax, s); }, &g))
@@ -584,9 +593,9 @@ constexpr uint64_t CHAIN0_MAX_SITES = 16384, CHAIN0_MAX_SITES_F64 = 4096;
 const ChainGeom* chain_of(su2_lattice* L)
 {
     if (L->hybrid || L->row == ROW_F32_PAIRS || L->n != 1) return nullptr;
-    if (L->cluster) return L->cluster_chain ? &L->chain_geom : nullptr;
+    if (L->chosen == CFG_CLUSTER) return L->cluster_chain ? &L->chain_geom : nullptr;
     const bool f64 = L->row == ROW_F64;
-    if (L->cfg != 0 || L->V[0] > (f64 ? CHAIN0_MAX_SITES_F64 : CHAIN0_MAX_SITES)) return nullptr;
+    if (L->chosen != 0 || L->V[0] > (f64 ? CHAIN0_MAX_SITES_F64 : CHAIN0_MAX_SITES)) return nullptr;
     if (L->chain0_ok < 0) {
         DeviceGuard dg(L->device);
         const uint32_t Vh = (uint32_t)(L->V[0] / 2);
@@ -602,17 +611,25 @@ cudaError_t run_chain(su2_lattice* L, const ChainGeom& g, bool plaq, int nsweeps
                              : launch_chain(L->ctx, g, plaq, nsweeps, L->stream);
 }
 
-// select launch index cfg (0 .. NUM_LAUNCH_CFG - 1, or CFG_CLUSTER)
-bool select_cfg(su2_lattice* L, int cfg)
+// Launch indices (0 .. NUM_LAUNCH_CFG - 1, or CFG_CLUSTER): the one selected,
+// and those of the sweeps replayed from a graph without and with measurements
+// (a shape in both places is the same one).
+struct Choice {
+    int cfg = -1, replay = -1, measured = -1;
+    Choice() = default;
+    explicit Choice(int c) : cfg(c), replay(c), measured(c) {}
+};
+// false, and nothing changed, when one is not available
+bool select_cfg(su2_lattice* L, const Choice& c)
 {
-    if (cfg == CFG_CLUSTER) {
-        if (!cluster_available(L)) return false;
-        L->cluster = true;  // L->cfg stays: the single-phase entry point uses it
-        return true;
-    }
-    if (cfg < 0 || cfg >= NUM_LAUNCH_CFG) return false;
-    L->cluster = false;
-    L->cfg = cfg;
+    for (int k : {c.cfg, c.replay, c.measured})
+        if (k < 0 || k > CFG_CLUSTER || (k == CFG_CLUSTER && !cluster_available(L))) return false;
+    L->chosen = c.cfg;
+    L->cluster = c.replay == CFG_CLUSTER;
+    L->cluster_measured = c.measured == CFG_CLUSTER;
+    // (where both are the cluster sweep cfg stays, for single phases)
+    if (!L->cluster) L->cfg = c.replay;
+    else if (!L->cluster_measured) L->cfg = c.measured;
     return true;
 }
 
@@ -783,8 +800,9 @@ std::string tune_key(const su2_lattice* L, int dev, int band)
     return buf;
 }
 
-// Cache file: one line per key, "key cfg ms_per_phase"; later lines win.
-bool cache_lookup(const char* path, const std::string& key, int* cfg)
+// Cache file: one line per key, "key cfg ms_per_sweep [replay measured]"; later
+// lines win.  The last two (Choice) are cfg where absent.
+bool cache_lookup(const char* path, const std::string& key, Choice* out)
 {
     FILE* f = fopen(path, "r");
     if (!f) return false;
@@ -792,10 +810,11 @@ bool cache_lookup(const char* path, const std::string& key, int* cfg)
     bool found = false;
     while (fgets(line, sizeof line, f)) {
         char k[400];
-        int c = -1;
+        Choice c;
         double ms = 0;
-        if (sscanf(line, "%399s %d %lf", k, &c, &ms) >= 2 && key == k) {
-            *cfg = c;
+        const int got = sscanf(line, "%399s %d %lf %d %d", k, &c.cfg, &ms, &c.replay, &c.measured);
+        if (got >= 2 && key == k) {
+            *out = got == 5 ? c : Choice(c.cfg);
             found = true;
         }
     }
@@ -803,11 +822,11 @@ bool cache_lookup(const char* path, const std::string& key, int* cfg)
     return found;
 }
 
-bool cache_store(const char* path, const std::string& key, int cfg, double ms)
+bool cache_store(const char* path, const std::string& key, const Choice& c, double ms)
 {
     FILE* f = fopen(path, "a");
     if (!f) return false;
-    const bool ok = fprintf(f, "%s %d %.6f\n", key.c_str(), cfg, ms) > 0;
+    const bool ok = fprintf(f, "%s %d %.6f %d %d\n", key.c_str(), c.cfg, ms, c.replay, c.measured) > 0;
     return fclose(f) == 0 && ok;
 }
 
@@ -1100,11 +1119,10 @@ int su2_bind_memory(su2_lattice* lat, void* links, size_t link_bytes, void* work
     // a launch shape tuned earlier for these shapes on this GPU, if cached
     // (at the default tuning coupling)
     lat->tune_key = tune_key(lat, dev, beta_band(lat, nullptr, TUNE_BETA));
-    lat->cfg = 0;
-    lat->cluster = false;
     lat->cluster_ok = lat->chain0_ok = -1;
+    select_cfg(lat, Choice(0));
     if (const char* path = getenv("SU2_AUTOTUNE_CACHE")) {
-        int cached = -1;
+        Choice cached;
         if (cache_lookup(path, lat->tune_key, &cached)) select_cfg(lat, cached);
     }
     return SU2_OK;
@@ -1126,9 +1144,8 @@ int su2_set_link_layout(su2_lattice* lat, int layout_code)
     } else {
         return fail(SU2_E_INVAL, "bad link layout %d", layout_code);
     }
-    lat->cfg = 0;
-    lat->cluster = false;
     lat->cluster_ok = lat->chain0_ok = -1;
+    select_cfg(lat, Choice(0));
     return layout(lat);
 }
 
@@ -1341,10 +1358,10 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen)
         SU2_CUDA(launch_init(lat->ctx, lat->dtype, l, (uint32_t)lat->V[l], SU2_HOT, tune_seed + l, s));
     // a choice cached for this GPU, shapes and coupling band: no timing
     if (const char* path = getenv("SU2_AUTOTUNE_CACHE")) {
-        int cached = -1;
+        Choice cached;
         if (cache_lookup(path, lat->tune_key, &cached) && select_cfg(lat, cached)) {
             if (int r2 = sync_status(lat)) return r2;
-            if (chosen) *chosen = cached;
+            if (chosen) *chosen = cached.cfg;
             return SU2_OK;
         }
     }
@@ -1353,21 +1370,26 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen)
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     SU2_CUDA(cudaEventCreate(&e0));
     SU2_CUDA(cudaEventCreate(&e1));
-    const int saved = lat->cfg;
-    const bool saved_cluster = lat->cluster;
-    constexpr int NC = NUM_LAUNCH_CFG + 1;  // the shapes and the cluster sweep
+    const int saved_chosen = lat->chosen, saved = lat->cfg;
+    const bool saved_cluster = lat->cluster, saved_measured = lat->cluster_measured;
+    // the shapes and the cluster sweep replayed from a graph, then the two
+    // one-launch chains (of shape 0 and of the cluster index) where they apply
+    constexpr int NI = NUM_LAUNCH_CFG + 1, NC = NI + 2;
+    auto index_of = [](int k) { return k < NI ? k : (k == NI ? 0 : CFG_CLUSTER); };
+    int rmax = -1;  // the measured sweeps' once those are timed
     double best_ms[NC];
     int reps[NC];
     int rc = SU2_OK;
-    // Time what production runs: whole sweeps (graph replay, fused
-    // plaquette), shapes interleaved over three rounds, best round kept.
+    // Time what production runs: whole sweeps (graph replay or chain, fused
+    // plaquette), candidates interleaved over three rounds, best round kept.
     auto time_sweeps = [&](int k, int n, float* ms) -> int {
-        lat->cluster = k == CFG_CLUSTER;
-        if (k != CFG_CLUSTER) lat->cfg = k;
-        const ChainGeom* chain = chain_of(lat);
+        lat->chosen = index_of(k);
+        lat->cluster = lat->cluster_measured = k == CFG_CLUSTER;
+        if (k < NUM_LAUNCH_CFG) lat->cfg = k;
+        const ChainGeom* chain = k < NI ? nullptr : chain_of(lat);
         cudaGraphExec_t g = nullptr;
         if (!chain)
-            if (int r = sweep_graph(lat, true, -1, &g)) return r;
+            if (int r = sweep_graph(lat, true, rmax, &g)) return r;
         cudaError_t e = cudaEventRecord(e0, s);
         if (chain && e == cudaSuccess) e = run_chain(lat, *chain, true, n);
         for (int i = 0; i < n && !chain && e == cudaSuccess; ++i) e = cudaGraphLaunch(g, s);
@@ -1382,31 +1404,63 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen)
     bool cand[NC];
     for (int k = 0; k < NUM_LAUNCH_CFG; ++k) cand[k] = any_slab || !LAUNCH_CFG[lat->row][k].slab;
     cand[CFG_CLUSTER] = cluster_available(lat);
-    const int ncand = NC;
-    for (int k = 0; k < ncand && rc == SU2_OK; ++k) {
-        if (!cand[k]) continue;
-        float ms = 0.f;
-        rc = time_sweeps(k, 1, &ms);  // builds the graph, warms up
-        if (rc == SU2_OK) rc = time_sweeps(k, 1, &ms);
-        // about 20 ms of sweeps per round, between 1 and 50
-        reps[k] = std::max(1, std::min(50, (int)(20.0 / std::max(ms, 1e-3f))));
-        best_ms[k] = 1e300;
+    for (int k = NI; k < NC; ++k) {
+        lat->chosen = index_of(k);
+        cand[k] = cand[index_of(k)] && chain_of(lat) != nullptr;
     }
-    for (int round = 0; round < 3 && rc == SU2_OK; ++round)
-        for (int k = 0; k < ncand && rc == SU2_OK; ++k) {
+    auto time_candidates = [&]() {
+        for (int k = 0; k < NC && rc == SU2_OK; ++k) {
             if (!cand[k]) continue;
             float ms = 0.f;
-            rc = time_sweeps(k, reps[k], &ms);
-            best_ms[k] = std::min(best_ms[k], (double)ms / reps[k]);
+            rc = time_sweeps(k, 1, &ms);  // builds the graph, warms up
+            if (rc == SU2_OK) rc = time_sweeps(k, 1, &ms);
+            // about 20 ms of sweeps per round, between 1 and 50
+            reps[k] = std::max(1, std::min(50, (int)(20.0 / std::max(ms, 1e-3f))));
+            best_ms[k] = 1e300;
         }
+        for (int round = 0; round < 3 && rc == SU2_OK; ++round)
+            for (int k = 0; k < NC && rc == SU2_OK; ++k) {
+                if (!cand[k]) continue;
+                float ms = 0.f;
+                rc = time_sweeps(k, reps[k], &ms);
+                best_ms[k] = std::min(best_ms[k], (double)ms / reps[k]);
+            }
+    };
+    // the best candidate below n
+    auto best_of = [&](int n, bool chains) {
+        int best = -1;
+        for (int k = 0; k < n; ++k) {
+            // an index whose chain applies runs as the chain
+            if (!cand[k] || (chains && ((k == 0 && cand[NI]) || (k == CFG_CLUSTER && cand[NI + 1]))))
+                continue;
+            if (best < 0 || best_ms[k] < best_ms[best]) best = k;
+        }
+        return best;
+    };
+    time_candidates();
+    Choice pick;
+    double ms_chosen = 0.0;
+    if (rc == SU2_OK) {
+        const int best = best_of(NC, true), shape = best_of(NUM_LAUNCH_CFG, false);
+        ms_chosen = best_ms[best];
+        pick = Choice(index_of(best));
+        // no chain: every sweep is a replayed one
+        pick.replay = pick.measured = best < NI ? best : best_of(NI, false);
+        if (pick.replay == CFG_CLUSTER) {
+            // the measured sweeps: the cluster sweep or the best shape
+            for (int k = 0; k < NC; ++k) cand[k] = k == shape || k == CFG_CLUSTER;
+            rmax = lat->rmax_limit;
+            time_candidates();
+            if (rc == SU2_OK) pick.measured = best_of(NI, false);
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    lat->chosen = saved_chosen;
     lat->cfg = saved;
     lat->cluster = saved_cluster;
+    lat->cluster_measured = saved_measured;
     if (rc != SU2_OK) return rc;
-    int best = 0;
-    for (int k = 1; k < ncand; ++k)
-        if (cand[k] && best_ms[k] < best_ms[best]) best = k;
     // leave the handle as su2_init(SU2_HOT) with the tuning seed would; trial
     // caps hit by the tuning sweeps (small couplings under Kennedy-Pendleton
     // alone) belong to no run of the caller and are not reported
@@ -1414,11 +1468,11 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen)
     for (int l = 0; l < lat->n; ++l)
         SU2_CUDA(launch_init(lat->ctx, lat->dtype, l, (uint32_t)lat->V[l], SU2_HOT, tune_seed + l, s));
     if (int r2 = sync_status(lat)) return r2;
-    select_cfg(lat, best);
+    select_cfg(lat, pick);
     if (const char* path = getenv("SU2_AUTOTUNE_CACHE"))
-        if (!cache_store(path, lat->tune_key, best, best_ms[best]))
+        if (!cache_store(path, lat->tune_key, pick, ms_chosen))
             return fail(SU2_E_INVAL, "cannot append to autotune cache %s", path);
-    if (chosen) *chosen = best;
+    if (chosen) *chosen = pick.cfg;
     return SU2_OK;
 }
 
@@ -1427,7 +1481,7 @@ int su2_set_launch_config(su2_lattice* lat, int cfg)
     if (int rc = check_handle(lat, false)) return rc;
     if (cfg == CFG_CLUSTER && !lat->bound())
         return fail(SU2_E_INVAL, "the cluster sweep is chosen once memory is bound");
-    if (!select_cfg(lat, cfg)) {  // graphs are kept per launch shape
+    if (!select_cfg(lat, Choice(cfg))) {  // graphs are kept per launch shape
         if (cfg == CFG_CLUSTER)
             return fail(SU2_E_INVAL, "the cluster sweep needs one FP32 lattice in the plain "
                                      "layout whose links fit one thread-block cluster");
@@ -1439,15 +1493,15 @@ int su2_set_launch_config(su2_lattice* lat, int cfg)
 int su2_get_launch_config(const su2_lattice* lat, int* cfg, int* threads, int* min_blocks)
 {
     if (int rc = check_handle(lat, false)) return rc;
-    if (lat->cluster) {
+    if (lat->chosen == CFG_CLUSTER) {
         if (cfg) *cfg = CFG_CLUSTER;
         if (threads) *threads = lat->cgeom.threads;
         if (min_blocks) *min_blocks = lat->cgeom.S;
         return SU2_OK;
     }
-    if (cfg) *cfg = lat->cfg;
-    if (threads) *threads = LAUNCH_CFG[lat->row][lat->cfg].threads;
-    if (min_blocks) *min_blocks = LAUNCH_CFG[lat->row][lat->cfg].min_blocks;
+    if (cfg) *cfg = lat->chosen;
+    if (threads) *threads = LAUNCH_CFG[lat->row][lat->chosen].threads;
+    if (min_blocks) *min_blocks = LAUNCH_CFG[lat->row][lat->chosen].min_blocks;
     return SU2_OK;
 }
 
@@ -1516,14 +1570,26 @@ int su2_tune_key(const su2_lattice* lat, char* buf, size_t len)
 int su2_tune_cache_lookup(const char* path, const char* key, int* cfg)
 {
     if (!path || !key || !cfg) return fail(SU2_E_INVAL, "null argument");
-    return cache_lookup(path, key, cfg) ? 1 : 0;
+    Choice c;
+    if (!cache_lookup(path, key, &c)) return 0;
+    *cfg = c.cfg;
+    return 1;
 }
 
 int su2_tune_cache_store(const char* path, const char* key, int cfg, double ms)
 {
     if (!path || !key) return fail(SU2_E_INVAL, "null argument");
     if (cfg < 0 || cfg > CFG_CLUSTER) return fail(SU2_E_INVAL, "bad config");
-    return cache_store(path, key, cfg, ms) ? SU2_OK : fail(SU2_E_INVAL, "cannot write %s", path);
+    return cache_store(path, key, Choice(cfg), ms) ? SU2_OK : fail(SU2_E_INVAL, "cannot write %s", path);
+}
+
+int su2_replay_config(const su2_lattice* lat, int* plain, int* measured)
+{
+    if (int rc = check_handle(lat, false)) return rc;
+    if (!plain || !measured) return fail(SU2_E_INVAL, "null output");
+    *plain = lat->cluster ? CFG_CLUSTER : lat->cfg;
+    *measured = lat->cluster_measured ? CFG_CLUSTER : lat->cfg;
+    return SU2_OK;
 }
 
 const char* su2_last_error(void) { return g_err.c_str(); }

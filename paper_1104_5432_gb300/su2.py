@@ -100,6 +100,7 @@ def load(build_if_needed: bool = True):
             "su2_tune_key": (i, [P, C.c_char_p, sz]),
             "su2_tune_cache_lookup": (i, [C.c_char_p, C.c_char_p, P]),
             "su2_tune_cache_store": (i, [C.c_char_p, C.c_char_p, i, d]),
+            "su2_replay_config": (i, [P, P, P]),
             "su2_set_slabs": (i, [P, i]),
             "su2_set_sampler": (i, [P, d]),
             "su2_set_link_layout": (i, [P, i]),

@@ -722,6 +722,56 @@ def test_autotune_times_the_cluster_sweep():
     np.testing.assert_array_equal(lat.get_links(), ref.get_links())
 
 
+@pytest.mark.parametrize("dtype,Ns,Nt", [(su2.F64, 8, 8), (su2.F64, 6, 4), (su2.F32, 8, 8),
+                                         (su2.F32, 12, 8)])
+def test_tuning_keeps_a_choice_for_replayed_sweeps(dtype, Ns, Nt, tmp_path, monkeypatch):
+    """On small lattices the chosen index runs its sweeps without measurements in
+    one launch; measured runs and the Creutz sampler replay sweeps from a graph,
+    where another index is the faster (8^4 FP64: four threads per link against
+    one, 59 against 96 us).  Tuning keeps that one beside the choice, in the
+    cache too, and both give the same chains; selecting an index sets both."""
+    def replay(lat):
+        v, m = C.c_int(-1), C.c_int(-1)
+        assert su2.load().su2_replay_config(lat._h, C.byref(v), C.byref(m)) == 0
+        return v.value, m.value
+
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("SU2_AUTOTUNE_CACHE", str(cache))
+    lat = lattice(Ns, Nt, dtype)
+    assert replay(lat) == (0, 0) and lat.launch_config()[0] == 0
+    chosen = lat.autotune(beta=2.4)
+    kept = replay(lat)
+    assert lat.launch_config()[0] == chosen
+    if dtype == su2.F64:
+        assert chosen == 0 and kept in ((10, 10), (11, 11))
+    else:
+        # a shape, or the cluster sweep and whichever measures faster
+        assert chosen in (0, su2.LAUNCH_CLUSTER)
+        assert kept[0] == kept[1] or kept[0] == su2.LAUNCH_CLUSTER
+    lines = cache.read_text().splitlines()
+    assert len(lines) == 1
+    assert [int(lines[0].split()[k]) for k in (1, 3, 4)] == [chosen, *kept]
+    again = lattice(Ns, Nt, dtype)
+    assert again.launch_config()[0] == chosen and replay(again) == kept
+    ref = lattice(Ns, Nt, dtype)
+    for h in (again, ref):
+        h.init(su2.HOT, 7)
+    for creutz in (0.0, 1.7):
+        runs = []
+        for h in (again, ref):
+            h.set_sampler(creutz)
+            h.heatbath(2.3, 2, 5, plaq=None)
+            runs.append(h.batch_heatbath_measure([0.9], 2, [5], 2))
+            h.heatbath_phase(2.3, 1, 1, 5)
+        np.testing.assert_array_equal(again.get_links(), ref.get_links())
+        for a, b in zip(*runs):
+            np.testing.assert_allclose(a, b, rtol=0, atol=1e-13 if dtype == su2.F64 else 1e-7)
+        assert again.stats() == ref.stats() and again.get_sweep() == ref.get_sweep()
+    assert again.launch_config()[0] == chosen and replay(again) == kept
+    again.set_launch_config(3)
+    assert again.launch_config()[0] == 3 and replay(again) == (3, 3)
+
+
 def test_autotune_and_cache(tmp_path, monkeypatch):
     cache = tmp_path / "tune.txt"
     monkeypatch.setenv("SU2_AUTOTUNE_CACHE", str(cache))
