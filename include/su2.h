@@ -305,7 +305,7 @@ int su2_set_sweep(su2_lattice* lat, int l, uint64_t sweep);
  * or su2_set_links.  If the environment variable SU2_AUTOTUNE_CACHE names
  * a file, the choice is appended there under a key made of the GPU name,
  * the precision and link layout, the lattice shapes, the shape table and
- * the coupling band, and su2_bind_memory of any later handle with the same
+ * the kernels behind it, the sampler and the coupling band, and su2_bind_memory of any later handle with the same
  * key (at beta = 2.4) starts with the cached shape.  Where the fastest index
  * is one whose sweeps without measurements run in one launch, the fastest
  * index of sweeps replayed from a graph is kept beside it, for runs under the

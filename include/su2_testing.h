@@ -24,7 +24,8 @@ extern "C" {
 
 /* The handle's tuning-cache key: GPU name | precision | lattice count |
  * total volume | hash of the lattice shapes | hash of the launch-shape
- * table.  buf receives a NUL-terminated string of at most len bytes
+ * table, a version of the kernels behind it and the sampler | coupling band.
+ * buf receives a NUL-terminated string of at most len bytes
  * (SU2_E_INVAL if it does not fit). */
 int su2_tune_key(const su2_lattice* lat, char* buf, size_t len);
 

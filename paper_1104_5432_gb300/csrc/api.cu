@@ -764,6 +764,10 @@ int beta_band(const su2_lattice* L, const double* betas, double beta)
 
 constexpr double TUNE_BETA = 2.4;  // coupling of su2_autotune without betas
 
+// Raised when another kernel comes to stand behind a launch index, so that no
+// choice timed with the old one is taken from a cache file.
+constexpr int KERNEL_VERSION = 1;
+
 // FNV-1a over the lattice shapes, with the GPU name and precision in clear,
 // and the coupling band
 std::string tune_key(const su2_lattice* L, int dev, int band)
@@ -780,15 +784,19 @@ std::string tune_key(const su2_lattice* L, int dev, int band)
             h ^= (uint64_t)v;
             h *= 1099511628211ull;
         }
-    // the launch-shape table of this precision: a cached index names a
-    // shape only in the table it was tuned with
+    // the launch-shape table of this precision, the kernels behind it and the
+    // sampler: a cached index names the kernel that was timed only with these
     uint32_t th = 2166136261u;
+    auto hash = [&](int v) {
+        th ^= (uint32_t)v;
+        th *= 16777619u;
+    };
     for (const LaunchCfg& c : LAUNCH_CFG[L->row])
         for (int v : {c.threads, c.min_blocks, (int)c.slab, c.rounds, (int)c.persistent, c.group,
-                      (int)c.stage}) {
-            th ^= (uint32_t)v;
-            th *= 16777619u;
-        }
+                      (int)c.stage})
+            hash(v);
+    hash(KERNEL_VERSION);
+    hash(L->hybrid ? 1 : 0);
     char buf[256];
     static const char* const rows[NUM_ROWS] = {"f32", "f64", "f32pairs"};
     snprintf(buf, sizeof buf, "%s|%s|n%d|V%llu|%016llx|t%08x|b%d", name.c_str(), rows[L->row],

@@ -142,6 +142,26 @@ def test_tune_key_and_launch_config_host_side():
     lib.su2_lattice_destroy(h)
 
 
+def test_tune_key_names_more_than_the_shape_table():
+    """The key's table hash covers more than the table: a version of the kernels
+    behind its indices (choices cached before the one-launch chains stood behind
+    FP32 indices 0 and 14, whose table is the same, must miss)."""
+    from paper_1104_5432_gb300.csrc_info import _F32
+    h = 2166136261
+    for t, m, slab, r, ps, *extra in _F32:
+        g = extra[0] if extra else 1
+        stage = len(extra) > 1 and extra[1]
+        for v in (t, m, int(slab), r, int(ps), g, int(stage)):
+            h = ((h ^ v) * 16777619) & 0xFFFFFFFF
+    lib = su2.load()
+    hd = C.c_void_p()
+    assert lib.su2_lattice_create(8, 8, su2.F32, C.byref(hd)) == 0
+    buf = C.create_string_buffer(256)
+    assert lib.su2_tune_key(hd, buf, 256) == 0
+    assert buf.value.decode().split("|")[5] != "t%08x" % h
+    lib.su2_lattice_destroy(hd)
+
+
 def test_cluster_launch_index_mirrors_the_header():
     """SU2_LAUNCH_CLUSTER of include/su2.h is the Python and shape-table
     mirrors' index, one past the shapes."""

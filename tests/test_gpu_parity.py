@@ -772,6 +772,23 @@ def test_tuning_keeps_a_choice_for_replayed_sweeps(dtype, Ns, Nt, tmp_path, monk
     assert again.launch_config()[0] == 3 and replay(again) == (3, 3)
 
 
+def test_tuning_cache_tells_the_samplers_apart(tmp_path, monkeypatch):
+    """A choice tuned under Kennedy-Pendleton alone is not taken by a handle
+    with the Creutz variant, whose kernels are others, nor the reverse; each
+    finds its own again."""
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("SU2_AUTOTUNE_CACHE", str(cache))
+    lat = lattice(8, 4, su2.F64)
+    picked = []
+    for n, creutz in ((1, 0.0), (2, 1.7), (2, 0.0), (2, 1.7)):
+        lat.set_sampler(creutz)
+        picked.append(lat.autotune(beta=2.3))
+        lines = cache.read_text().splitlines()
+        assert len(lines) == n
+    assert len({ln.split()[0] for ln in lines}) == 2
+    assert picked[2:] == picked[:2]
+
+
 def test_autotune_and_cache(tmp_path, monkeypatch):
     cache = tmp_path / "tune.txt"
     monkeypatch.setenv("SU2_AUTOTUNE_CACHE", str(cache))
