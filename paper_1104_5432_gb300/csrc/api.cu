@@ -443,7 +443,7 @@ int record_sweep(su2_lattice* L, bool plaq, int rmax, cudaStream_t s)
         if (branch && mu == 3) SU2_CUDA(cudaStreamWaitEvent(s, L->join_ev, 0));
         for (int p = 0; p < 2; ++p)
             SU2_CUDA(launch_phase(L->cfg_ctx[L->cfg], L->row, L->cfg, mu, p, plaq, nullptr,
-                                  L->hybrid, true, s));
+                                  L->hybrid, false, s));
     }
     SU2_CUDA(launch_sweep_end(L->cfg_ctx[L->cfg], L->row == ROW_F64, plaq, s));
     return SU2_OK;
@@ -1216,17 +1216,14 @@ int su2_heatbath_phase(su2_lattice* lat, double beta, int mu, int parity, uint64
     DeviceGuard dg(lat->device);
     // consecutive phases with the same beta and seed reuse the parameters
     // already on the device (no parameter kernel between the phases)
-    // (FP64: the parameter kernel also starts the look at the links)
-    const bool f64 = lat->row == ROW_F64;
-    if (f64 || !(lat->phase_params_valid && lat->phase_beta == beta && lat->phase_seed == seed)) {
+    if (!(lat->phase_params_valid && lat->phase_beta == beta && lat->phase_seed == seed)) {
         if (int rc = set_params(lat, nullptr, beta, nullptr, seed, nullptr, 0)) return rc;
         lat->phase_params_valid = true;
         lat->phase_beta = beta;
         lat->phase_seed = seed;
     }
-    if (f64) SU2_CUDA(launch_unit_check(lat->ctx, false, lat->stream));
     SU2_CUDA(launch_phase(lat->cfg_ctx[lat->cfg], lat->row, lat->cfg, mu, parity, false, trials,
-                          lat->hybrid, false, lat->stream));
+                          lat->hybrid, true, lat->stream));
     return SU2_OK;
 }
 

@@ -132,7 +132,7 @@ cudaError_t launch_fix_kind(const Ctx& c, const LaunchCfg& f, int mu, int parity
                             int32_t* dbg, bool mirror, cudaStream_t s);
 
 cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, bool plaq,
-                         int32_t* dbg_trials, bool hybrid, bool mirror, cudaStream_t s)
+                         int32_t* dbg_trials, bool hybrid, bool single, cudaStream_t s)
 {
     if (row < 0 || row >= NUM_ROWS || cfg < 0 || cfg >= NUM_LAUNCH_CFG) return cudaErrorInvalidValue;
     if (row == ROW_F64) {
@@ -148,7 +148,10 @@ cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, boo
             {launch_fix_kind<5, false>, launch_fix_kind<5, true>},
         };
         const LaunchCfg& f = LAUNCH_CFG[ROW_F64][cfg];
-        return kinds[fix_kind(f)][hybrid](c, f, mu, parity, plaq, dbg_trials, mirror && c.mirror, s);
+        Ctx cc = c;
+        cc.look = single;
+        return kinds[fix_kind(f)][hybrid](cc, f, mu, parity, plaq && !single, dbg_trials,
+                                          !single && c.mirror, s);
     }
     using Fn = cudaError_t (*)(const Ctx&, int, int, int, bool, int32_t*, bool, cudaStream_t);
     static_assert(NUM_LAUNCH_CFG == 14 && NUM_ROWS == 3, "one entry per pair of shapes below");

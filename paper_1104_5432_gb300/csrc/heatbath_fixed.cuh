@@ -19,7 +19,11 @@
 // every link before the sweeps of a call and sweep_end_kernel again after
 // each sweep of a lattice that failed; such a lattice, and one at a coupling
 // above FIX_BETA_MAX (D.general), takes the FP64 sequence, one link per
-// thread, in the same kernels.
+// thread, in the same kernels.  A single phase is launched without that look
+// (a pass over all links and the parameters' launch before it: 8^4 15.5 us a
+// phase, 16^4 22.7, 64^4 1652): each update looks at the 18 links it reads, and
+// a link with a neighbour that fails takes the FP64 sequence by itself (7.4,
+// 13.6, 1480).
 #pragma once
 #include "heatbath_kernel.cuh"
 #include "su2_mirror.cuh"
@@ -30,15 +34,21 @@ namespace su2 {
 // (MIR) or from the doubles; the stored values are doubles.
 template <bool MIR> struct FixLinks;
 template <> struct FixLinks<false> : Links<double> {
+    bool look;
+    mutable bool all_unit = true;  // (look) every link read so far is a unit quaternion
     __device__ __forceinline__ FixLinks(const Ctx& c, const LatDesc& d)
-        : Links<double>(c.links, d, c.status) {}
+        : Links<double>(c.links, d, c.status), look(c.look != 0) {}
     __device__ __forceinline__ FQuat fix(int mu, int p, uint32_t eo) const
     {
-        return fq_link(load(mu, p, eo));
+        const Quat<double> q = load(mu, p, eo);
+        const FQuat f = fq_link(q);
+        if (look && !unit_limbs(q, f)) all_unit = false;
+        return f;
     }
 };
 template <> struct FixLinks<true> : Links<double> {
     FixMirror m;
+    static constexpr bool all_unit = true;
     __device__ __forceinline__ FixLinks(const Ctx& c, const LatDesc& d)
         : Links<double>(c.links, d, c.status), m(c, d) {}
     __device__ __forceinline__ FQuat fix(int mu, int p, uint32_t eo) const { return m.load(mu, p, eo); }
@@ -216,6 +226,14 @@ __device__ __noinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, u
     *plaq += qretr(un, P);
     return tr;
 }
+template <typename LT>
+__device__ __forceinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, uint32_t i, int mu,
+                                                int p, bool hyb)
+{
+    double plaq = 0.0;
+    uint32_t lex;
+    return general_link<LT>(ctx, D, i, mu, p, hyb, &plaq, &lex);
+}
 // the links i0, i0 + step, ... below end of one thread, then the warp totals
 template <int MU, bool PLAQ>
 __device__ __noinline__ void general_links(const Ctx& ctx, int l, uint32_t blk0, uint32_t i0,
@@ -265,7 +283,10 @@ fix_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         Drawn d;
         double qc;
         int32_t tr = -1;
-        if (!fix_prepare<HYB>(C, A, &d, &qc)) {
+        if (!PLAQ && !U.all_unit) {
+            tr = general_link<Links<double>>(ctx, D, i, MU, p, HYB);
+            ncap = tr < 0;
+        } else if (!fix_prepare<HYB>(C, A, &d, &qc)) {
             const Quat<double> h = haar_link(st, C.tab);
             U.store(MU, p, i, h);
             if (PLAQ) fix_from_link(h, un);
@@ -376,8 +397,13 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
                 int64_t A[4];
                 fix_staple_sum<MU, PLAQ>(U, s, i, p, A, P);
                 key = s.lex() * 4u + MU;
-                pend = fix_prepare<HYB>(C, A, &d, &qc);
-                if (!pend) {
+                if (!PLAQ && !U.all_unit) {
+                    const int32_t tr = general_link<Links<double>>(ctx, D, i, MU, p, HYB);
+                    ncap += tr < 0;
+                    ntrial += tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
+                    if (dbg) dbg[key >> 2] = tr;
+                    if constexpr (!MIR) U.all_unit = true;
+                } else if (!(pend = fix_prepare<HYB>(C, A, &d, &qc))) {
                     const Quat<double> h = haar_link(C.stream(key), C.tab);
                     U.store(MU, p, i, h);
                     if (PLAQ) {
@@ -509,6 +535,7 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         Trial64 trial[4][32];
         Dir64 dir[32];
         uint32_t pend;
+        uint32_t bad[3];  // links with a neighbour that is not a unit quaternion, by plane
     };
     constexpr int SPEC = MINB > 4 ? 2 : 3;  // trials drawn ahead besides the first
     __shared__ Group G;
@@ -556,6 +583,10 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
             draw(C.stream(lex * 4u + MU), 0, 0);
         }
     }
+    if (!MIR && !PLAQ) {
+        const uint32_t m = __ballot_sync(0xffffffffu, !U.all_unit);
+        if (lane == 0 && role < 3) G.bad[role] = m;
+    }
     __syncthreads();
     const Stream st = C.stream(lex * 4u + MU);
     Drawn d;
@@ -563,8 +594,11 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     Lambda L = {0, 0, 0};
     int32_t tr = -1;
     uint32_t kd1 = 0, kd2 = 0;
-    bool haar = false, wait = false;
-    if (role == 0 && act) {
+    bool haar = false, wait = false, general = false;
+    if (!MIR && !PLAQ && role == 0 && act) general = ((G.bad[0] | G.bad[1] | G.bad[2]) >> lane) & 1u;
+    if (general) {
+        tr = general_link<Links<double>>(ctx, D, i, MU, p, HYB);
+    } else if (role == 0 && act) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) P[c] = A[c];
 #pragma unroll
@@ -637,7 +671,9 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     uint32_t ntrial = 0, ncap = 0;
     if (act) {
         int64_t un[4];
-        if (haar) {
+        if (general) {
+            ncap = tr < 0;  // general_link stored it
+        } else if (haar) {
             const Quat<double> h = haar_link(st, C.tab);
             U.store(MU, p, i, h);
             if (PLAQ) fix_from_link(h, un);

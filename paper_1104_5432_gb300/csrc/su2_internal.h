@@ -170,6 +170,7 @@ struct Ctx {
     uint32_t phase_blocks, site_blocks, spat_blocks;
     uint32_t max_chunks;
     uint32_t phase_wpb;            // warps per phase block of this launch shape
+    uint32_t look;                 // FP64 single phases: each update looks at the links it reads
 };
 
 // first grid block of lattice l; lattice 0 starts at block 0, so a single
@@ -203,9 +204,11 @@ struct ParamChunk {
 cudaError_t launch_set_params(const Ctx& c, const ParamChunk& pc, cudaStream_t s);
 // hybrid: compile-time variant with Creutz's draw below each lattice's
 // creutz_below (the plain variant never looks at it)
-// mirror (FP64): the neighbours come from the fixed-point copy of the links
+// single (FP64): a phase by itself, without launch_unit_check before it: the
+// fixed-point copy of the links is not read, and a link with a neighbour that
+// is not a unit quaternion takes the FP64 sequence (no fused plaquette)
 cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, bool plaq,
-                         int32_t* dbg_trials, bool hybrid, bool mirror, cudaStream_t s);
+                         int32_t* dbg_trials, bool hybrid, bool single, cudaStream_t s);
 cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s);
 // FP64 lattices, after launch_set_params: looks at every link and sets
 // GENERAL_LINKS where | |U|^2 - 1 | > UNIT_TOLERANCE; mirror: also writes the

@@ -1285,6 +1285,48 @@ def test_fp64_lattice_with_non_unit_links(cfg):
     np.testing.assert_allclose(out[0][1], rplaq, rtol=1e-13, atol=0)
 
 
+@pytest.mark.parametrize("Ns,Nt,creutz", [(6, 4, 0.0), (2, 2, 0.0), (4, 6, 1.7)])
+def test_fp64_single_phases_look_at_the_links_they_read(Ns, Nt, creutz):
+    """A single phase is one kernel without a pass over the links before it: a
+    link one of whose 18 neighbours is not a unit quaternion (three links of the
+    lattice, scaled, one of them to zero) takes the FP64 sequence by itself.
+    All shapes give the same links and trial counts bit by bit, within 1e-12 of
+    the oracle, and links written into the buffer between two phases, past
+    every entry point, are seen by the next one."""
+    V, beta, seed = Ns ** 3 * Nt, 2.3, 29
+    rng = np.random.default_rng(6)
+    links = inputs.random_links(Ns, Nt, 9)
+    bent = links.copy()
+    for k, scale in zip(rng.choice(4 * V, 3, replace=False), (1.9, 0.0, 0.99)):
+        bent.reshape(-1, 4)[k] *= scale
+    odd = parity_mask(Ns, Nt)
+    first = None
+    for cfg in (0, 2, 4, 5, 6, 9, 10, 11, 12, 13):
+        lat = lattice(Ns, Nt, su2.F64)
+        lat.set_launch_config(cfg)
+        lat.set_sampler(creutz)
+        lat.set_links(bent)
+        written = lat.links_buf.clone()
+        lat.set_links(links)
+        lat.heatbath_phase(beta, 2, 0, seed)
+        lat.links_buf.copy_(written)
+        got = []
+        for mu, p in ((0, 1), (3, 0)):
+            trials = torch.full((V,), -2, dtype=torch.int32, device="cuda")
+            lat.heatbath_phase(beta, mu, p, seed, trials)
+            got += [lat.get_links(), trials.cpu().numpy()]
+        if first is None:
+            first = got
+            ref = bent
+            for n, (mu, p) in enumerate(((0, 1), (3, 0))):
+                ref, rt, _ = O.heatbath_phase(Ns, Nt, ref, beta, mu, p, seed, 0, creutz_below=creutz)
+                assert np.max(np.abs(got[2 * n] - ref)) <= 1e-12
+                np.testing.assert_array_equal(got[2 * n + 1][odd == p], rt[odd == p, mu])
+        for a, b in zip(got, first):
+            np.testing.assert_array_equal(a, b)
+        assert lat.stats()["updates"] == 3 * V // 2
+
+
 @pytest.mark.parametrize("cfg", [0, 4, 8, 11, 12])
 def test_fp64_vector_parts_at_large_couplings(cfg):
     """At beta = 1e8 the vector part of a link is of the size of 1e-4 and its
