@@ -518,13 +518,14 @@ fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
 struct Trial64 {
     int64_t t;
     int32_t e;
-    uint32_t w3;
+    uint32_t w3;  // the word of the accept test
 };
 struct Dir64 {
     int64_t sth, cph, sph;
     int32_t cth, pad;
 };
 static_assert(sizeof(Trial64) == 16 && sizeof(Dir64) == 32, "16-byte accesses");
+static_assert(KP_CAP % 4 == 0, "whole rounds of four trials");
 
 template <int MU, bool PLAQ, bool HYB, bool MIR, int MINB>
 __global__ void __launch_bounds__(128, MINB)
@@ -532,12 +533,23 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
     struct Group {
         longlong2 sums[2][2][32];  // planes 1 and 2
-        Trial64 trial[4][32];
+        Trial64 trial[4][32];  // HYB: lambda^2 of a trial, and whether it was accepted
         Dir64 dir[32];
+        struct Hyb {  // a link's inputs to its trials
+            int64_t inv[HYB ? 32 : 1];
+            double qc[HYB ? 32 : 1];
+            int32_t ei[HYB ? 32 : 1];
+        } hyb;
         uint32_t pend;
         uint32_t bad[3];  // links with a neighbour that is not a unit quaternion, by plane
     };
     constexpr int SPEC = MINB > 4 ? 2 : 3;  // trials drawn ahead besides the first
+    // HYB: Creutz's logarithm runs on the FP64 unit (~2,500 clocks a warp), so
+    // with few blocks an SM each of the four sub-partitions takes a trial of
+    // the waiting links (8^4, beta = 0.9, Creutz's draw below alpha = 1.7: 128 ->
+    // 88 us a sweep); where the SM is full the trials after an accepted one
+    // would cost others their turn (16^4 189 us one by one, 223 so)
+    constexpr bool SPREAD = MINB <= 4;
     __shared__ Group G;
     const int l = lattice_of_block(ctx.phase_start, ctx.n, blockIdx.x);
     const LatDesc& D = ctx.desc[l];
@@ -554,8 +566,10 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const FixCall C(D);
     auto draw = [&](const Stream& st, int t, int slot) {
         const U4 w = st.draw(TAG_TRIAL, (uint32_t)t);
-        const KpSum k = kp_sum(w.x, w.y, w.z, C.tab);
-        G.trial[slot][lane] = {k.t, k.e, w.w};
+        if (!HYB) {
+            const KpSum k = kp_sum(w.x, w.y, w.z, C.tab);
+            G.trial[slot][lane] = {k.t, k.e, w.w};
+        }
         if (t == 0) {
             const FixDir f = direction_fix(spare_bits_1(w), spare_bits_2(w), C.tab);
             G.dir[lane] = {f.sth, f.cph, f.sph, f.cth, 0};
@@ -579,7 +593,7 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
                 G.sums[role - 1][0][lane] = make_longlong2(A[0], A[1]);
                 G.sums[role - 1][1][lane] = make_longlong2(A[2], A[3]);
             }
-        } else if (!HYB) {
+        } else {
             draw(C.stream(lex * 4u + MU), 0, 0);
         }
     }
@@ -593,7 +607,6 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     double qc = 0.0;
     Lambda L = {0, 0, 0};
     int32_t tr = -1;
-    uint32_t kd1 = 0, kd2 = 0;
     bool haar = false, wait = false, general = false;
     if (!MIR && !PLAQ && role == 0 && act) general = ((G.bad[0] | G.bad[1] | G.bad[2]) >> lane) & 1u;
     if (general) {
@@ -616,15 +629,14 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         haar = !fix_prepare<HYB>(C, A, &d, &qc);
         if (haar) {
             tr = 0;
+        } else if (HYB && !SPREAD) {
+            for (int t = 0; t < KP_CAP && tr < 0; ++t)
+                if (fix_try<HYB>(C, st.draw(TAG_TRIAL, (uint32_t)t), d.inv, d.ei, qc, &L)) tr = t + 1;
         } else if (HYB) {
-            U4 w = st.draw(TAG_TRIAL, 0u);
-            kd1 = spare_bits_1(w);
-            kd2 = spare_bits_2(w);
-            for (int t = 0; t < KP_CAP; w = st.draw(TAG_TRIAL, (uint32_t)++t))
-                if (fix_try<true>(C, w, d.inv, d.ei, qc, &L)) {
-                    tr = t + 1;
-                    break;
-                }
+            wait = true;
+            G.hyb.inv[lane] = d.inv;
+            G.hyb.qc[lane] = qc;
+            G.hyb.ei[lane] = d.ei;
         } else {
             const Trial64 a = G.trial[0][lane];
             L = kp_lambda(KpSum{a.t, a.e}, d.inv, d.ei);
@@ -632,7 +644,32 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
             else wait = true;
         }
     }
-    if (!HYB) {
+    if (HYB && SPREAD) {
+        for (int t0 = 0; t0 < KP_CAP; t0 += 4) {
+            if (role == 0) {
+                const uint32_t m = __ballot_sync(0xffffffffu, wait);
+                if (lane == 0) G.pend = m;
+            }
+            __syncthreads();
+            const uint32_t m = G.pend;
+            if (m == 0) break;
+            if ((m >> lane) & 1u) {
+                const U4 w = st.draw(TAG_TRIAL, (uint32_t)(t0 + role));
+                Lambda t;
+                const bool ok = fix_try<HYB>(C, w, G.hyb.inv[lane], G.hyb.ei[lane], G.hyb.qc[lane], &t);
+                G.trial[role][lane] = {t.P, t.qe, ok ? 1u : 0u};
+            }
+            __syncthreads();
+            for (int k = 0; k < 4 && wait; ++k) {
+                const Trial64 a = G.trial[k][lane];
+                if (a.w3) {
+                    L = lambda_of(a.t, a.e);
+                    tr = t0 + k + 1;
+                    wait = false;
+                }
+            }
+        }
+    } else if (!HYB) {
         // tests trials t0 .. t0 + n - 1 (slots t & 3) of the waiting links
         auto pick = [&](int t0, int n) {
             for (int k = 0; k < n && wait; ++k) {
@@ -678,12 +715,8 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
             U.store(MU, p, i, h);
             if (PLAQ) fix_from_link(h, un);
         } else if (tr > 0) {
-            if (HYB) {
-                new_link_fix(L, kd1, kd2, d.V, C.tab, un);
-            } else {
-                const Dir64 f = G.dir[lane];
-                new_link_dir_fix(L, {f.cth, f.sth, f.cph, f.sph}, d.V, un);
-            }
+            const Dir64 f = G.dir[lane];
+            new_link_dir_fix(L, {f.cth, f.sth, f.cph, f.sph}, d.V, un);
             U.store(MU, p, i, dq_link(un));
         } else {
             ncap = 1;
