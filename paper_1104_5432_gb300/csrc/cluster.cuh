@@ -44,7 +44,7 @@ __device__ __forceinline__ void chain_addresses(const LatDesc& D, uint32_t i, in
                                                 const LinkCheck& chk, uint32_t* ad)
 {
     const EoSite s(D, i, p);
-    int hp[4], hm[4];
+    uint32_t hp[4], hm[4];
     s.hops(hp, hm);
     auto put = [&](int slot, uint32_t e) {
         if (!chk.ok(0, 0, e)) e = 0;

@@ -70,8 +70,8 @@ __device__ __forceinline__ void fix_from_link(const Quat<double>& q, int64_t* U)
 
 // one staple term of U_mu(x) in the plane (nu, mu), added to A (fq_staple)
 template <typename LT>
-__device__ __forceinline__ void fix_term(const LT& U, int mu, int nu, int p, uint32_t i, int hpm,
-                                         int hpn, int hmn, bool lower, int64_t* A)
+__device__ __forceinline__ void fix_term(const LT& U, int mu, int nu, int p, uint32_t i, uint32_t hpm,
+                                         uint32_t hpn, uint32_t hmn, bool lower, int64_t* A)
 {
     const int q = p ^ 1;
     const FQuat x = U.fix(lower ? mu : nu, q, i + (lower ? hmn : hpm));
@@ -88,15 +88,15 @@ template <int MU, bool PLAQ, typename LT>
 __device__ __forceinline__ void fix_staple_sum(const LT& U, const EoSite& s, uint32_t i,
                                                int p, int64_t* A, int64_t* P)
 {
-    int hp[4], hm[4];
+    uint32_t hp[4], hm[4];
     s.hops(hp, hm);
     A[0] = A[1] = A[2] = A[3] = 0;
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
         constexpr int n0 = nu_of<MU>(0), n1 = nu_of<MU>(1), n2 = nu_of<MU>(2);
         const int nu = k == 0 ? n0 : (k == 1 ? n1 : n2);
-        const int hpn = k == 0 ? hp[n0] : (k == 1 ? hp[n1] : hp[n2]);
-        const int hmn = k == 0 ? hm[n0] : (k == 1 ? hm[n1] : hm[n2]);
+        const uint32_t hpn = k == 0 ? hp[n0] : (k == 1 ? hp[n1] : hp[n2]);
+        const uint32_t hmn = k == 0 ? hm[n0] : (k == 1 ? hm[n1] : hm[n2]);
         fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, false, A);
         fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, true, A);
         if (PLAQ && k == MU - 1) {
@@ -208,7 +208,7 @@ __device__ __noinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, u
 {
     const LT U(ctx.links, D, ctx.status);
     const EoSite s(D, i, p);
-    int hp[4], hm[4];
+    uint32_t hp[4], hm[4];
     s.hops(hp, hm);
     Quat<double> A = {0, 0, 0, 0}, P = A;
     for (int nu = 0, k = 0; nu < 4; ++nu) {
@@ -582,11 +582,11 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
         const EoSite s(D, i, p);
         lex = s.lex();
         if (role < 3) {
-            int hp[4], hm[4];
+            uint32_t hp[4], hm[4];
             s.hops(hp, hm);
             const int nu = nu_of<MU>(role);
-            const int hpn = nu == 0 ? hp[0] : (nu == 1 ? hp[1] : (nu == 2 ? hp[2] : hp[3]));
-            const int hmn = nu == 0 ? hm[0] : (nu == 1 ? hm[1] : (nu == 2 ? hm[2] : hm[3]));
+            const uint32_t hpn = nu == 0 ? hp[0] : (nu == 1 ? hp[1] : (nu == 2 ? hp[2] : hp[3]));
+            const uint32_t hmn = nu == 0 ? hm[0] : (nu == 1 ? hm[1] : (nu == 2 ? hm[2] : hm[3]));
             fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, false, A);
             fix_term(U, MU, nu, p, i, hp[MU], hpn, hmn, true, A);
             if (role > 0) {

@@ -89,7 +89,7 @@ __device__ __forceinline__ constexpr int nu_of(int k) { return k + (k >= MU ? 1 
 // of U_mu(x) in the plane (nu, mu), as the FP64 sequence forms them
 template <typename T, typename LT>
 __device__ __forceinline__ Quat<T> staple_term(const LT& U, int mu, int nu, int p, uint32_t i,
-                                               const int* hp, const int* hm, bool lower)
+                                               const uint32_t* hp, const uint32_t* hm, bool lower)
 {
     const int q = p ^ 1;
     if (!lower) {
@@ -110,7 +110,7 @@ template <typename T, int MU, bool PLAQ, typename LT>
 __device__ __forceinline__ void staple_sum(const LT& U, const EoSite& s, uint32_t i, int p,
                                            Quat<T>& A, Quat<T>& P)
 {
-    int hp[4], hm[4];
+    uint32_t hp[4], hm[4];
     s.hops(hp, hm, LT::UNIT);
     const int q = p ^ 1;
     const uint32_t o = i * (uint32_t)LT::UNIT;
@@ -494,8 +494,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* m, uint32_t parity)
 // storage index of load slot k (ν by ν: a, b, c, d, e, f as in staple_sum)
 // and its (direction, parity) plane
 template <int MU>
-__device__ __forceinline__ uint32_t stage_site(int k, int p, uint32_t i, const int* hp,
-                                               const int* hm, int* plane)
+__device__ __forceinline__ uint32_t stage_site(int k, int p, uint32_t i, const uint32_t* hp,
+                                               const uint32_t* hm, int* plane)
 {
     const int nu = nu_of<MU>(k / 6), q = p ^ 1;
     switch (k % 6) {
@@ -512,7 +512,7 @@ __device__ __forceinline__ uint32_t stage_site(int k, int p, uint32_t i, const i
 // name the rows); the caller waits on m
 template <int MU>
 __device__ __forceinline__ void stage_issue(const Links<float>& U, int p, uint32_t i,
-                                            const int* hp, const int* hm,
+                                            const uint32_t* hp, const uint32_t* hm,
                                             float4 (*rows)[32], uint64_t* m)
 {
     mbar_expect_tx(m, STAGE_ROWS * STAGE_ROW_BYTES);
@@ -527,7 +527,7 @@ __device__ __forceinline__ void stage_issue(const Links<float>& U, int p, uint32
 // staple_sum's FP32 arithmetic on the staged rows
 template <int MU, bool PLAQ>
 __device__ __forceinline__ void staple_sum_staged(const float4 (*rows)[32], int p, uint32_t i,
-                                                  const int* hp, const int* hm, Quat<float>& A,
+                                                  const uint32_t* hp, const uint32_t* hm, Quat<float>& A,
                                                   Quat<float>& P)
 {
     auto ld = [&](int k) {
@@ -698,7 +698,7 @@ hb_phase_queue_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
                 const EoSite s = SLAB ? EoSite::from_slab(D, j, p, &i) : EoSite(D, j, p);
                 if constexpr (STAGE) {
                     if (staged) {
-                        int hp[4], hm[4];
+                        uint32_t hp[4], hm[4];
                         s.hops(hp, hm);
                         float4 (*rows)[32] = srows[threadIdx.x >> 5];
                         // the previous round's reads are done before new copies land
@@ -782,7 +782,7 @@ __device__ __forceinline__ void staple_sum_pair(const PairLinks& U, const EoSite
                                                 Quat<float2>& P)
 {
     const int q = p ^ 1;
-    int hp[4], hm[4];
+    uint32_t hp[4], hm[4];
     s.hops(hp, hm);
     const uint32_t e_pmu = i + hp[MU];
     const float2 z = splat<float2>(0.0f);

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(TPB) plaquette_kernel(Ctx ctx)
         const LT U(ctx.links, D, ctx.status);
         int p;
         const EoSite s = EoSite::from_lex(D, lex, &p);
-        int hp[4], hm[4];
+        uint32_t hp[4], hm[4];
         s.hops(hp, hm, LT::UNIT);
         const uint32_t o = (lex >> 1) * (uint32_t)LT::UNIT;
         const int q = p ^ 1;
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(TPB) plaquette_fix_kernel(Ctx ctx)
         const Links<double> U(ctx.links, D, ctx.status);
         int p;
         const EoSite s = EoSite::from_lex(D, lex, &p);
-        int hp[4], hm[4];
+        uint32_t hp[4], hm[4];
         s.hops(hp, hm);
         const uint32_t eo = lex >> 1;
         const int q = p ^ 1;

@@ -305,20 +305,22 @@ struct EoSite {
     }
 
     // eo offsets of x + e_d (plus) and x - e_d (minus), wrap included, in units
-    // of 1 / unit sites (modulo 2^32)
-    __device__ __forceinline__ void hops(int* plus, int* minus, int unit = 1) const
+    // of 1 / unit sites, modulo 2^32 (unsigned: a plane of 2^28 links of 16
+    // bytes is 2^32 units long)
+    __device__ __forceinline__ void hops(uint32_t* plus, uint32_t* minus, uint32_t unit = 1) const
     {
-        const int b = c[0] & 1;
-        const int nh = (int)Nh * unit;
-        plus[0] = b ? (c[0] == Ns - 1 ? unit - nh : unit) : 0;
-        minus[0] = b ? 0 : (c[0] == 0 ? nh - unit : -unit);
-        int st = nh;
+        const bool b = c[0] & 1;
+        const uint32_t nh = Nh * unit;
+        plus[0] = b ? (c[0] == Ns - 1 ? unit - nh : unit) : 0u;
+        minus[0] = b ? 0u : (c[0] == 0 ? nh - unit : 0u - unit);
+        uint32_t st = nh;
 #pragma unroll
         for (int d = 1; d < 4; ++d) {
             const int L = d == 3 ? Nt : Ns;
-            plus[d] = c[d] == L - 1 ? -(L - 1) * st : st;
-            minus[d] = c[d] == 0 ? (L - 1) * st : -st;
-            st *= Ns;
+            const uint32_t wrap = (uint32_t)(L - 1) * st;
+            plus[d] = c[d] == L - 1 ? 0u - wrap : st;
+            minus[d] = c[d] == 0 ? wrap : 0u - st;
+            st *= (uint32_t)Ns;
         }
     }
 

@@ -1448,6 +1448,41 @@ def test_small_lattices_from_two_host_threads(dtype, big):
         assert got[k][1] == stats
 
 
+@pytest.mark.parametrize("shape", [0, 13])
+def test_largest_lattice_of_32_bit_link_offsets(shape):
+    """128^3 x 256 FP32 (2^29 sites, 34 GB of links): a (mu, parity) plane is
+    2^32 bytes long, so the offsets of the wrapping hops reach beyond 2^31 and
+    hold modulo 2^32.  The first phase from the hot start, links sampled over
+    the whole lattice and in its first and last time slices, against the
+    oracle's draws; then one sweep, whose fused plaquette (every direction's
+    hops, in the phase kernels) equals the stand-alone one."""
+    Ns, Nt, seed = 128, 256, 3
+    V = Ns ** 3 * Nt
+    lat = lattice(Ns, Nt, su2.F32)
+    lat.set_launch_config(shape)
+    lat.init(su2.HOT, seed)
+    lat.heatbath_phase(2.5, 0, 0, seed)
+    lat.sync()
+    rng = np.random.default_rng(2)
+    lex = np.concatenate([rng.integers(0, V, 200), rng.integers(0, Ns ** 3, 200),
+                          V - 1 - rng.integers(0, Ns ** 3, 200)])
+    x, y, z, t = lex % Ns, (lex // Ns) % Ns, (lex // Ns ** 2) % Ns, lex // Ns ** 3
+    lex = lex[(x + y + z + t) % 2 == 0]
+    got = sampled_links(lat, V, lex, su2.F32)
+    fused = lat.heatbath(2.5, 1, seed)[0, 0]
+    alone = lat.plaquette()[0]
+    st = lat.stats()
+    lat.close()
+    torch.cuda.empty_cache()
+    assert st["updates"] == V // 2 + 4 * V and st["cap_hits"] == 0
+    assert abs(fused - alone) <= 1e-7
+    flips = 0
+    for k, i in enumerate(lex):
+        u, tr = O.heatbath_link_hot(Ns, Nt, seed, 2.5, 0, int(i), seed, 0)
+        flips += float(np.max(np.abs(got[k, 0] - u))) > 2e-5
+    assert len(lex) > 200 and flips <= 1
+
+
 @pytest.mark.parametrize("shape", [0, 7])
 def test_lattice_beyond_32_bit_link_offsets(shape):
     """128^3 x 258 FP32 (2^29 + 2^22 sites, 35 GB of links): a (mu, parity)
