@@ -21,7 +21,8 @@ LIB = os.path.join(PKG, "libsu2gb300.so")
 SOURCES = ["heatbath.cu", "observables.cu", "links.cu", "api.cu", "plaquette_static.cu",
            "selftest.cu", "cluster.cu", "cluster64.cu"]
 # heatbath_shapes.cu once per pair of launch shapes of the FP32 rows of the
-# 14-entry table in csrc/su2_internal.h (FP32, FP32 site pairs), heatbath_fp64.cu
+# 14-entry table in csrc/su2_internal.h (FP32, FP32 site pairs, and FP32 again
+# with 64-bit link indices for lattices of more than 2^29 sites), heatbath_fp64.cu
 # once per kernel and sampler of the FP64 row: (object name, defines, flags);
 # the source is the name's first part.
 # The FP32 phase kernels flush denormals to zero: none can occur on their
@@ -29,10 +30,10 @@ SOURCES = ["heatbath.cu", "observables.cu", "links.cu", "api.cu", "plaquette_sta
 # 0, the log series is evaluated in Horner form, alpha and 1/(2 alpha) stay
 # normal down to beta = 1e-9), and without denormal handling the division
 # and square-root sequences are shorter (2% at 64^4).
-ROW_NAMES = ("f32", "f64", "f32pairs")
-SHAPE_UNITS = [(f"heatbath_shapes_{ROW_NAMES[row]}_{k}",
-                (f"SU2_ROW={row}", f"SU2_FIRST={k}"), ("-ftz=true",))
-               for row in (0, 2) for k in range(0, 14, 2)]
+SHAPE_UNITS = [(f"heatbath_shapes_{name}_{k}",
+                (f"SU2_ROW={row}", f"SU2_FIRST={k}", f"SU2_WIDE={wide}"), ("-ftz=true",))
+               for name, row, wide in (("f32", 0, 0), ("f32pairs", 2, 0), ("f32wide", 0, 1))
+               for k in range(0, 14, 2)]
 SHAPE_UNITS += [(f"heatbath_fp64_{kind}_{hyb}",
                  (f"SU2_KIND={kind}", f"SU2_HYB={hyb}"), ())
                 for kind in range(6) for hyb in (0, 1)]

@@ -128,7 +128,7 @@ struct su2_lattice {
     size_t off_status = 0, off_desc = 0, off_sstart = 0, off_spstart = 0;
     size_t off_plaq = 0, off_obs = 0, off_field = 0, off_ring = 0, off_res = 0, off_stage = 0;
     size_t off_chunks = 0, off_tickets = 0, off_acc = 0, off_tslots = 0, off_fp64tab = 0, off_fixtab = 0, off_mirror = 0, off_oflag = 0;
-    bool wide = false;              // some lattice of more than 2^29 sites
+    bool wide = false;              // some lattice of more than 2 OFF32_MAX_VH sites
     bool mirror = false;            // FP64: the work buffer holds a fixed-point copy of the links
     uint32_t max_chunks = 1;
     size_t res_doubles = 0;
@@ -262,7 +262,7 @@ int layout(su2_lattice* L)
         const uint64_t Ns = (uint64_t)L->Ns[l], Nt = (uint64_t)L->Nt[l];
         L->Vs[l] = Ns * Ns * Ns;
         L->V[l] = L->Vs[l] * Nt;
-        L->wide = L->wide || L->V[l] > (uint64_t(1) << 29);
+        L->wide = L->wide || L->V[l] / 2 > OFF32_MAX_VH;
         L->link_off[l] = lb;
         lb += align256(4 * L->V[l] * link_size);
         L->field_off[l] = fo;
@@ -413,7 +413,7 @@ int set_params(su2_lattice* L, const double* betas, double beta, const uint64_t*
 int record_measure(su2_lattice* L, int rmax, cudaStream_t s)
 {
     double* acc = L->acc_dev();
-    SU2_CUDA(launch_polyakov(L->ctx, L->row, L->wide, acc, acc + L->n, 1, s));
+    SU2_CUDA(launch_polyakov(L->ctx, L->row, acc, acc + L->n, 1, s));
     SU2_CUDA(launch_correlator(L->ctx, L->dtype, rmax, acc + 2 * L->n, 1, s));
     return SU2_OK;
 }
@@ -1114,6 +1114,7 @@ int su2_bind_memory(su2_lattice* lat, void* links, size_t link_bytes, void* work
     c.status = reinterpret_cast<uint32_t*>(w + lat->off_status);
     c.obs_flag = reinterpret_cast<uint32_t*>(w + lat->off_oflag);
     c.n = lat->n;
+    c.wide = lat->wide;
     c.phase_blocks = lat->phase_blocks[0];
     c.site_blocks = lat->site_blocks;
     c.spat_blocks = lat->spat_blocks;
@@ -1234,7 +1235,7 @@ int su2_plaquette(su2_lattice* lat, double* out)
     DeviceGuard dg(lat->device);
     const bool dev = is_device_ptr(out);
     double* tgt = dev ? out : lat->res_dev();
-    SU2_CUDA(launch_plaquette(lat->ctx, lat->row, lat->wide, tgt, lat->stream));
+    SU2_CUDA(launch_plaquette(lat->ctx, lat->row, tgt, lat->stream));
     if (!dev) return finish_output(lat, out, tgt, lat->n);
     return SU2_OK;
 }
@@ -1249,7 +1250,7 @@ int su2_polyakov_loop(su2_lattice* lat, double* out_signed, double* out_abs)
         return fail(SU2_E_INVAL, "out_signed and out_abs must both be host or both device");
     double* ts = dev ? out_signed : lat->res_dev();
     double* ta = out_abs ? (dev ? out_abs : lat->res_dev() + lat->n) : nullptr;
-    SU2_CUDA(launch_polyakov(lat->ctx, lat->row, lat->wide, ts, ta, 0, lat->stream));
+    SU2_CUDA(launch_polyakov(lat->ctx, lat->row, ts, ta, 0, lat->stream));
     if (!dev) {
         const double* host = nullptr;
         const int rc = fetch_status(lat, ts, sizeof(double) * 2 * lat->n, &host);
@@ -1273,7 +1274,7 @@ int su2_polyakov_correlator(su2_lattice* lat, int rmax, double* out, int accumul
     const size_t cnt = (size_t)lat->n * (rmax + 1);
     double* scratch = lat->res_dev();  // [2n] Polyakov means, then correlator rows
     double* tgt = dev ? out : scratch + 2 * lat->n;
-    SU2_CUDA(launch_polyakov(lat->ctx, lat->row, lat->wide, nullptr, nullptr, 0, lat->stream));
+    SU2_CUDA(launch_polyakov(lat->ctx, lat->row, nullptr, nullptr, 0, lat->stream));
     if (!dev && accumulate)
         SU2_CUDA(cudaMemcpyAsync(tgt, out, sizeof(double) * cnt, cudaMemcpyHostToDevice,
                                  lat->stream));

@@ -124,7 +124,7 @@ __global__ void set_params_kernel(Ctx ctx, ParamChunk pc)
 
 // one pair of FP32 launch shapes per instantiation of heatbath_shapes.cu, one
 // FP64 kernel and sampler per instantiation of heatbath_fp64.cu
-template <int ROW, int FIRST>
+template <int ROW, int FIRST, bool WIDE>
 cudaError_t launch_phase_pair(const Ctx& c, int cfg, int mu, int parity, bool plaq, int32_t* dbg,
                               bool hyb, cudaStream_t s);
 template <int KIND, bool HYB>
@@ -155,15 +155,19 @@ cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, boo
     }
     using Fn = cudaError_t (*)(const Ctx&, int, int, int, bool, int32_t*, bool, cudaStream_t);
     static_assert(NUM_LAUNCH_CFG == 14 && NUM_ROWS == 3, "one entry per pair of shapes below");
-    static const Fn pairs[2][NUM_LAUNCH_CFG / 2] = {
-        {launch_phase_pair<0, 0>, launch_phase_pair<0, 2>, launch_phase_pair<0, 4>,
-         launch_phase_pair<0, 6>, launch_phase_pair<0, 8>, launch_phase_pair<0, 10>,
-         launch_phase_pair<0, 12>},
-        {launch_phase_pair<2, 0>, launch_phase_pair<2, 2>, launch_phase_pair<2, 4>,
-         launch_phase_pair<2, 6>, launch_phase_pair<2, 8>, launch_phase_pair<2, 10>,
-         launch_phase_pair<2, 12>},
+    static const Fn pairs[3][NUM_LAUNCH_CFG / 2] = {
+        {launch_phase_pair<0, 0, false>, launch_phase_pair<0, 2, false>, launch_phase_pair<0, 4, false>,
+         launch_phase_pair<0, 6, false>, launch_phase_pair<0, 8, false>, launch_phase_pair<0, 10, false>,
+         launch_phase_pair<0, 12, false>},
+        {launch_phase_pair<2, 0, false>, launch_phase_pair<2, 2, false>, launch_phase_pair<2, 4, false>,
+         launch_phase_pair<2, 6, false>, launch_phase_pair<2, 8, false>, launch_phase_pair<2, 10, false>,
+         launch_phase_pair<2, 12, false>},
+        {launch_phase_pair<0, 0, true>, launch_phase_pair<0, 2, true>, launch_phase_pair<0, 4, true>,
+         launch_phase_pair<0, 6, true>, launch_phase_pair<0, 8, true>, launch_phase_pair<0, 10, true>,
+         launch_phase_pair<0, 12, true>},
     };
-    return pairs[row == ROW_F32_PAIRS][cfg >> 1](c, cfg, mu, parity, plaq, dbg_trials, hybrid, s);
+    const int table = row == ROW_F32_PAIRS ? 1 : (c.wide ? 2 : 0);
+    return pairs[table][cfg >> 1](c, cfg, mu, parity, plaq, dbg_trials, hybrid, s);
 }
 
 cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s)

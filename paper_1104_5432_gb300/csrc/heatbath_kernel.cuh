@@ -351,57 +351,12 @@ __device__ __forceinline__ int32_t update_link(const LT& U, const LatDesc& D, co
 }
 
 // ---------------------------------------------------------------------------
-// lattices of more than 2^29 sites: 64-bit link indices, one link at a time
-// ---------------------------------------------------------------------------
-template <bool HYB>
-__device__ __noinline__ int32_t wide_link(const Ctx& ctx, const LatDesc& D, uint32_t j, bool slab, int mu,
-                                          int p, float* plaq, uint32_t* lex)
-{
-    const WideLinks U(ctx.links, D, ctx.status);
-    uint32_t i = j;
-    const EoSite s = slab ? EoSite::from_slab(D, j, p, &i) : EoSite(D, j, p);
-    Quat<float> un, P = {0.f, 0.f, 0.f, 0.f};
-    int32_t tr;
-    switch (mu) {
-    case 0: tr = update_link<float, 0, false, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
-    case 1: tr = update_link<float, 1, true, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
-    case 2: tr = update_link<float, 2, true, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
-    default: tr = update_link<float, 3, true, HYB>(U, D, s, i, p, D.sweep, &un, &P); break;
-    }
-    if (tr >= 0) U.store(mu, p, i, un);
-    else un = U.load_rw(mu, p, i);
-    *plaq = add_(*plaq, qretr(un, P));
-    *lex = s.lex();
-    return tr;
-}
-// a block's tiles of NT R positions, as the kernels below take them
-template <int MU, bool PLAQ, int NT, bool HYB>
-__device__ __noinline__ void wide_links(const Ctx& ctx, int l, uint32_t blk0, uint32_t tile, uint32_t nb,
-                                        int R, bool slab, int p, int32_t* dbg)
-{
-    const LatDesc& D = ctx.desc[l];
-    float plaq = 0.0f;
-    uint32_t ntrial = 0, ncap = 0, lex;
-    const uint32_t ntiles = (D.Vh + NT * (uint32_t)R - 1) / (NT * (uint32_t)R);
-    do {
-        for (int r = 0; r < R; ++r) {
-            const uint32_t j = tile * (NT * (uint32_t)R) + (uint32_t)r * NT + threadIdx.x;
-            if (j >= D.Vh) break;
-            const int32_t tr = wide_link<HYB>(ctx, D, j, slab, MU, p, &plaq, &lex);
-            ncap += tr < 0;
-            ntrial += tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
-            if (dbg) dbg[lex] = tr;
-        }
-        tile += nb;
-    } while (nb && tile < ntiles);
-    __syncwarp();
-    warp_totals<float, MU, PLAQ, NT>(ctx, l, blk0, D.Vh, plaq, ntrial, ncap);
-}
-
-// ---------------------------------------------------------------------------
 // one link per thread
 // ---------------------------------------------------------------------------
-template <typename T, int MU, bool PLAQ, bool DBG, int NT, int MINB, bool SLAB, bool HYB>
+// LT: the links, with 32-bit offsets or (lattices of more than 2^29 sites,
+// compiled apart) 64-bit indices: 128^3 x 258, shape 13, 49.9 ms a sweep; with
+// one link at a time behind a branch in these kernels 62
+template <typename T, int MU, bool PLAQ, bool DBG, int NT, int MINB, bool SLAB, bool HYB, typename LT>
 __global__ void __launch_bounds__(NT, MINB)
 hb_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
@@ -410,11 +365,7 @@ hb_phase_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const uint32_t Vh = D.Vh;
     const uint32_t blk0 = first_block(ctx.phase_start, l);
     const uint32_t j = (blockIdx.x - blk0) * NT + threadIdx.x;  // traversal position
-    if (Vh > OFF32_MAX_VH) {
-        wide_links<MU, PLAQ, NT, HYB>(ctx, l, blk0, blockIdx.x - blk0, 0u, 1, SLAB, p, dbg);
-        return;
-    }
-    const Links<T> U(ctx.links, D, ctx.status);
+    const LT U(ctx.links, D, ctx.status);
 
     T plaq = T(0);
     uint32_t ntrial = 0, ncap = 0;
@@ -571,7 +522,7 @@ struct RetryQueue {
 };
 
 template <typename T, int MU, bool PLAQ, bool DBG, int NT, int MINB, bool SLAB, bool HYB, int R,
-          bool PERSIST, bool STAGE = false>
+          bool PERSIST, bool STAGE, typename LT>
 __global__ void __launch_bounds__(NT, MINB)
 hb_phase_queue_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
@@ -593,11 +544,7 @@ hb_phase_queue_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const uint32_t nb = PERSIST ? __ldg(ctx.phase_start + l + 1) - blk0 : 0u;
     const uint32_t ntiles = PERSIST ? (Vh + NT * R - 1) / (NT * R) : 0u;
     uint32_t tile = blockIdx.x - blk0;
-    if (Vh > OFF32_MAX_VH) {
-        wide_links<MU, PLAQ, NT, HYB>(ctx, l, blk0, tile, nb, R, SLAB, p, dbg);
-        return;
-    }
-    const Links<T> U(ctx.links, D, ctx.status);
+    const LT U(ctx.links, D, ctx.status);
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
     Queue& Q = sq[threadIdx.x >> 5];
@@ -999,23 +946,25 @@ hb_pair_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 // links -- or with PAIRS, R site pairs -- per thread, persistent or not) of
 // the phase kernel; the grid covers ctx.phase_blocks blocks of NT R links
 // or pairs (fewer, each walking several tiles, for a persistent shape on a
-// single lattice).
+// single lattice).  WIDE: links indexed in 64 bits.
 template <typename T, int NT, int MINB, bool SLAB, int R = 1, bool PERSIST = false,
-          bool PAIRS = false, bool STAGE = false>
+          bool PAIRS = false, bool STAGE = false, bool WIDE = false>
 cudaError_t launch_phase_shape(const Ctx& c, int mu, int parity, bool plaq, int32_t* dbg,
                                bool hyb, cudaStream_t s)
 {
     // the fused plaquette exists only in the odd phases with mu >= 1
     const bool pl = plaq && parity == 1 && mu >= 1;
     const dim3 grid(c.phase_blocks), block(NT);
+    using LT = std::conditional_t<WIDE, WideLinks, Links<T>>;
 #define SU2_K(MUV, PL, DB, H)                                                                   \
     if constexpr (PAIRS)                                                                        \
         hb_pair_kernel<MUV, PL, DB, NT, MINB, SLAB, H, R, PERSIST><<<grid, block, 0, s>>>(      \
             c, parity, dbg);                                                                    \
     else if constexpr (R == 1 && !PERSIST && !STAGE)                                            \
-        hb_phase_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H><<<grid, block, 0, s>>>(c, parity, dbg); \
+        hb_phase_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H, LT>                                  \
+            <<<grid, block, 0, s>>>(c, parity, dbg);                                            \
     else                                                                                        \
-        hb_phase_queue_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H, R, PERSIST, STAGE>              \
+        hb_phase_queue_kernel<T, MUV, PL, DB, NT, MINB, SLAB, H, R, PERSIST, STAGE, LT>          \
             <<<grid, block, 0, s>>>(c, parity, dbg)
 #define SU2_LAUNCH_H(MUV, H)                                    \
     do {                                                        \

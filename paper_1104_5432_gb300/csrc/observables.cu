@@ -269,7 +269,7 @@ finalize_kernel(Ctx ctx, const uint32_t* __restrict__ start, uint32_t stride, in
     }
 }
 
-cudaError_t launch_plaquette(const Ctx& c, int row, bool wide, double* out_dev, cudaStream_t s)
+cudaError_t launch_plaquette(const Ctx& c, int row, double* out_dev, cudaStream_t s)
 {
     const unsigned g = c.site_blocks;
     if (row == ROW_F64) {
@@ -277,7 +277,7 @@ cudaError_t launch_plaquette(const Ctx& c, int row, bool wide, double* out_dev, 
         plaquette_kernel<double, Links<double>, true><<<g, TPB, 0, s>>>(c);
     } else if (row == ROW_F32_PAIRS) {
         plaquette_kernel<float, PairLinks, false><<<g, TPB, 0, s>>>(c);
-    } else if (wide) {
+    } else if (c.wide) {
         plaquette_kernel<float, WideLinks, false><<<g, TPB, 0, s>>>(c);
     } else {
         plaquette_kernel<float, Links<float>, false><<<g, TPB, 0, s>>>(c);
@@ -287,13 +287,13 @@ cudaError_t launch_plaquette(const Ctx& c, int row, bool wide, double* out_dev, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_polyakov(const Ctx& c, int row, bool wide, double* out_signed_dev,
-                            double* out_abs_dev, int accumulate, cudaStream_t s)
+cudaError_t launch_polyakov(const Ctx& c, int row, double* out_signed_dev, double* out_abs_dev,
+                            int accumulate, cudaStream_t s)
 {
     const unsigned g = c.spat_blocks;
     if (row == ROW_F64) polyakov_kernel<double, Links<double>><<<g, TPB, 0, s>>>(c);
     else if (row == ROW_F32_PAIRS) polyakov_kernel<float, PairLinks><<<g, TPB, 0, s>>>(c);
-    else if (wide) polyakov_kernel<float, WideLinks><<<g, TPB, 0, s>>>(c);
+    else if (c.wide) polyakov_kernel<float, WideLinks><<<g, TPB, 0, s>>>(c);
     else polyakov_kernel<float, Links<float>><<<g, TPB, 0, s>>>(c);
     if (out_signed_dev)
         finalize_kernel<<<dim3(c.n, 1), TPB, 0, s>>>(c, c.spat_start, c.spat_blocks, 1, 1,

@@ -110,6 +110,13 @@ constexpr uint32_t STATUS_BOUNDS = 2u;  // bounds-checked builds only
 constexpr uint32_t STATUS_STAGE = 4u;   // a bulk copy of neighbour rows did not arrive in time
 constexpr int SWEEP_CHUNK = TPB * 8;   // plaquette partials summed per sweep_end block
 constexpr int MAX_RMAX = 128;          // largest correlator separation
+// Largest links per (mu, parity) whose 16-byte links a 32-bit byte offset
+// reaches: FP32 lattices of at most 2^29 sites.  Handles with a larger one
+// index links in 64 bits (WideLinks; a test build lowers the line).
+#ifndef SU2_OFF32_MAX_VH
+#define SU2_OFF32_MAX_VH (1u << 28)
+#endif
+constexpr uint32_t OFF32_MAX_VH = SU2_OFF32_MAX_VH;
 constexpr int TRIAL_SLOTS = 64;        // per-lattice trial counters (spread atomics)
 // reasons for an FP64 lattice to take the FP64 sequence: some link is not a
 // unit quaternion (unit_check_kernel, looked at again after each sweep), the
@@ -170,6 +177,7 @@ struct Ctx {
     uint32_t phase_blocks, site_blocks, spat_blocks;
     uint32_t max_chunks;
     uint32_t phase_wpb;            // warps per phase block of this launch shape
+    uint32_t wide;                 // some lattice has more than 2 OFF32_MAX_VH sites
     uint32_t look;                 // FP64 single phases: each update looks at the links it reads
 };
 
@@ -267,11 +275,11 @@ cudaError_t launch_links_from_canonical(const Ctx& c, int dtype, int l, uint32_t
                                         uint32_t nsite, const void* src, int cdtype,
                                         cudaStream_t s, bool pairs_whole = false);
 cudaError_t launch_gauge(const Ctx& c, int dtype, int l, uint32_t V, uint64_t seed, cudaStream_t s);
-// row: the links' layout; wide: some lattice of more than 2^29 sites.
+// row: the links' layout
 // launch_polyakov with a null out_signed_dev fills the field only.
-cudaError_t launch_plaquette(const Ctx& c, int row, bool wide, double* out_dev, cudaStream_t s);
-cudaError_t launch_polyakov(const Ctx& c, int row, bool wide, double* out_signed_dev,
-                            double* out_abs_dev, int accumulate, cudaStream_t s);
+cudaError_t launch_plaquette(const Ctx& c, int row, double* out_dev, cudaStream_t s);
+cudaError_t launch_polyakov(const Ctx& c, int row, double* out_signed_dev, double* out_abs_dev,
+                            int accumulate, cudaStream_t s);
 cudaError_t launch_correlator(const Ctx& c, int dtype, int rmax, double* out_dev, int accumulate,
                               cudaStream_t s);
 

@@ -74,9 +74,7 @@ template <> struct Links<float> {
     }
 };
 
-// Largest links per (mu, parity) whose 16-byte links a 32-bit byte offset
-// reaches (lattices of at most 2^29 sites); WideLinks for the others.
-constexpr uint32_t OFF32_MAX_VH = 1u << 28;
+// 64-bit indices, for planes of more than 4 GiB
 struct WideLinks : Links<float> {
     using Links<float>::Links;
     static constexpr int UNIT = 1;
