@@ -3,6 +3,8 @@
 // kernel and the dispatch of the phase kernels (heatbath_kernel.cuh,
 // instantiated per pair of launch shapes and precision by
 // heatbath_shapes.cu).
+#include <algorithm>
+
 #include "su2_internal.h"
 #include "su2_mirror.cuh"
 #include "su2_reduce.cuh"
@@ -38,23 +40,35 @@ __global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx, bool mirror)
     if (eo < D->Vh && !unit_links_at(ctx, *D, eo, mirror)) D->general = GENERAL_LINKS;
 }
 
-// the same by one block, after a sweep of a lattice that failed the check:
-// once every link has been updated the lattice takes the fixed-point path
-__device__ void unit_recheck(const Ctx& ctx, LatDesc* D)
+// The same by `nb` blocks after a sweep of a lattice that failed the check:
+// once every link has been updated the lattice takes the fixed-point path.  The
+// last block to finish (the counter D->recheck) clears the lattice's flag, so
+// every block has read it by then.  (By one block a sweep of 64^4 with one bad
+// link took 254 ms in all instead of 56.)
+constexpr unsigned RECHECK_BLOCKS = 304;  // over all lattices, two an SM
+__device__ void unit_recheck(const Ctx& ctx, LatDesc* D, uint32_t nb)
 {
     bool ok = true;
-    for (uint32_t eo = threadIdx.x; eo < D->Vh; eo += TPB)
+    for (uint32_t eo = blockIdx.x * TPB + threadIdx.x; eo < D->Vh; eo += nb * TPB)
         if (!unit_links_at(ctx, *D, eo, ctx.mirror != nullptr)) ok = false;
-    if (__syncthreads_and(ok) && threadIdx.x == 0) D->general = 0u;
+    ok = __syncthreads_and(ok);
+    if (threadIdx.x == 0) {
+        const uint32_t mine = ok ? 1u : 0x10001u, sum = atomicAdd(&D->recheck, mine) + mine;
+        if ((sum & 0xFFFFu) == nb) {
+            D->recheck = 0u;
+            if (sum >> 16 == 0u) D->general = 0u;
+        }
+    }
 }
 
 // Finishes a sweep: the fixed-order sum of the fused plaquette partials and
 // the lattice's sweep counter.  Grid (chunks, lattices); each block sums
 // SWEEP_CHUNK partials of its lattice, the last block of a lattice to finish
 // (ticket counter) adds the chunk sums in chunk order.
-// FP64 lattices with non-unit links are looked at again (F64).
+// FP64 lattices with non-unit links are looked at again (F64), by the first
+// nrecheck blocks of each (the grid has at least as many).
 template <bool PLAQ, bool F64>
-__global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
+__global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx, uint32_t nrecheck)
 {
     __shared__ double sred[TPB / 32];
     __shared__ int s_last;
@@ -62,9 +76,10 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
     LatDesc* D = ctx.desc + l;
     if (!PLAQ) {
         if (blockIdx.x == 0 && threadIdx.x == 0) D->sweep += 1;
-        if (F64 && D->general == GENERAL_LINKS) unit_recheck(ctx, D);
+        if (F64 && D->general == GENERAL_LINKS) unit_recheck(ctx, D, nrecheck);
         return;
     }
+    if (F64 && blockIdx.x < nrecheck && D->general == GENERAL_LINKS) unit_recheck(ctx, D, nrecheck);
     // partials are per warp: lattice l owns warps [b0, b0 + nb) of each slot
     const uint32_t b0 = ctx.phase_start[l] * ctx.phase_wpb;
     const uint32_t nb = ctx.phase_start[l + 1] * ctx.phase_wpb - b0;
@@ -102,7 +117,6 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx)
         if (D->plaq_out) D->plaq_out[k] = P;
         D->sweep += 1;
     }
-    if (F64 && D->general == GENERAL_LINKS) unit_recheck(ctx, D);
 }
 
 // Per-call parameters go in by value (no host-to-device copy); the
@@ -172,12 +186,15 @@ cudaError_t launch_phase(const Ctx& c, int row, int cfg, int mu, int parity, boo
 
 cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s)
 {
-    const dim3 grid(plaq ? c.max_chunks : 1u, c.n);
+    // a block for each TPB of an average lattice's Vh (site_blocks count V)
+    const unsigned n = (unsigned)c.n, most = std::max(1u, RECHECK_BLOCKS / n);
+    const unsigned nrecheck = fp64 ? std::min(most, std::max(1u, c.site_blocks / (2 * n))) : 1u;
+    const dim3 grid(std::max(plaq ? c.max_chunks : 1u, nrecheck), n);
     const unsigned nt = plaq || fp64 ? TPB : 32;
-    if (fp64 && plaq) sweep_end_kernel<true, true><<<grid, nt, 0, s>>>(c);
-    else if (fp64) sweep_end_kernel<false, true><<<grid, nt, 0, s>>>(c);
-    else if (plaq) sweep_end_kernel<true, false><<<grid, nt, 0, s>>>(c);
-    else sweep_end_kernel<false, false><<<grid, nt, 0, s>>>(c);
+    if (fp64 && plaq) sweep_end_kernel<true, true><<<grid, nt, 0, s>>>(c, nrecheck);
+    else if (fp64) sweep_end_kernel<false, true><<<grid, nt, 0, s>>>(c, nrecheck);
+    else if (plaq) sweep_end_kernel<true, false><<<grid, nt, 0, s>>>(c, nrecheck);
+    else sweep_end_kernel<false, false><<<grid, nt, 0, s>>>(c, nrecheck);
     return cudaGetLastError();
 }
 

@@ -151,6 +151,7 @@ struct LatDesc {
     uint64_t sweep_base;    // sweep index stored at plaq_out[0]
     double* plaq_out;       // device, nullable
     uint32_t general;       // FP64: why the sweeps take the FP64 sequence (GENERAL_*), or 0
+    uint32_t recheck;       // blocks done with unit_recheck, and << 16 those that failed (zero between)
     // advanced by the kernels
     uint64_t sweep;         // cumulative sweep counter
     unsigned long long trials, updates, caps;

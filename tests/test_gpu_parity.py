@@ -1285,6 +1285,35 @@ def test_fp64_lattice_with_non_unit_links(cfg):
     np.testing.assert_allclose(out[0][1], rplaq, rtol=1e-13, atol=0)
 
 
+@pytest.mark.parametrize("cfg,plaq", [(1, True), (1, None), (8, True), (11, None), (13, True)])
+def test_fp64_non_unit_links_are_looked_at_again_by_many_blocks(cfg, plaq):
+    """16^4 and 4^4 FP64 in a batch, and 16^4 alone, with one link scaled: after
+    the first sweep, in the FP64 sequence, the blocks of the sweep's end find
+    all links unit quaternions again and the next sweeps run in fixed point, as
+    a call by itself would start them -- links and plaquettes equal bit by bit
+    those of calls of one sweep each.  (One link is bad, near the lattice's end,
+    so that one block alone sees it.)"""
+    shapes = [(16, 16), (4, 4)]
+    links = [inputs.random_links(*s, 3 + k) for k, s in enumerate(shapes)]
+    links[0].reshape(-1, 4)[4 * 16 ** 4 - 7] *= 1.3
+    for members in ((0, 1), (0,)):
+        out = []
+        for calls in ((3,), (1, 1, 1)):
+            B = su2.Lattice([shapes[m][0] for m in members], [shapes[m][1] for m in members], su2.F64)
+            B.set_launch_config(cfg)
+            for l, m in enumerate(members):
+                B.set_links(links[m], l)
+            p = [B.batch_heatbath([2.3, 2.5][:len(members)], n, [5, 6][:len(members)], plaq=plaq)
+                 for n in calls]
+            out.append([B.get_links(l) for l in range(len(members))] +
+                       ([np.concatenate(p, axis=1)] if plaq else []))
+            B.close()
+        for a, b in zip(*out):
+            np.testing.assert_array_equal(a, b)
+        norm = np.sum(out[0][0] ** 2, axis=2)
+        assert np.max(np.abs(norm - 1)) <= 4e-15
+
+
 @pytest.mark.parametrize("Ns,Nt,creutz", [(6, 4, 0.0), (2, 2, 0.0), (4, 6, 1.7)])
 def test_fp64_single_phases_look_at_the_links_they_read(Ns, Nt, creutz):
     """A single phase is one kernel without a pass over the links before it: a
