@@ -199,6 +199,19 @@ __device__ __forceinline__ double plaq_double(int64_t v)  // v 2^-51
 // ---------------------------------------------------------------------------
 // lattices with non-unit links or a large coupling: the FP64 sequence
 // ---------------------------------------------------------------------------
+// the draw and the new link from the staple sum A and its plaquette part P
+template <typename LT>
+__device__ __forceinline__ int32_t general_draw(const LT& U, const LatDesc& D, uint32_t i, int mu, int p,
+                                                bool hyb, const Quat<double>& A, const Quat<double>& P,
+                                                uint32_t lex, double* plaq)
+{
+    Quat<double> un;
+    const int32_t tr = draw_link<double>(D, hyb, A, lex * 4u + (uint32_t)mu, D.sweep, &un);
+    if (tr >= 0) U.store(mu, p, i, un);
+    else un = U.load_rw(mu, p, i);
+    *plaq += qretr(un, P);
+    return tr;
+}
 // Staple sum by the tree s_k = up_k + lo_k for the k-th nu != mu,
 // A = (s_0 + s_1) + s_2 (P = its prefix over nu < mu), FP64 draw, new link.
 // Returns what update_link returns; *un is the link's final value.
@@ -219,12 +232,7 @@ __device__ __noinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, u
         if (nu == mu - 1) P = A;
     }
     *lex = s.lex();
-    Quat<double> un;
-    const int32_t tr = draw_link<double>(D, hyb, A, s.lex() * 4u + (uint32_t)mu, D.sweep, &un);
-    if (tr >= 0) U.store(mu, p, i, un);
-    else un = U.load_rw(mu, p, i);
-    *plaq += qretr(un, P);
-    return tr;
+    return general_draw(U, D, i, mu, p, hyb, A, P, s.lex(), plaq);
 }
 template <typename LT>
 __device__ __forceinline__ int32_t general_link(const Ctx& ctx, const LatDesc& D, uint32_t i, int mu,
@@ -527,12 +535,60 @@ struct Dir64 {
 static_assert(sizeof(Trial64) == 16 && sizeof(Dir64) == 32, "16-byte accesses");
 static_assert(KP_CAP % 4 == 0, "whole rounds of four trials");
 
+// general_link's sum of 32 links by their four warps: a warp forms s_k of one
+// plane (planes 1 and 2 through `sums`), the first adds them and draws.  The
+// other three give the FP64 unit of their sub-partition a third of the staple
+// each: 8^4 at beta = 1000 92 us a sweep, 126 with one link per thread in one
+// cluster launch.
+template <int MU, bool PLAQ, bool HYB>
+__device__ __noinline__ void general_quad(const Ctx& ctx, int l, uint32_t blk0, uint32_t i, int p,
+                                          double2 (*sums)[2][32], int32_t* dbg)
+{
+    const LatDesc& D = ctx.desc[l];
+    const Links<double> U(ctx.links, D, ctx.status);
+    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+    const bool act = i < D.Vh;
+    Quat<double> s0 = {0, 0, 0, 0};
+    uint32_t lex = 0;
+    if (act && role < 3) {
+        const EoSite s(D, i, p);
+        lex = s.lex();
+        uint32_t hp[4], hm[4];
+        s.hops(hp, hm);
+        const int nu = nu_of<MU>(role);
+        s0 = qadd(staple_term<double>(U, MU, nu, p, i, hp, hm, false),
+                  staple_term<double>(U, MU, nu, p, i, hp, hm, true));
+        if (role > 0) {
+            sums[role - 1][0][lane] = make_double2(s0.a0, s0.a1);
+            sums[role - 1][1][lane] = make_double2(s0.a2, s0.a3);
+        }
+    }
+    __syncthreads();
+    double plaq = 0.0;
+    uint32_t ntrial = 0, ncap = 0;
+    if (act && role == 0) {
+        auto plane = [&](int k) -> Quat<double> {
+            const double2 lo = sums[k - 1][0][lane], hi = sums[k - 1][1][lane];
+            return {lo.x, lo.y, hi.x, hi.y};
+        };
+        const Quat<double> s01 = qadd(s0, plane(1));
+        const Quat<double> A = qadd(s01, plane(2));
+        const Quat<double> P = MU == 1 ? s0 : (MU == 2 ? s01 : A);
+        const int32_t tr = general_draw(U, D, i, MU, p, HYB, A, P, lex, &plaq);
+        ncap = tr < 0;
+        ntrial = tr < 0 ? (uint32_t)KP_CAP : (uint32_t)tr;
+        if (dbg) dbg[lex] = tr;
+    }
+    __syncwarp();
+    fix_totals<MU, PLAQ>(ctx, l, blk0, D.Vh, PLAQ ? warp_sum_t(plaq) : 0.0, ntrial, ncap);
+}
+
 template <int MU, bool PLAQ, bool HYB, bool MIR, int MINB>
 __global__ void __launch_bounds__(128, MINB)
 fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
 {
     struct Group {
-        longlong2 sums[2][2][32];  // planes 1 and 2
+        longlong2 sums[2][2][32];  // planes 1 and 2 (general_quad: as double2)
         Trial64 trial[4][32];  // HYB: lambda^2 of a trial, and whether it was accepted
         Dir64 dir[32];
         struct Hyb {  // a link's inputs to its trials
@@ -559,7 +615,7 @@ fix_quad_kernel(Ctx ctx, int p, int32_t* __restrict__ dbg)
     const uint32_t i = (blockIdx.x - blk0) * 32u + (uint32_t)lane;
     const bool act = i < Vh;
     if (D.general) {
-        general_links<MU, PLAQ>(ctx, l, blk0, i, 1u, act && role == 0 ? i + 1 : i, p, HYB, dbg);
+        general_quad<MU, PLAQ, HYB>(ctx, l, blk0, i, p, reinterpret_cast<double2(*)[2][32]>(G.sums), dbg);
         return;
     }
     const FixLinks<MIR> U(ctx, D);

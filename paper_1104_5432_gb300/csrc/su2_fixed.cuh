@@ -23,7 +23,7 @@
 // to 0.49 at 64, the same from about 300 on and 12 to 15 times larger at 10^5
 // (tests/test_fixed_point.py).  So lattices at couplings above FIX_BETA_MAX
 // take the FP64 sequence (general_link), at its speed: beta = 1000, us a
-// sweep, 16^4 216, 32^4 2558, 64^4 39800 (fixed point 80, 596, 8650).
+// sweep, 8^4 92, 16^4 217, 32^4 2557, 64^4 39800 (fixed point 36, 80, 594, 8654).
 //
 // Range: |sum of four h l'| <= |h|_1 2^31, and |h|_1 <= 2 |h|_2 for four
 // components, so with unit quaternions at 2^61 (h <= 2^29) the two cross
