@@ -237,7 +237,9 @@ def shape_name(lat, idx=None):
     from paper_1104_5432_gb300.csrc_info import row_name
     from paper_1104_5432_gb300.csrc_info import shape_name as name_of
     row = row_name(lat.dtype, lat.link_layout())
-    return row, name_of(row, lat.launch_config()[0] if idx is None else idx)
+    if idx is None:
+        return row, name_of(row, lat.launch_config()[0], lat.one_launch())
+    return row, name_of(row, idx)
 
 
 def gpu_arm(args, rank, world, local):

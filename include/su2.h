@@ -293,8 +293,9 @@ int su2_set_sweep(su2_lattice* lat, int l, uint64_t sweep);
  * (su2_heatbath_phase) keeps using the last shape.  Where each CTA's share
  * is at most 512 links of a phase, all sweeps of a call without measurements
  * run in one launch; so do shape 0's on one FP32 lattice in the plain layout
- * of at most 16384 sites, with the links and plaquettes of its phase
- * launches bit by bit. */
+ * of at most 16384 sites or one FP64 lattice of at most 4096, with the links and
+ * plaquettes of its phase launches bit by bit (Kennedy-Pendleton's draw only,
+ * in both cases). */
 #define SU2_LAUNCH_CLUSTER 14
 
 /* Times every launch shape on this handle's lattices (whole sweeps with the
@@ -326,7 +327,8 @@ int su2_autotune_beta(su2_lattice* lat, const double* betas, int* chosen);
 /* Select a launch shape by index (0 .. SU2_NUM_LAUNCH_CONFIGS-1, or
  * SU2_LAUNCH_CLUSTER once memory is bound) / read the current one with its
  * threads per block and minimum blocks per SM (for the cluster sweep: the
- * threads per CTA that update links and the CTAs in the cluster). */
+ * threads per CTA that update links, in the one-launch form where that is what
+ * runs, and the CTAs in the cluster). */
 int su2_set_launch_config(su2_lattice* lat, int cfg);
 int su2_get_launch_config(const su2_lattice* lat, int* cfg, int* threads, int* min_blocks);
 

@@ -42,6 +42,11 @@ int su2_tune_cache_store(const char* path, const char* key, int cfg, double ms);
  * index that su2_get_launch_config reports; su2_set_launch_config sets all. */
 int su2_replay_config(const su2_lattice* lat, int* plain, int* measured);
 
+/* *on: whether the handle's sweeps without measurements run in one launch of
+ * one thread-block cluster per call (SU2_LAUNCH_CLUSTER), at the selected index
+ * and sampler. */
+int su2_one_launch(su2_lattice* lat, int* on);
+
 /* Walk every lattice in S y-slabs under the slab launch shapes (S must
  * divide every Ns; by default S is chosen from the lattice size so that
  * the +-t neighbour window stays within 8 MB of L2).  Synchronous. */

@@ -1501,7 +1501,8 @@ int su2_get_launch_config(const su2_lattice* lat, int* cfg, int* threads, int* m
     if (int rc = check_handle(lat, false)) return rc;
     if (lat->chosen == CFG_CLUSTER) {
         if (cfg) *cfg = CFG_CLUSTER;
-        if (threads) *threads = lat->cgeom.threads;
+        const bool chain = lat->cluster_chain && !lat->hybrid;
+        if (threads) *threads = chain ? lat->chain_geom.updaters : lat->cgeom.threads;
         if (min_blocks) *min_blocks = lat->cgeom.S;
         return SU2_OK;
     }
@@ -1587,6 +1588,14 @@ int su2_tune_cache_store(const char* path, const char* key, int cfg, double ms)
     if (!path || !key) return fail(SU2_E_INVAL, "null argument");
     if (cfg < 0 || cfg > CFG_CLUSTER) return fail(SU2_E_INVAL, "bad config");
     return cache_store(path, key, Choice(cfg), ms) ? SU2_OK : fail(SU2_E_INVAL, "cannot write %s", path);
+}
+
+int su2_one_launch(su2_lattice* lat, int* on)
+{
+    if (int rc = check_handle(lat)) return rc;
+    if (!on) return fail(SU2_E_INVAL, "null output");
+    *on = chain_of(lat) != nullptr;
+    return SU2_OK;
 }
 
 int su2_replay_config(const su2_lattice* lat, int* plain, int* measured)

@@ -29,6 +29,9 @@ ROWS = {"f32": _F32, "f64": _F64, "f32pairs": _F32P}
 CLUSTER = 14
 CLUSTER_NAME = ("one thread-block cluster (up to 16 CTAs), whole lattice in distributed "
                 "shared memory, one launch per sweep")
+# small lattices at index 0 or 14 (Lattice.one_launch)
+ONE_LAUNCH_NAME = ("one thread-block cluster (up to 16 CTAs), whole lattice in distributed "
+                   "shared memory, one launch for all sweeps of a call")
 
 
 def row_name(dtype: int, layout: int) -> str:
@@ -36,8 +39,11 @@ def row_name(dtype: int, layout: int) -> str:
     return "f64" if dtype == 1 else ("f32pairs" if layout == 1 else "f32")
 
 
-def shape_name(row, idx):
-    """Name of launch index idx of a row: a shape, or the cluster sweep."""
+def shape_name(row, idx, one_launch=False):
+    """Name of launch index idx of a row: a shape, the cluster sweep, or the
+    one-launch form of either on small lattices."""
+    if one_launch:
+        return ONE_LAUNCH_NAME
     return CLUSTER_NAME if idx == CLUSTER else launch_shapes(row)[idx]
 
 

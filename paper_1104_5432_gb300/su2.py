@@ -101,6 +101,7 @@ def load(build_if_needed: bool = True):
             "su2_tune_cache_lookup": (i, [C.c_char_p, C.c_char_p, P]),
             "su2_tune_cache_store": (i, [C.c_char_p, C.c_char_p, i, d]),
             "su2_replay_config": (i, [P, P, P]),
+            "su2_one_launch": (i, [P, P]),
             "su2_set_slabs": (i, [P, i]),
             "su2_set_sampler": (i, [P, d]),
             "su2_set_link_layout": (i, [P, i]),
@@ -377,6 +378,12 @@ class Lattice:
         c, t, m = C.c_int(), C.c_int(), C.c_int()
         _check(load().su2_get_launch_config(self._h, C.byref(c), C.byref(t), C.byref(m)))
         return c.value, t.value, m.value
+
+    def one_launch(self) -> bool:
+        """Whether sweeps without measurements run in one launch per call."""
+        v = C.c_int()
+        _check(load().su2_one_launch(self._h, C.byref(v)))
+        return bool(v.value)
 
     def sync(self):
         _check(load().su2_sync(self._h))

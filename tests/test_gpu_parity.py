@@ -642,6 +642,26 @@ def test_cluster_sweep_matches_the_shapes(Ns, Nt):
     assert lat.stats() == ref.stats() and lat.get_sweep() == 9
 
 
+def test_launch_config_reports_the_kernel_that_runs():
+    """Index 14 reports the threads that update links: 512 on 10^3 x 6 (375
+    links of a phase on each of 8 CTAs) in one launch for all sweeps, 1024 under
+    the Creutz sampler, which runs the one-sweep kernel; the names follow."""
+    from paper_1104_5432_gb300 import csrc_info
+    lat = lattice(10, 6, su2.F32)
+    assert lat.one_launch()  # shape 0
+    lat.set_launch_config(su2.LAUNCH_CLUSTER)
+    assert lat.launch_config() == (su2.LAUNCH_CLUSTER, 512, 8) and lat.one_launch()
+    lat.set_sampler(1.7)
+    assert lat.launch_config() == (su2.LAUNCH_CLUSTER, 1024, 8) and not lat.one_launch()
+    lat.set_sampler(0.0)
+    lat.set_launch_config(3)
+    assert lat.launch_config() == (3, 32, 32) and not lat.one_launch()
+    assert not lattice(16, 6, su2.F32).one_launch() and not lattice(10, 6, su2.F64).one_launch()
+    assert lattice(8, 8, su2.F64).one_launch()
+    assert "all sweeps" in csrc_info.shape_name("f32", 14, True)
+    assert "per sweep" in csrc_info.shape_name("f32", 14)
+
+
 def test_cluster_sweep_from_the_tuning_cache_and_single_phases(tmp_path, monkeypatch):
     """A cached cluster choice (launch index 14) is taken by the next 8^4
     FP32 handle at binding; the single-phase entry point of a handle in
