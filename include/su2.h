@@ -261,8 +261,8 @@ int su2_set_sweep(su2_lattice* lat, int l, uint64_t sweep);
  *   FP32:  0 256x4   1 128x8   2 64x16   3 32x32   4 256x4 slab  5 128x8 slab
  *          6 32x32 /2  7 32x32 /4  8 32x32 /8  9 32x16 /4 staged
  *          10 32x32 /2 P  11 32x32 /1 P  12 32x32 slab /8  13 32x32 slab /16
- *   FP64:  0 256x1   1 128x4   2 64x8   3 64x4   4 32x16   5 32x8
- *          6 32x16 /2  7 32x16 /4  8 32x16 /8  9 32x16 /16  10 128x4 G4
+ *   FP64:  0 256x1   1 128x5   2 64x10   3 64x4   4 32x20   5 32x8
+ *          6 32x24 /2  7 32x24 /4  8 32x24 /8  9 32x24 /16  10 128x4 G4
  *          11 128x7 G4  12 32x16 /2 P  13 32x16 /8 P
  *   FP32 site pairs (SU2_LAYOUT_PAIRS; R counts pairs): 0 256x2  1 32x16
  *          2 32x20  3 32x24  4 32x28  5 32x16 /2  6 32x20 /2  7 32x24 /2

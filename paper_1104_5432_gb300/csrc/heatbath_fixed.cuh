@@ -357,7 +357,7 @@ struct FixQueue {
 // links) stays below 2^63.
 constexpr int FIX_MAX_ROUNDS = 16;
 template <int MU, bool PLAQ, bool HYB, bool MIR, bool PERSIST>
-__global__ void __launch_bounds__(32, PERSIST ? 16 : 24)
+__global__ void __launch_bounds__(32, FIX_THREADS[PERSIST ? FIX_PERSIST : FIX_QUEUE] / 32)
 fix_queue_kernel(Ctx ctx, int p, int R, int32_t* __restrict__ dbg)
 {
     static_assert(KP_CAP <= (1 << 13), "trial index must fit 13 bits");

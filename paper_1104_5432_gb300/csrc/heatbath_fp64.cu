@@ -15,13 +15,13 @@ static void launch_fix_k(const Ctx& c, const LaunchCfg& f, int parity, int32_t* 
 {
     const dim3 grid(c.phase_blocks), block(f.threads);
     if constexpr (KIND == FIX_LINK_255)
-        fix_phase_kernel<MU, PLAQ, HYB, MIR, 256, 1><<<grid, block, 0, s>>>(c, parity, dbg);
+        fix_phase_kernel<MU, PLAQ, HYB, MIR, 256, FIX_THREADS[FIX_LINK_255] / 256><<<grid, block, 0, s>>>(c, parity, dbg);
     else if constexpr (KIND == FIX_LINK_96)
-        fix_phase_kernel<MU, PLAQ, HYB, MIR, 128, 5><<<grid, block, 0, s>>>(c, parity, dbg);
+        fix_phase_kernel<MU, PLAQ, HYB, MIR, 128, FIX_THREADS[FIX_LINK_96] / 128><<<grid, block, 0, s>>>(c, parity, dbg);
     else if constexpr (KIND == FIX_QUAD_128)
-        fix_quad_kernel<MU, PLAQ, HYB, MIR, 4><<<grid, block, 0, s>>>(c, parity, dbg);
+        fix_quad_kernel<MU, PLAQ, HYB, MIR, FIX_THREADS[FIX_QUAD_128] / 128><<<grid, block, 0, s>>>(c, parity, dbg);
     else if constexpr (KIND == FIX_QUAD_72)
-        fix_quad_kernel<MU, PLAQ, HYB, MIR, 7><<<grid, block, 0, s>>>(c, parity, dbg);
+        fix_quad_kernel<MU, PLAQ, HYB, MIR, FIX_THREADS[FIX_QUAD_72] / 128><<<grid, block, 0, s>>>(c, parity, dbg);
     else
         fix_queue_kernel<MU, PLAQ, HYB, MIR, KIND == FIX_PERSIST>
             <<<grid, block, 0, s>>>(c, parity, f.rounds, dbg);

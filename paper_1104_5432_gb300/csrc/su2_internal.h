@@ -63,10 +63,10 @@ constexpr LaunchCfg LAUNCH_CFG[NUM_ROWS][NUM_LAUNCH_CFG] = {
      {32, 32, false, 2, false}, {32, 32, false, 4, false}, {32, 32, false, 8, false},
      {32, 16, false, 4, false, 1, true}, {32, 32, false, 2, true}, {32, 32, false, 1, true},
      {32, 32, true, 8, false}, {32, 32, true, 16, false}},
-    {{256, 1, false, 1, false}, {128, 4, false, 1, false}, {64, 8, false, 1, false},
-     {64, 4, false, 1, false}, {32, 16, false, 1, false}, {32, 8, false, 1, false},
-     {32, 16, false, 2, false}, {32, 16, false, 4, false}, {32, 16, false, 8, false},
-     {32, 16, false, 16, false}, {128, 4, false, 1, false, 4}, {128, 7, false, 1, false, 4},
+    {{256, 1, false, 1, false}, {128, 5, false, 1, false}, {64, 10, false, 1, false},
+     {64, 4, false, 1, false}, {32, 20, false, 1, false}, {32, 8, false, 1, false},
+     {32, 24, false, 2, false}, {32, 24, false, 4, false}, {32, 24, false, 8, false},
+     {32, 24, false, 16, false}, {128, 4, false, 1, false, 4}, {128, 7, false, 1, false, 4},
      {32, 16, false, 2, true}, {32, 16, false, 8, true}},
     // FP32 site pairs: one thread updates two links (t and t + Nt/2) per
     // round with packed two-lane arithmetic; `rounds` counts pairs
@@ -98,6 +98,16 @@ constexpr FixKind fix_kind(const LaunchCfg& f)
            : f.threads * f.min_blocks <= 256 ? FIX_LINK_255
                                              : FIX_LINK_96;
 }
+// threads an SM holds at least of each kernel, as it is compiled (a block of
+// fewer threads runs in as many more blocks)
+constexpr int FIX_THREADS[NUM_FIX_KINDS] = {256, 640, 512, 896, 768, 512};
+constexpr bool fix_table_holds()
+{
+    for (const LaunchCfg& f : LAUNCH_CFG[ROW_F64])
+        if (f.threads * f.min_blocks != FIX_THREADS[fix_kind(f)]) return false;
+    return true;
+}
+static_assert(fix_table_holds(), "the FP64 row states what is compiled");
 // largest y-slab window (sites between a site and its t neighbour, times
 // the bytes a site's update touches) kept in L2
 constexpr double SLAB_WINDOW_BYTES = 8.0 * (1 << 20);

@@ -11,10 +11,10 @@ _F32 = [(256, 4, False, 1, False), (128, 8, False, 1, False), (64, 16, False, 1,
         (32, 32, False, 2, False), (32, 32, False, 4, False), (32, 32, False, 8, False),
         (32, 16, False, 4, False, 1, True), (32, 32, False, 2, True), (32, 32, False, 1, True),
         (32, 32, True, 8, False), (32, 32, True, 16, False)]
-_F64 = [(256, 1, False, 1, False), (128, 4, False, 1, False), (64, 8, False, 1, False),
-        (64, 4, False, 1, False), (32, 16, False, 1, False), (32, 8, False, 1, False),
-        (32, 16, False, 2, False), (32, 16, False, 4, False), (32, 16, False, 8, False),
-        (32, 16, False, 16, False), (128, 4, False, 1, False, 4), (128, 7, False, 1, False, 4),
+_F64 = [(256, 1, False, 1, False), (128, 5, False, 1, False), (64, 10, False, 1, False),
+        (64, 4, False, 1, False), (32, 20, False, 1, False), (32, 8, False, 1, False),
+        (32, 24, False, 2, False), (32, 24, False, 4, False), (32, 24, False, 8, False),
+        (32, 24, False, 16, False), (128, 4, False, 1, False, 4), (128, 7, False, 1, False, 4),
         (32, 16, False, 2, True), (32, 16, False, 8, True)]
 
 
