@@ -112,6 +112,14 @@ int su2_probe_special_rate(int fn, int iters, double* calls_per_s, void* stream)
  * the table (synchronous); the kernel is asynchronous on `stream`. */
 int su2_selftest_ln(void* out, void* stream);
 
+/* The fixed-point FP64 update's functions on the device against their host
+ * build, on nsample arguments of each: out (host, 6 values) gets the largest
+ * difference of the reciprocal square root (units of 2^-60), the square root
+ * (2^-62), -ln u, the cosine and the sine of a grid angle, and a double taken
+ * in and out again (differences of their integers).  scratch: 16-byte aligned
+ * device memory of at least 64 KiB.  Synchronous; allocates no device memory. */
+int su2_selftest_fixed(uint32_t nsample, uint64_t* out, void* scratch, size_t scratch_bytes, void* stream);
+
 /* The FP64 heat bath's table-driven sine and cosine of pi y against CUDA's
  * sincospi: out (device, 2 doubles) gets the cosine's largest absolute
  * difference over the trials' 2^23 arguments y = (2k + 1) 2^-23 and the

@@ -3,7 +3,13 @@
 // uniform grid u = (k + 1/2) 2^-23, k = 0 .. 2^23 - 1; and the FMA-rate
 // and FP64 math-function probes that give the arithmetic rooflines their
 // measured denominators (declared in su2_testing.h).
+#include <algorithm>
+#include <cstdlib>
+#include <new>
+#include <vector>
+
 #include "su2_testing.h"
+#include "su2_fixed.cuh"
 #include "su2_internal.h"
 #include "su2_math.cuh"
 
@@ -106,6 +112,47 @@ __global__ void ln_selftest_kernel(unsigned long long* out)
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
         if ((threadIdx.x & 31) == 0) atomic_max_pos(out + j, m);
     }
+}
+
+// The fixed-point update's functions on the device against their host build
+// (whose errors the host test measures): sample k of each.  Only rsqrt_fix is
+// not integers throughout: its seed is the hardware's reciprocal square root.
+struct FixSample {
+    int64_t rsqrt, sqrt, ln, cos, sin, link;
+};
+__host__ __device__ inline uint64_t mix64(uint64_t x)
+{
+    x += 0x9E3779B97F4A7C15ull;
+    x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
+    x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
+    return x ^ (x >> 31);
+}
+__host__ __device__ inline FixSample fix_sample(uint32_t k, const FixTables* tab)
+{
+    const uint64_t a = mix64(2ull * k), b = mix64(2ull * k + 1);
+    FixSample r;
+    // K in [2^56, 2^60], its ends and the powers of two first
+    const uint64_t K = k < 10 ? (uint64_t(1) << (56 + k / 2)) - (k & 1) + (k == 1)
+                              : (uint64_t(1) << 56) + a % (uint64_t(15) << 56);
+    r.rsqrt = rsqrt_fix(K);
+    // v 2^e <= 1 down to 2^-24
+    r.sqrt = sqrt_fix((uint64_t(1) << 58) + b % (uint64_t(31) << 58), -63 - (int)(a % 22));
+    const uint32_t u = k < 4096 ? (1u << 24) - 1u - 2u * k : 2u * (uint32_t)(a >> 41) + 1u;
+    const NegLn l = neg_ln(u, tab);
+    r.ln = neg_ln_at(l, l.n == 0 ? 0 : 4);
+    const Arc arc = arc_at((uint32_t)(b >> 40), tab);
+    r.cos = arc_cos(arc);
+    r.sin = arc_sin(arc);
+    // a link component in and a value out
+    const uint32_t e = 1022u - (uint32_t)(a & 63u);
+    const Fx f = fx_link((uint32_t)(b >> 63 << 31) | (e << 20) | (uint32_t)(b >> 44 & 0xFFFFFu), (uint32_t)b);
+    r.link = (int64_t)double_bits((int64_t)((uint64_t)(int64_t)f.h << 32) + f.l, -61);
+    return r;
+}
+__global__ void fixed_selftest_kernel(FixSample* out, uint32_t k0, uint32_t n, const FixTables* tab)
+{
+    const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) out[j] = fix_sample(k0 + j, tab);
 }
 
 // 8 independent FMA chains per thread: the pipe never waits on a result
@@ -260,6 +307,47 @@ extern "C" int su2_selftest_ln(void* out, void* stream)
     su2::ln_selftest_kernel<<<(1u << 23) / 256, 256, 0, s>>>(
         static_cast<unsigned long long*>(out));
     return cudaGetLastError() == cudaSuccess ? SU2_OK : SU2_E_CUDA;
+}
+
+extern "C" int su2_selftest_fixed(uint32_t nsample, uint64_t* out, void* scratch, size_t scratch_bytes,
+                                  void* stream)
+{
+    using namespace su2;
+    constexpr size_t TAB = (sizeof(FixTables) + 255) / 256 * 256;
+    if (!out || !scratch || ((uintptr_t)scratch & 15) || scratch_bytes < TAB + 256 * sizeof(FixSample))
+        return SU2_E_INVAL;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    FixTables* const dtab = static_cast<FixTables*>(scratch);
+    FixSample* const dev = reinterpret_cast<FixSample*>(static_cast<char*>(scratch) + TAB);
+    const uint32_t per = (uint32_t)std::min<size_t>((scratch_bytes - TAB) / sizeof(FixSample), 1u << 18);
+    std::fill(out, out + 6, uint64_t(0));
+    try {
+        std::vector<FixTables> tab(1);
+        std::vector<FixSample> got(per);
+        fill_fix_tables(tab.data());
+        if (cudaMemcpyAsync(dtab, tab.data(), sizeof(FixTables), cudaMemcpyHostToDevice, s) != cudaSuccess)
+            return SU2_E_CUDA;
+        for (uint32_t k0 = 0; k0 < nsample; k0 += per) {
+            const uint32_t n = std::min(per, nsample - k0);
+            fixed_selftest_kernel<<<(n + 255) / 256, 256, 0, s>>>(dev, k0, n, dtab);
+            if (cudaGetLastError() != cudaSuccess ||
+                cudaMemcpyAsync(got.data(), dev, n * sizeof(FixSample), cudaMemcpyDeviceToHost, s) !=
+                    cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess)
+                return SU2_E_CUDA;
+            for (uint32_t j = 0; j < n; ++j) {
+                const FixSample h = fix_sample(k0 + j, tab.data());
+                const int64_t d[6] = {h.rsqrt - got[j].rsqrt, h.sqrt - got[j].sqrt, h.ln - got[j].ln,
+                                      h.cos - got[j].cos,     h.sin - got[j].sin,   h.link - got[j].link};
+                for (int c = 0; c < 6; ++c)
+                    out[c] = std::max(out[c], (uint64_t)(d[c] < 0 ? -d[c] : d[c]));
+            }
+            if (n < per) break;  // (k0 + per may pass 2^32)
+        }
+    } catch (const std::bad_alloc&) {
+        return SU2_E_NOMEM;
+    }
+    return SU2_OK;
 }
 
 extern "C" int su2_selftest_trig(void* out, void* stream)

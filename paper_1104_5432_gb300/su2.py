@@ -89,6 +89,7 @@ def load(build_if_needed: bool = True):
             "su2_selftest_math": (i, [P, P]),
             "su2_selftest_ln": (i, [P, P]),
             "su2_selftest_trig": (i, [P, P]),
+            "su2_selftest_fixed": (i, [C.c_uint32, P, P, sz, P]),
             "su2_get_links_f32": (i, [P, i, P]),
             "su2_set_links_f32": (i, [P, i, P]),
             "su2_probe_fma_rate": (i, [i, i, P, P]),

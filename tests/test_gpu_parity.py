@@ -574,6 +574,28 @@ def test_table_logarithm_on_every_uniform():
     assert err_abs <= 4e-15, (err_abs, err_ulp)
 
 
+def test_fixed_point_functions_on_the_device_against_the_host_build():
+    """The functions of the fixed-point FP64 update as the device runs them,
+    against the host build whose errors against extended precision
+    test_fixed_point.py measures: integers throughout, so the same ones, but
+    for the reciprocal square root (and the square root from it), which starts
+    from the hardware's seed.  There each side is within 2^-59 (relative; the
+    value below 4) and 2^-57 of the true one, so they lie within 2 * 4 * 2 units
+    of 2^-60 and 2 * 32 of 2^-62 of one another.  (The gates of 1e-12 on whole
+    links would pass ten bits lost here.)"""
+    scratch = torch.zeros(1 << 22, dtype=torch.uint8, device="cuda")
+    out = np.zeros(6, np.uint64)
+    rc = su2.load().su2_selftest_fixed(1 << 20, out.ctypes.data, scratch.data_ptr(), scratch.numel(),
+                                       torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    rsqrt, sqrt, ln, cos, sin, link = [int(v) for v in out]
+    assert rsqrt <= 16 and sqrt <= 64, out
+    assert (ln, cos, sin, link) == (0, 0, 0, 0), out
+    # too little scratch, null buffers
+    assert su2.load().su2_selftest_fixed(16, out.ctypes.data, scratch.data_ptr(), 1024, None) == su2.SU2_E_INVAL
+    assert su2.load().su2_selftest_fixed(16, None, scratch.data_ptr(), scratch.numel(), None) == su2.SU2_E_INVAL
+
+
 @pytest.mark.parametrize("dtype", [su2.F32, su2.F64])
 def test_every_launch_shape_gives_identical_results(dtype):
     """The random streams are keyed by link and sweep, never by thread: each
