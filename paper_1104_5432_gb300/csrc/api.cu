@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -540,23 +541,23 @@ int sync_status(su2_lattice* L)
 }
 
 // As sync_status, and the work buffer's bytes between the status word and
-// `bytes` past src come with it in the same copy (each copy to pageable memory
-// and its wait take ~10 us): *host points at src's values.
-int fetch_status(su2_lattice* L, const double* src, size_t bytes, const double** host)
+// src + count come with it in the same copy (each copy to pageable memory and
+// its wait take ~10 us): the `count` values at src go to out, and n2 more that
+// follow to out2.
+int fetch_status(su2_lattice* L, const double* src, size_t count, double* out, size_t n2 = 0,
+                 double* out2 = nullptr)
 {
-    static thread_local std::vector<char> buf;
     const size_t at = (size_t)(reinterpret_cast<const char*>(src) - (L->work + L->off_status));
-    try {
-        buf.resize(at + bytes);
-    } catch (const std::bad_alloc&) {
-        return fail(SU2_E_NOMEM, "no host memory for the results");
-    }
-    SU2_CUDA(cudaMemcpyAsync(buf.data(), L->work + L->off_status, at + bytes, cudaMemcpyDeviceToHost,
+    const size_t bytes = at + sizeof(double) * (count + n2);
+    const std::unique_ptr<char[]> buf(new (std::nothrow) char[bytes]);
+    if (!buf) return fail(SU2_E_NOMEM, "no host memory for the results");
+    SU2_CUDA(cudaMemcpyAsync(buf.get(), L->work + L->off_status, bytes, cudaMemcpyDeviceToHost,
                              L->stream));
     SU2_CUDA(cudaStreamSynchronize(L->stream));
     uint32_t st = 0;
-    memcpy(&st, buf.data(), sizeof st);
-    *host = reinterpret_cast<const double*>(buf.data() + at);
+    memcpy(&st, buf.get(), sizeof st);
+    memcpy(out, buf.get() + at, sizeof(double) * count);
+    if (out2) memcpy(out2, buf.get() + at + sizeof(double) * count, sizeof(double) * n2);
     return report_status(L, st);
 }
 
@@ -681,12 +682,8 @@ int heatbath_impl(su2_lattice* L, const double* betas, double beta, int nsweeps,
                 SU2_CUDA(cudaGraphLaunch(g_first && done + s == 0 ? g_first : g, L->stream));
         }
         if (want && !dev_out) {
-            if (L->n == 1 && rmax < 0 && done + chunk == nsweeps) {
-                const double* host = nullptr;
-                const int rc = fetch_status(L, L->ring_dev(), sizeof(double) * chunk, &host);
-                if (host) memcpy(plaq + done, host, sizeof(double) * chunk);
-                return rc;
-            }
+            if (L->n == 1 && rmax < 0 && done + chunk == nsweeps)
+                return fetch_status(L, L->ring_dev(), (size_t)chunk, plaq + done);
             // one pitched copy when its rows fill the caller's buffer; a pitched
             // copy of part of the sweeps would span a whole pitch past its last
             // row, beyond the buffer's end
@@ -732,15 +729,6 @@ int init_impl(su2_lattice* L, int start, const uint64_t* seeds, uint64_t seed)
         SU2_CUDA(launch_init(L->ctx, L->dtype, l, (uint32_t)L->V[l], start,
                              seeds ? seeds[l] : seed + (uint64_t)l, L->stream));
     return SU2_OK;
-}
-
-// out: host or device; produce n*rows doubles through the result area
-int finish_output(su2_lattice* L, double* out, const double* dev_src, size_t count)
-{
-    const double* host = nullptr;
-    const int rc = fetch_status(L, dev_src, sizeof(double) * count, &host);
-    if (host) memcpy(out, host, sizeof(double) * count);
-    return rc;
 }
 
 }  // namespace
@@ -1236,7 +1224,7 @@ int su2_plaquette(su2_lattice* lat, double* out)
     const bool dev = is_device_ptr(out);
     double* tgt = dev ? out : lat->res_dev();
     SU2_CUDA(launch_plaquette(lat->ctx, lat->row, tgt, lat->stream));
-    if (!dev) return finish_output(lat, out, tgt, lat->n);
+    if (!dev) return fetch_status(lat, tgt, lat->n, out);
     return SU2_OK;
 }
 
@@ -1251,15 +1239,7 @@ int su2_polyakov_loop(su2_lattice* lat, double* out_signed, double* out_abs)
     double* ts = dev ? out_signed : lat->res_dev();
     double* ta = out_abs ? (dev ? out_abs : lat->res_dev() + lat->n) : nullptr;
     SU2_CUDA(launch_polyakov(lat->ctx, lat->row, ts, ta, 0, lat->stream));
-    if (!dev) {
-        const double* host = nullptr;
-        const int rc = fetch_status(lat, ts, sizeof(double) * 2 * lat->n, &host);
-        if (host) {
-            memcpy(out_signed, host, sizeof(double) * lat->n);
-            if (out_abs) memcpy(out_abs, host + lat->n, sizeof(double) * lat->n);
-        }
-        return rc;
-    }
+    if (!dev) return fetch_status(lat, ts, lat->n, out_signed, out_abs ? lat->n : 0, out_abs);
     return SU2_OK;
 }
 
@@ -1279,7 +1259,7 @@ int su2_polyakov_correlator(su2_lattice* lat, int rmax, double* out, int accumul
         SU2_CUDA(cudaMemcpyAsync(tgt, out, sizeof(double) * cnt, cudaMemcpyHostToDevice,
                                  lat->stream));
     SU2_CUDA(launch_correlator(lat->ctx, lat->dtype, rmax, tgt, accumulate, lat->stream));
-    if (!dev) return finish_output(lat, out, tgt, cnt);
+    if (!dev) return fetch_status(lat, tgt, cnt, out);
     return SU2_OK;
 }
 
