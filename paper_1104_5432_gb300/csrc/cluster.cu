@@ -194,10 +194,11 @@ hb_cluster_kernel(Ctx ctx, uint32_t C, FastDiv div_c, int pl)
 // plaquettes are reproduced bit by bit too.
 // Measured per sweep with the plaquette (beta = 2.4): 8^4 12.2 us (28.7 in
 // launch shape 0's phase launches, 22.6 in the whole-sweep kernel above),
-// 10^3 x 6 13.8 (28.7), 12^3 x 8 23.1 (28.8); 4^4 9.5, i.e. 1.2 us a phase
-// whatever the size: one update's remaining chain and the barrier.  (With only
-// the first trial drawn ahead 8^4 took 13.0: some link rejects it in every
-// phase, and all wait.)
+// 10^3 x 6 13.8 (28.7), 12^3 x 8 23.1 (28.8), 4^4 9.5.  A phase takes 1.2 us at
+// 4^4, one update's remaining chain and the barrier, and grows with the links
+// a CTA updates: 1.5 us at 128 (8^4), 1.7 at 192, 2.9 at 448.  (With only the
+// first trial drawn ahead 8^4 took 13.0: some link rejects it in every phase,
+// and all wait.)
 struct ChainShared {
     float4* own;       // [8][C] links
     float4* tdir;      // [2][C] (t, r4^2, cos theta, sin theta) of the coming phase

@@ -8,10 +8,12 @@
 // (general_link: ~270 FP64 instructions, 20,600 clocks per warp) was
 // bound by the FP64 unit alone: 1.66 G link updates/s at 64^4, beta = 2.5,
 // whatever the shape.  The integer update issues ~2,730 instructions per
-// 32 links (1,410 on the half-rate multiply pipe, 82% busy, 1,090 on the ALU
-// pipe) and runs at 7.16 G/s there (R = 8 or 16, 24 blocks a SM; 6.76 with 16)
-// and 6.3 G/s at 32^4, beta = 6.0 (one link per thread, from 1.57); without
-// the fixed-point copy of the links 5.76 and 5.22.  All forms call the same
+// 32 links, 1,360 to 1,490 of them on the multiply pipe, which is busy 2.8 to
+// 3.2 clocks for each (32^4, by its counters: a product takes 2, one with a
+// 64-bit addend more), i.e. ~4,500 clocks of it, and ~1,090 on the ALU pipe.
+// With that pipe 79 to 82% busy it runs at 7.16 G/s at 64^4 (R = 8 or 16, 24
+// blocks a SM; 6.76 with 16) and 6.3 G/s at 32^4, beta = 6.0 (one link per
+// thread, from 1.57); without the fixed-point copy of the links 5.76 and 5.22.  All forms call the same
 // functions on integers, so links and trial counts are bit-identical between
 // them.
 //
