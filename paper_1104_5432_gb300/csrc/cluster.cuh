@@ -22,6 +22,7 @@ __device__ __forceinline__ void cluster_sync()
 // host thread of another lattice never lowers the limit under a launch.
 inline cudaError_t allow_cluster(const void* k, size_t max_smem)
 {
+    if (max_smem == 0) return cudaErrorInvalidDevice;  // (cluster_room: the device did not answer)
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e != cudaSuccess
                ? e

@@ -44,12 +44,12 @@ __global__ void __launch_bounds__(TPB) unit_check_kernel(Ctx ctx, bool mirror)
 // once every link has been updated the lattice takes the fixed-point path.  The
 // last block to finish (the counter D->recheck) clears the lattice's flag, so
 // every block has read it by then.  (By one block a sweep of 64^4 with one bad
-// link took 254 ms in all instead of 56.)
-constexpr unsigned RECHECK_BLOCKS = 304;  // over all lattices, two an SM
-__device__ void unit_recheck(const Ctx& ctx, LatDesc* D, uint32_t nb)
+// link took 254 ms in all, by 32 62, by 304 56.)
+constexpr unsigned RECHECK_BLOCKS = 32;  // over all lattices (200 idle ones took 0.9 us a sweep)
+__device__ void unit_recheck(const Ctx& ctx, LatDesc* D, uint32_t block, uint32_t nb)
 {
     bool ok = true;
-    for (uint32_t eo = blockIdx.x * TPB + threadIdx.x; eo < D->Vh; eo += nb * TPB)
+    for (uint32_t eo = block * TPB + threadIdx.x; eo < D->Vh; eo += nb * TPB)
         if (!unit_links_at(ctx, *D, eo, ctx.mirror != nullptr)) ok = false;
     ok = __syncthreads_and(ok);
     if (threadIdx.x == 0) {
@@ -65,8 +65,8 @@ __device__ void unit_recheck(const Ctx& ctx, LatDesc* D, uint32_t nb)
 // the lattice's sweep counter.  Grid (chunks, lattices); each block sums
 // SWEEP_CHUNK partials of its lattice, the last block of a lattice to finish
 // (ticket counter) adds the chunk sums in chunk order.
-// FP64 lattices with non-unit links are looked at again (F64), by the first
-// nrecheck blocks of each (the grid has at least as many).
+// F64: nrecheck further blocks per lattice look again at the links of one that
+// has non-unit ones (without the plaquette the first nrecheck blocks do).
 template <bool PLAQ, bool F64>
 __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx, uint32_t nrecheck)
 {
@@ -74,12 +74,12 @@ __global__ void __launch_bounds__(TPB) sweep_end_kernel(Ctx ctx, uint32_t nreche
     __shared__ int s_last;
     const int l = blockIdx.y;
     LatDesc* D = ctx.desc + l;
-    if (!PLAQ) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) D->sweep += 1;
-        if (F64 && D->general == GENERAL_LINKS) unit_recheck(ctx, D, nrecheck);
+    if (!PLAQ && blockIdx.x == 0 && threadIdx.x == 0) D->sweep += 1;
+    if (!PLAQ || (F64 && blockIdx.x >= ctx.max_chunks)) {
+        if (F64 && D->general == GENERAL_LINKS)
+            unit_recheck(ctx, D, PLAQ ? blockIdx.x - ctx.max_chunks : blockIdx.x, nrecheck);
         return;
     }
-    if (F64 && blockIdx.x < nrecheck && D->general == GENERAL_LINKS) unit_recheck(ctx, D, nrecheck);
     // partials are per warp: lattice l owns warps [b0, b0 + nb) of each slot
     const uint32_t b0 = ctx.phase_start[l] * ctx.phase_wpb;
     const uint32_t nb = ctx.phase_start[l + 1] * ctx.phase_wpb - b0;
@@ -188,8 +188,8 @@ cudaError_t launch_sweep_end(const Ctx& c, bool fp64, bool plaq, cudaStream_t s)
 {
     // a block for each TPB of an average lattice's Vh (site_blocks count V)
     const unsigned n = (unsigned)c.n, most = std::max(1u, RECHECK_BLOCKS / n);
-    const unsigned nrecheck = fp64 ? std::min(most, std::max(1u, c.site_blocks / (2 * n))) : 1u;
-    const dim3 grid(std::max(plaq ? c.max_chunks : 1u, nrecheck), n);
+    const unsigned nrecheck = fp64 ? std::min(most, std::max(1u, c.site_blocks / (2 * n))) : 0u;
+    const dim3 grid(plaq ? c.max_chunks + nrecheck : std::max(1u, nrecheck), n);
     const unsigned nt = plaq || fp64 ? TPB : 32;
     if (fp64 && plaq) sweep_end_kernel<true, true><<<grid, nt, 0, s>>>(c, nrecheck);
     else if (fp64) sweep_end_kernel<false, true><<<grid, nt, 0, s>>>(c, nrecheck);
